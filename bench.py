@@ -691,7 +691,7 @@ def main():
                  "positions per thread)" if N % 4 == 0 else
                  "k_gs_lat (Gauss-Seidel colour sweep, finest level, FP32, tabulated lattice stencil)")
                 if infos[-1].lattice_stencil else "k_gs (Gauss-Seidel colour sweep, finest level, FP32)"),
-        "gs": "k_sgs_flags / k_sgs_coop / k_sgs_cluster (symmetric Gauss-Seidel step, coarse levels, FP32)",
+        "gs": "k_sweep (symmetric Gauss-Seidel step, coarse levels, FP32)",
         "jz": ("k_jz_latdf (double-FP32 Jacobian apply fused with the Lanczos dot; SM-pipe bound)"
                if infos[-1].df_jacobian else "k_jz (Jacobian apply fused with the Lanczos dot, FP64)"),
         "coarse": "k_dense_mv_df (double-FP32 dense coarsest product)",
@@ -713,20 +713,20 @@ def main():
             "launches_timed": pr["timed"], "avg_launch_us": 1e3 * pr["ms"] / pr["timed"],
             "ms_per_solve": pr["ms"] / nsolves, "peak_kind": f"{peak_kind} hbm_gbs (copy)",
         }
-    # the coarse sweep is a chain of dependent phases: each waits for a hand-off
-    # from the CTAs it reads (release store -> acquiring poll), gathers the
-    # neighbours' x from L2, and publishes its own writes behind a GPU-scope fence;
-    # its floor per phase is the sum of those three measured latencies
+    # the coarse sweep is a chain of dependent phases: each row polls its
+    # neighbours' values (a store seen by a poll on another SM) after a first
+    # request of them from L2; its floor per phase is the sum of those two
+    # measured latencies
     sweep_levels = [lv for lv in levels[1:-1]]
     if "gs" in rooflines and sweep_levels:
         phases = sum(2 * lv["ncolors"] - 1 for lv in sweep_levels)  # per pre- or post-smoothing
         us_phase = rooflines["gs"]["avg_launch_us"] * len(sweep_levels) / phases
-        floor_us = (sync_lat["handoff_ns"] + sync_lat["l2_load_ns"] + sync_lat["fence_ns"]) / 1e3
+        floor_us = (sync_lat["handoff_ns"] + sync_lat["l2_load_ns"]) / 1e3
         rooflines["gs"]["latency"] = {
             "bound": "latency", "phases_per_launch": phases / len(sweep_levels), "us_per_phase": us_phase,
             "floor_us_per_phase": floor_us, "frac": floor_us / us_phase, **sync_lat,
-            "how": "floor = median one-way CTA hand-off + dependent L2 load + store and GPU-scope fence, "
-                   "measured by gl_measure_sync_latency"}
+            "how": "floor = median one-way CTA hand-off + dependent L2 load, measured by "
+                   "gl_measure_sync_latency"}
     # the double-FP32 Jacobian is bounded by the FP32 pipe: its min(HBM, ALU) roofline
     if "jz" in rooflines and profs["jz"][0]["flops"] > 0 and infos[-1].df_jacobian:
         rooflines["jz"]["alu"] = alu_roofline(profs["jz"][0], 2, peak, fp32_gflops,
@@ -734,7 +734,7 @@ def main():
     # the FP64 form's classes against min(HBM, FP64 ALU)
     rooflines_fp64 = {}
     KERNELS64 = {"gs0": "k_gs (Gauss-Seidel colour sweep, finest level, FP64)",
-                 "gs": "k_sgs_flags / k_sgs_coop (symmetric Gauss-Seidel step, coarse levels, FP64)",
+                 "gs": "k_sweep (symmetric Gauss-Seidel step, coarse levels, FP64)",
                  "jz": "k_jz (Jacobian apply fused with the Lanczos dot, FP64)"}
     for cls in ("gs0", "gs", "jz"):
         _, _, pr = timed(opts_fp64, 2, 1, profile_class=cls)

@@ -101,10 +101,8 @@ typedef struct {
                             reads a quarter of the bytes but is bound by this GPU's FP64 rate, and took
                             longer than the stored form when measured); 0: always the stored stencil
                             (default 1) */
-    int cluster_sweeps;  /* 1: FP32 coarse-level Gauss-Seidel steps whose level vector fits the shared memory
-                            of one thread-block cluster may run in that cluster (hardware barrier between
-                            colours) instead of a cooperative grid: with autotune, where the setup timing
-                            finds it faster; without, wherever it fits; 0: always the grid (default 1) */
+    int cluster_sweeps;  /* accepted for compatibility and without effect: the coarse-level sweeps no longer
+                            have a thread-block-cluster form (default 1) */
     gl_warmstart warmstart; /* learned initial guess: when set, gl_jacobian_solve and gl_newton_step ignore the
                             x passed in, start from the network's x0 (with warmstart_hint, below), and fall
                             back to x0 = 0 when ||b - J x0||_D >= ||b||_D (default NULL: start from x as
@@ -118,12 +116,10 @@ typedef struct {
                             device).  Each colour is one dependent phase of a sweep.  The finest lattice
                             level is always red-black. */
     int sweep_sync;      /* synchronisation between the colours of a coarse-level Gauss-Seidel step:
-                            0 = chosen per level (timed at setup with autotune; else the neighbour flags
-                            where their partition fits), 1 = a grid-wide barrier, 2 = neighbour flags
-                            (each CTA waits only for the CTAs whose rows its rows read; the grid barrier
-                            where no partition fits).  The result is the same; only the time differs.
-                            Every wait is bounded (1 s); one that runs out ends the call with
-                            GL_ERR_TIMEOUT (default 0) */
+                            0 and 2 = dataflow (every row polls the neighbour values it needs; no barrier
+                            and no flag between colours), 1 = a grid-wide barrier.  The result is the same;
+                            only the time differs.  Every wait is bounded (1 s); one that runs out ends the
+                            call with GL_ERR_TIMEOUT (default 0) */
     int coarse_df;       /* the dense coarsest product of the FP32 V-cycle (GL_MIXED, GL_MIXED_PRECOND):
                             1 = double-FP32 arithmetic (the FP64 inverse as FP32 hi + lo pairs, error-free
                             products and compensated sums, about 48 significant bits: the FP64 product's
@@ -361,10 +357,9 @@ GL_API gl_status gl_precond_level_info(gl_prec prec, int level, int64_t *n, int6
                                 int64_t *p_nnz, double *omega);
 /* How level l's Gauss-Seidel steps run in the given precision's V-cycle
  * (GL_FP64, or GL_MIXED / GL_MIXED_PRECOND for the FP32 V-cycle once built):
- * *lanes = lanes per row, *sync = 0 for a cooperative grid with a grid
- * barrier between colours, 1 for neighbour flags (*ctas = CTAs of the launch),
- * 3 for one thread-block cluster (*ctas = its size); 0 / -1 / 0 on the lattice
- * and the coarsest level, which have no such sweep.  Any output may be NULL. */
+ * *lanes = lanes per row, *sync = 0 for a grid barrier between colours, 1 for
+ * dataflow, *ctas = CTAs of the launch; 0 / -1 / 0 on the lattice and the
+ * coarsest level, which have no such sweep.  Any output may be NULL. */
 GL_API gl_status gl_precond_level_sweep(gl_prec prec, int level, int precision, int *lanes, int *sync, int *ctas);
 
 /* agg_host: n int32, the coarse node of each node of this level (not the coarsest). */

@@ -405,7 +405,7 @@ def gl_precond_debug(prec, action: int):
 
 def gl_precond_level_sweep(prec, level: int, precision=GL_FP64) -> dict:
     """How a level's Gauss-Seidel steps run: lanes per row, sync (0 grid barrier,
-    1 neighbour flags, 3 cluster, -1 none) and CTAs."""
+    1 dataflow, -1 none) and CTAs."""
     a, b, c = C.c_int(), C.c_int(), C.c_int()
     _check(library().gl_precond_level_sweep(prec, level, precision, C.byref(a), C.byref(b), C.byref(c)))
     return dict(lanes=a.value, sync=b.value, ctas=c.value)

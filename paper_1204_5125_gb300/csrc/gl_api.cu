@@ -392,16 +392,11 @@ gl_status gl_precond_level_sweep(gl_prec p, int l, int precision, int *lanes, in
         const Level &L = p->L[l];
         const bool f32 = precision != GL_FP64;
         const bool coarse = l > 0 && l < p->nlev - 1;
-        if (lanes) *lanes = coarse ? (f32 ? L.sgs_G32 : L.sgs_G64) : 0;
+        if (lanes) *lanes = coarse ? (f32 ? L.sw32.G : L.sw64.G) : 0;
         int sy = -1, nb = 0;
         if (coarse) {
-            if (f32 && L.cl_size > 0 && p->cluster_sweeps) {
-                sy = 3;
-                nb = L.cl_size;
-            } else {
-                sy = f32 ? L.sync32 : L.sync64;
-                nb = sy == 1 ? (f32 ? L.fl32.nb : L.fl64.nb) : 0;
-            }
+            sy = f32 ? L.sw32.sync : L.sw64.sync;
+            nb = f32 ? L.sw32.nb : L.sw64.nb;
         }
         if (sync) *sync = sy;
         if (ctas) *ctas = nb;

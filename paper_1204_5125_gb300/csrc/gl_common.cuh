@@ -75,6 +75,10 @@ struct DBuf {
         if (count) GL_CUDA(cudaMalloc(&p, count * sizeof(T)));
         n = count;
     }
+    // room for at least `count` elements; the contents are not kept
+    void reserve(size_t count) {
+        if (n < count) alloc(count);
+    }
     void release() {
         if (p) cudaFree(p);
         p = nullptr;

@@ -52,51 +52,52 @@ struct gl_mesh_s {
 namespace gl {
 
 constexpr int MAX_LEVELS = 16;
-// grid-barrier state of a level's cooperative sweeps: one 64-bit arrival
-// counter for the FP32 and one for the FP64 sweep
-constexpr int GRID_BARRIER_WORDS = 4;
 constexpr int MAX_COARSE_DENSE = 4096;
-// neighbour-flag form of the coarse sweeps: one completed-phase counter per
-// CTA, FLAG_STRIDE 64-bit words apart, at most MAX_FLAG_CTAS CTAs per launch,
-// and at most FLAG_MAXN neighbour CTAs per (CTA, colour)
-constexpr int FLAG_STRIDE = 16;
-constexpr int MAX_FLAG_CTAS = 1024;
-constexpr int FLAG_MAXN = 32;
 // status word value a bounded device-side wait writes when it runs out
 constexpr int STATUS_TIMEOUT = 6;
 // bound of every device-side wait of the coarse sweeps (globaltimer ns)
 constexpr long long SWEEP_WAIT_NS = 1000000000ll;
 
-// Partition and dependency lists of the neighbour-flag sweep of one level in one
-// precision: CTA b owns chunk b of nb equal contiguous chunks of every colour's
-// positions (ascending node ids within a colour, so chunk b of every colour lies
-// in about the same part of the level); before a phase it waits only for the
-// CTAs owning columns of its rows in that phase's colour.
-struct FlagPlan {
-    int nb = 0;                  // CTAs of the launch (0: no plan)
-    int G = 0;                   // lanes per row the plan was built for
-    DBuf<int64_t> rstart;        // [colour][nb + 1]: first solve position of each CTA's rows in the colour
-    DBuf<int32_t> nbr;           // [cta][colour][FLAG_MAXN]: CTAs whose rows those rows read
-    DBuf<int32_t> nbrc;          // [cta][colour]: lengths of those lists
-    // the row pointers of each CTA's rows, colour after colour (each colour's
-    // rows and their end), which the sweep keeps in shared memory: CTA b's list
-    // starts at rbase[b]; its colour c part at roff[b (nc + 1) + c]
-    DBuf<int64_t> rpl, rbase;
-    DBuf<int32_t> roff;
-    int smem = 0;                // dynamic shared memory of the launch (bytes)
+// One row of a many-coloured level's operator: its entries of lower colours at
+// [q0, q0 + nl), those of higher colours behind them.
+struct RowSplit {
+    int64_t q0;
+    int32_t nl, nu;
 };
-// what the sweep kernel reads of a FlagPlan
-struct FlagView {
-    const int64_t *rstart;
-    const int32_t *nbr, *nbrc;
-    const int64_t *rpl, *rbase;
-    const int32_t *roff;
+// One row in a warp's list of rows (gl_sweep.cu): its entries as above, the row (-1:
+// none), whether it belongs to the level's last colour (bit 0), and the entries per
+// lane of the longest lower (bits 1-15) and upper (bits 17-31) part among the rows
+// that the warp relaxes with it.
+struct alignas(16) RowDesc {
+    uint32_t q0;
+    uint32_t n;  // nl | nu << 16
+    int32_t row;
+    uint32_t flags;
 };
-inline FlagView flag_view(const FlagPlan &F) {
-    return FlagView{F.rstart.get(), F.nbr.get(), F.nbrc.get(), F.rpl.get(), F.rbase.get(), F.roff.get()};
-}
-constexpr int FLAG_SMEM_MAX = 40 * 1024;  // bound of a plan's shared-memory row pointers (bytes; with the
-                                          // kernel's static shared memory below the 48 KiB default)
+template <typename C>
+struct SplitCsr {
+    int64_t nrows = 0, nnz = 0;
+    DBuf<RowSplit> rows;
+    DBuf<int32_t> col;
+    DBuf<C> val;
+};
+// Everything the symmetric Gauss-Seidel steps of a level need in one precision
+// (gl_sweep.cu).
+constexpr int SWEEP_STATE_WORDS = 4;
+template <typename C, typename R>
+struct SweepData {
+    SplitCsr<C> A;
+    DBuf<R> idiag;               // 1 / A_ii
+    DBuf<C> xs;                  // two sets of forward and backward slots (dataflow form)
+    DBuf<unsigned> state;        // launches and CTAs done (dataflow), or the barrier's counter
+    DBuf<RowDesc> desc;          // every warp's rows
+    DBuf<int32_t> woff, cfirst;  // where a warp's list starts, and its part of every colour
+    int sync = 1;                // 1 dataflow, 0 grid barrier
+    int G = 2;                   // lanes per row
+    int K = 1;                   // shifts of warps that take the colours in turn
+    int PF = 4;                  // entries per lane loaded ahead
+    int nb = 1;                  // CTAs
+};
 
 struct Level {
     int64_t n = 0;
@@ -113,29 +114,23 @@ struct Level {
     // solve ordering (colour-major)
     DBuf<int32_t> perm_own, iperm_own;  // coarse levels own theirs; level 0 uses the mesh's
     const int32_t *perm = nullptr, *iperm = nullptr;
-    Sell<double2> A_own;            // coarse levels: off-diagonals of A
-    const Sell<double2> *A = nullptr;  // level 0 points at the mesh's K (row-scaled)
+    const Sell<double2> *A = nullptr;  // level 0: the mesh's K (row-scaled)
     DBuf<double> diag;              // level 0: K_ii + 2|psi_i|^2; else A_ii
-    Sell<double2> P, PH;            // permuted prolongator / its adjoint
-    CsrG<double2> Ag, PHg;          // grouped-CSR forms: coarse-level A (ell >= 1) and P^H
+    Sell<double2> P;                // permuted prolongator
+    CsrG<double2> PHg;              // its adjoint, grouped CSR
+    SweepData<double2, double> sw64;  // coarse levels: the operator in the form of the sweeps
+    SweepData<float2, float> sw32;
     DBuf<int64_t> cstart_dev;       // cstart on the device (cooperative sweeps)
-    DBuf<unsigned> barrier;         // grid-barrier state of the cooperative coarse sweeps
-    DBuf<unsigned long long> flags; // neighbour-flag sweeps: [precision][MAX_FLAG_CTAS][FLAG_STRIDE] counters
-    FlagPlan fl32, fl64;            // their partitions (FP32 / FP64 sweep)
-    int sync32 = 0, sync64 = 0;     // coarse sweep synchronisation: 0 grid barrier, 1 neighbour flags
     DBuf<double2> b, x, r;          // level vectors (solve ordering)
     DBuf<double2> Ainv;             // coarsest: dense inverse, row-major
     // FP32 copies (mixed precision)
-    Sell<float2> A32_own;
     const Sell<float2> *A32 = nullptr;
     DBuf<float> diag32;
-    Sell<float2> P32, PH32;
-    CsrG<float2> Ag32, PHg32;
+    Sell<float2> P32;
+    CsrG<float2> PHg32;
     CsrG<float2> PHg32b;            // level 0 with two colours: P^H without the colour-0 columns
     DBuf<float2> b32, x32, r32;
     DBuf<float4> Ainv_df;           // coarsest: the dense inverse as double-FP32 (re hi, re lo, im hi, im lo)
-    int cl_size = 0, cl_chunk = 0;  // FP32 sweeps by one thread-block cluster (0: cooperative grid)
-    int sgs_G32 = 1, sgs_G64 = 1;   // lanes per row of the coarse Gauss-Seidel sweeps
 };
 
 // R_inf (Eq. prec1): V-cycles until the scaled residual is RINF_TOL of the input
@@ -166,7 +161,6 @@ struct gl_prec_s {
     bool autotune = true;
     bool lattice = true;              // closed-form finest-level stencil in the FP32 V-cycle when available
     bool lattice64 = false;           // and MINRES's FP64 Jacobian from its FP64 tables (options.lattice = 2)
-    bool cluster_sweeps = true;       // FP32 coarse sweeps by one thread-block cluster when the level fits
     gl::Level L[gl::MAX_LEVELS];
     gl::DBuf<double2> psi_p;          // psi in solve ordering
     gl::DBuf<double2> cyc_r, cyc_e;   // work vectors for k > 1 cycles
@@ -180,8 +174,7 @@ struct gl_prec_s {
     int maxlev_used = 0, coloring_used = 0;
     // kernel choices taken over from a template instead of timing them again
     struct Tuned {
-        int ag64 = 1, phg64 = 1, sgs64 = 1, ag32 = 1, phg32 = 1, sgs32 = 1, cl_size = 0, cl_chunk = 0;
-        int sync64 = 0, nb64 = 0, sync32 = 0, nb32 = 0;
+        int phg64 = 1, sgs64 = 2, shifts64 = 1, sync64 = 1, phg32 = 1, sgs32 = 2, shifts32 = 1, sync32 = 1;
     } tuned[gl::MAX_LEVELS];
     int sweep_sync = 0;               // gl_options.sweep_sync the setup ran with
     bool coarse_df = true;            // FP32 V-cycle: double-FP32 coarsest product (else FP64)
@@ -316,14 +309,22 @@ void precond_apply_p(gl_prec_s *p, const double2 *v, double2 *z, const int *stop
 void precond_apply_p32(gl_prec_s *p, const float2 *v, float2 *z, const int *stop, cudaStream_t s);
 // autotuner: picks the lanes-per-row width of every grouped-CSR operator by timing
 void autotune_levels(gl_prec_s *p, bool fp32, cudaStream_t s);
-// picks, per coarse level, the lanes per row of the Gauss-Seidel sweep, its
-// synchronisation (grid barrier or neighbour flags) and (FP32) the
-// thread-block-cluster form (timed when autotuning)
+// gl_sweep.cu: the operator of a many-coloured level in the sweeps' form (and its
+// diagonal), in the solve ordering given by perm / iperm
+template <typename C>
+void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const CsrDev &A, SplitCsr<C> &out,
+                 double *diag_out, cudaStream_t s);
+// one symmetric Gauss-Seidel step on level l, from x = 0 (zero_start) or from x;
+// r (nullable, zero_start only) receives the residual b - A x times scale (nullable)
+template <typename T>
+void sweep_step(gl_prec_s *p, int l, const typename CT<T>::type *b, typename CT<T>::type *x, bool zero_start,
+                typename CT<T>::type *r, const T *scale, const int *stop, cudaStream_t s);
+// picks, per level, the form of the sweep and its lanes per row (timed when autotuning)
 void plan_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s);
-// rebuilds the neighbour-flag partitions of the sweep choices taken over from a template
-void rebuild_flag_plans(gl_prec_s *p, bool fp32, cudaStream_t s);
-// after a wait of the coarse sweeps ran out: zeroes every level's barrier
-// counters and flags and the error word, so later launches start in step
+// the same choices as a template's (p->tuned)
+void adopt_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s);
+// after a wait of the coarse sweeps ran out: zeroes every level's synchronisation
+// state and the error word, so later launches start in step
 void sweeps_reset(gl_prec_s *p, cudaStream_t s);
 // 1 if a device-side wait of p's sweeps ran out since the last reset (synchronises s)
 int sweeps_failed(gl_prec_s *p, cudaStream_t s);

@@ -1200,23 +1200,16 @@ void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_
             k_pdiag<<<grid_for(n, 256), 256, 0, s>>>(n, m->kdiag.get(), p->psi_p.get(), L.diag.get());
             GL_LAUNCH_CHECK();
         } else if (!coarsest) {
-            build_sell<double2>(L.n, L.n, L.perm, L.iperm, L.A_can, nullptr, true, L.A_own, L.diag.get(), s);
-            L.A = &L.A_own;
-            build_csrg<double2>(L.n, L.perm, L.iperm, L.A_can, true, L.Ag, nullptr, s);
+            build_split<double2>(L.n, L.perm, L.iperm, L.A_can, L.sw64.A, L.diag.get(), s);
             L.cstart_dev.alloc(L.ncolors + 1);
             GL_CUDA(cudaMemcpyAsync(L.cstart_dev.get(), L.cstart.data(), (L.ncolors + 1) * sizeof(int64_t),
                                     cudaMemcpyHostToDevice, s));
-            L.barrier.alloc(GRID_BARRIER_WORDS);
-            GL_CUDA(cudaMemsetAsync(L.barrier.get(), 0, GRID_BARRIER_WORDS * sizeof(unsigned), s));
-            L.flags.alloc(2 * (size_t)MAX_FLAG_CTAS * FLAG_STRIDE);
-            GL_CUDA(cudaMemsetAsync(L.flags.get(), 0, L.flags.bytes(), s));
         }
         if (!coarsest) {
             Level &Lc = p->L[k + 1];
             build_sell<double2>(L.n, Lc.n, L.perm, Lc.iperm, L.P_can, nullptr, false, L.P, nullptr, s);
             CsrDev PH;
             transpose_conj(L.P_can, PH, s);
-            build_sell<double2>(Lc.n, L.n, Lc.perm, L.iperm, PH, nullptr, false, L.PH, nullptr, s);
             build_csrg<double2>(Lc.n, Lc.perm, L.iperm, PH, false, L.PHg, nullptr, s);
         }
         L.b.alloc(L.n);
@@ -1284,40 +1277,28 @@ void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_
     p->autotune = o.autotune != 0;
     p->lattice = o.lattice != 0;
     p->lattice64 = o.lattice == 2;
-    p->cluster_sweeps = o.cluster_sweeps != 0;
     p->sweep_sync = o.sweep_sync;
     p->coarse_df = o.coarse_df != 0;
-    if (T && T->nlev == p->nlev && T->autotune == p->autotune && T->cluster_sweeps == p->cluster_sweeps &&
-        T->sweep_sync == p->sweep_sync) {
+    if (T && T->nlev == p->nlev && T->autotune == p->autotune && T->sweep_sync == p->sweep_sync) {
         for (int k = 0; k < p->nlev; ++k) {
             const Level &S = T->L[k];
             auto &t = p->tuned[k];
-            t.ag64 = S.Ag.G;
             t.phg64 = S.PHg.G;
-            t.sgs64 = S.sgs_G64;
-            t.ag32 = S.Ag32.G;
+            t.sgs64 = S.sw64.G;
+            t.shifts64 = S.sw64.K;
+            t.sync64 = S.sw64.sync;
             t.phg32 = S.PHg32.G;
-            t.sgs32 = S.sgs_G32;
-            t.cl_size = S.cl_size;
-            t.cl_chunk = S.cl_chunk;
-            t.sync64 = S.sync64;
-            t.nb64 = S.fl64.nb;
-            t.sync32 = S.sync32;
-            t.nb32 = S.fl32.nb;
+            t.sgs32 = S.sw32.G;
+            t.shifts32 = S.sw32.K;
+            t.sync32 = S.sw32.sync;
         }
         p->tuned64 = true;
         p->tuned32 = T->has32;
     }
     mark("solve-order operators, cost");
     if (p->tuned64) {
-        for (int k = 0; k < p->nlev; ++k) {
-            Level &L = p->L[k];
-            L.Ag.G = p->tuned[k].ag64;
-            L.PHg.G = p->tuned[k].phg64;
-            L.sgs_G64 = p->tuned[k].sgs64;
-            L.sync64 = p->tuned[k].sync64;
-        }
-        rebuild_flag_plans(p, false, s);
+        for (int k = 0; k < p->nlev; ++k) p->L[k].PHg.G = p->tuned[k].phg64;
+        adopt_sweeps(p, false, s);
     } else {
         if (p->autotune) autotune_levels(p, false, s);
         plan_sweeps(p, false, s);
@@ -1340,16 +1321,13 @@ void precond_ensure_fp32(gl_prec_s *p, cudaStream_t s) {
         if (k == 0) {
             L.A32 = &m->K32;
         } else if (!coarsest) {
-            build_sell<float2>(L.n, L.n, L.perm, L.iperm, L.A_can, nullptr, true, L.A32_own, nullptr, s);
-            L.A32 = &L.A32_own;
-            build_csrg<float2>(L.n, L.perm, L.iperm, L.A_can, true, L.Ag32, nullptr, s);
+            build_split<float2>(L.n, L.perm, L.iperm, L.A_can, L.sw32.A, nullptr, s);
         }
         if (!coarsest) {
             Level &Lc = p->L[k + 1];
             build_sell<float2>(L.n, Lc.n, L.perm, Lc.iperm, L.P_can, nullptr, false, L.P32, nullptr, s);
             CsrDev PH;
             transpose_conj(L.P_can, PH, s);
-            build_sell<float2>(Lc.n, L.n, Lc.perm, L.iperm, PH, nullptr, false, L.PH32, nullptr, s);
             build_csrg<float2>(Lc.n, Lc.perm, L.iperm, PH, false, L.PHg32, nullptr, s);
             // after the pre-smoothing of a red-black level 0 the residual of every
             // colour-0 row is zero, so its restriction needs only the other columns
@@ -1365,16 +1343,8 @@ void precond_ensure_fp32(gl_prec_s *p, cudaStream_t s) {
         p->cyc_e32.alloc(m->n);
     }
     if (p->tuned32) {
-        for (int k = 0; k < p->nlev; ++k) {
-            Level &L = p->L[k];
-            L.Ag32.G = p->tuned[k].ag32;
-            L.PHg32.G = p->tuned[k].phg32;
-            L.sgs_G32 = p->tuned[k].sgs32;
-            L.cl_size = p->tuned[k].cl_size;
-            L.cl_chunk = p->tuned[k].cl_chunk;
-            L.sync32 = p->tuned[k].sync32;
-        }
-        rebuild_flag_plans(p, true, s);
+        for (int k = 0; k < p->nlev; ++k) p->L[k].PHg32.G = p->tuned[k].phg32;
+        adopt_sweeps(p, true, s);
     } else {
         if (p->autotune) autotune_levels(p, true, s);
         plan_sweeps(p, true, s);

@@ -9,8 +9,6 @@
 // K + 2|psi|^2 = D^-1 (K-hat + 2 D|psi|^2): Gauss-Seidel on D^-1 A with right-hand
 // side v is Gauss-Seidel on A with right-hand side D v, and the residual handed
 // to the restriction is multiplied by D.
-#include <cooperative_groups.h>
-
 #include "gl_internal.cuh"
 #include "gl_kernels.cuh"
 #include "gl_profile.cuh"
@@ -25,8 +23,6 @@ struct LevelOps<double> {
     static const Sell<C> &A(const Level &L) { return *L.A; }
     static const double *diag(const Level &L) { return L.diag.get(); }
     static const Sell<C> &P(const Level &L) { return L.P; }
-    static const Sell<C> &PH(const Level &L) { return L.PH; }
-    static const CsrG<C> &Ag(const Level &L) { return L.Ag; }
     static const CsrG<C> &PHg(const Level &L) { return L.PHg; }
     static C *b(Level &L) { return L.b.get(); }
     static C *x(Level &L) { return L.x.get(); }
@@ -38,8 +34,6 @@ struct LevelOps<float> {
     static const Sell<C> &A(const Level &L) { return *L.A32; }
     static const float *diag(const Level &L) { return L.diag32.get(); }
     static const Sell<C> &P(const Level &L) { return L.P32; }
-    static const Sell<C> &PH(const Level &L) { return L.PH32; }
-    static const CsrG<C> &Ag(const Level &L) { return L.Ag32; }
     static const CsrG<C> &PHg(const Level &L) { return L.PHg32; }
     static C *b(Level &L) { return L.b32.get(); }
     static C *x(Level &L) { return L.x32.get(); }
@@ -324,745 +318,6 @@ __global__ void __launch_bounds__(256) k_spmv_g(CsrGView<C> S, const C *__restri
     if (ok && lane == 0) y[row] = add ? cadd(acc, y[row]) : acc;
 }
 
-// r = b - A x (coarse levels, no scaling), grouped CSR
-template <int G, typename C, typename R>
-__global__ void __launch_bounds__(256) k_resid_g(CsrGView<C> A, const R *__restrict__ diag, const C *__restrict__ b,
-                                                 const C *__restrict__ x, C *__restrict__ r,
-                                                 const int *__restrict__ stop) {
-    if (stop && *stop) return;
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t row = t / G;
-    int lane = (int)(t % G);
-    bool ok = row < A.nrows;
-    C acc = group_row<G, C>(A, ok ? row : -1, lane, x, INT64_MAX);
-    if (ok && lane == 0) {
-        C xx = x[row], bb = b[row];
-        R d = diag[row];
-        r[row] = mk(bb.x - acc.x - d * xx.x, bb.y - acc.y - d * xx.y);
-    }
-}
-
-// ---------------------------------------------------------------- coarse-level SGS
-// Every wait of the coarse sweeps is bounded by SWEEP_WAIT_NS of the global
-// timer.  A wait that runs out sets the preconditioner's error word and, when
-// the launch belongs to a solve, the solve's status word to STATUS_TIMEOUT, so
-// every later kernel of the solve returns at once and the host reports
-// GL_ERR_TIMEOUT; every sweep launch returns at once while the error word is
-// set, until the host resets the synchronisation state (sweeps_reset).
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_u64(unsigned long long *p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-// spins until *p >= want; false if SWEEP_WAIT_NS passed first
-__device__ __forceinline__ bool spin_geq(const unsigned long long *p, unsigned long long want) {
-    if (ld_acquire_u64(p) >= want) return true;
-    const unsigned long long t0 = globaltimer_ns();
-    for (unsigned spins = 1;; ++spins) {
-        if (ld_acquire_u64(p) >= want) return true;
-        if ((spins & 63u) == 0 && globaltimer_ns() - t0 > (unsigned long long)SWEEP_WAIT_NS) return false;
-    }
-}
-__device__ __forceinline__ void report_timeout(int *err, int *stop) {
-    atomicExch(err, 1);
-    if (stop) atomicExch(stop, STATUS_TIMEOUT);
-}
-__device__ __forceinline__ bool sweep_halted(const int *stop, const int *err) {
-    return (stop && *(volatile const int *)stop) || *(volatile const int *)err;
-}
-
-// Grid barrier of the cooperative sweeps: one 64-bit arrival counter per
-// (level, precision) that only grows.  Every launch on a counter uses the same
-// number of CTAs nb, so the counter is a multiple of nb between launches.  At
-// its first barrier a CTA takes a ticket with an atomic add (the round trip
-// tells it the launch's base: the ticket rounded down to a multiple of nb); at
-// every later barrier it only adds one with a release reduction that it does
-// not wait for.  Barrier k is passed when the counter reaches base + (k+1) nb,
-// which one thread per CTA observes with acquiring loads.  So the critical path
-// from the last CTA's work to everybody's next phase is one release reduction
-// and the loads that see it.  The release/acquire pair, after a CTA-wide
-// __syncthreads on both sides, orders every thread's x writes before the other
-// CTAs' reads.  (A flag per CTA polled by one warp, and a counter reset by the
-// last arriver, measured slower.)  A CTA that gives up a wait leaves the
-// counter out of step; the host zeroes it (sweeps_reset) before the next use.
-// arrival at barrier k; thread 0's base is set at k = 0
-__device__ __forceinline__ void grid_arrive(unsigned long long *cnt, unsigned k, unsigned long long &base) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (k == 0) {
-            unsigned long long t;
-            asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(t) : "l"(cnt) : "memory");
-            base = t - t % gridDim.x;
-        } else {
-            asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(cnt) : "memory");
-        }
-    }
-}
-// waits for barrier k; false if the wait ran out (thread 0 holds base and the
-// extra offset of every wait target, nonzero only when a test has asked for
-// waits that cannot end)
-__device__ __forceinline__ bool grid_wait(const unsigned long long *cnt, unsigned k, unsigned long long base,
-                                          unsigned long long extra, int *err, int *stop) {
-    __shared__ int ok;
-    if (threadIdx.x == 0) {
-        const unsigned long long want = base + (unsigned long long)(k + 1) * gridDim.x + extra;
-        ok = spin_geq(cnt, want) ? 1 : 0;
-        if (!ok) report_timeout(err, stop);
-    }
-    __syncthreads();
-    return ok;
-}
-
-// One symmetric Gauss-Seidel step on a coarse level in a single cooperative
-// launch: colours 0..nc-1 forward then nc-2..0 backward, a grid barrier between
-// colours.  zero_start: the forward pass starts from x = 0 (only columns of
-// earlier colours are read).  Between arriving at and leaving a barrier each
-// group loads the structure, values, b and diagonal of its row in the next
-// colour (they do not depend on x), so after the barrier only the neighbour
-// gathers remain.  The gathers are plain cached loads: other blocks wrote the
-// values, but every phase starts behind an acquiring load of the wait (and a CTA
-// barrier), which the memory model orders before them, and within a phase no
-// block writes the colours its rows read; the rows of a colour share many
-// neighbours, which then come from L1 (measured 3% faster than L2-only loads).
-constexpr int PF = 8;  // prefetched entries per lane
-
-template <typename R>
-constexpr int coop_threads() {
-    return sizeof(R) == 8 ? 512 : 1024;  // FP64 rows need more registers per thread
-}
-
-// relaxes the rows [lo, hi) of colour c (first round prefetched) with gpn groups
-// of G lanes; `lim`: only columns below it are read (first sweep from zero)
-template <int G, typename C, typename R>
-struct SweepRows {
-    CsrGView<C> A;
-    const R *__restrict__ diag;
-    const C *__restrict__ b;
-    C *x;
-    int lane;
-    int32_t pcol[PF];
-    C pval[PF];
-    C pb;
-    R pd = 1;
-    int64_t pq0 = 0, pq1 = 0;
-    __device__ SweepRows(const CsrGView<C> &A_, const R *d_, const C *b_, C *x_, int lane_)
-        : A(A_), diag(d_), b(b_), x(x_), lane(lane_) {
-        pb.x = 0;
-        pb.y = 0;
-    }
-    // loads the x-independent data of row `row` (first round of a phase)
-    __device__ __forceinline__ void prefetch(int64_t row, bool ok) {
-        if (ok)
-            prefetch_q(row, true, A.rp[row], A.rp[row + 1]);
-        else
-            prefetch_q(row, false, 0, 0);
-    }
-    // the same with the row's entry range [q0, q1) given
-    __device__ __forceinline__ void prefetch_q(int64_t row, bool ok, int64_t q0, int64_t q1) {
-        pq0 = pq1 = 0;
-        if (ok) {
-            pq0 = q0;
-            pq1 = q1;
-            pb = b[row];
-            pd = diag[row];
-        }
-#pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            int64_t q = pq0 + lane + (int64_t)k * G;
-            if (q < pq1) {
-                pcol[k] = __ldg(A.col + q);
-                pval[k] = A.val[q];
-            }
-        }
-    }
-    // one round: row (of this group) relaxed; k == 0 uses the prefetched data;
-    // none: every neighbour still holds zero (first colour from a zero guess)
-    __device__ __forceinline__ void relax(int64_t row, bool ok, int64_t k, int64_t lim, bool none) {
-        C acc;
-        acc.x = 0;
-        acc.y = 0;
-        if (!none) {
-            if (k == 0) {
-#pragma unroll
-                for (int e = 0; e < PF; ++e) {
-                    int64_t q = pq0 + lane + (int64_t)e * G;
-                    if (q < pq1 && pcol[e] < lim) cfma(acc, pval[e], __ldca(x + pcol[e]));
-                }
-                for (int64_t q = pq0 + lane + (int64_t)PF * G; q < pq1; q += G) {
-                    int32_t cc = __ldg(A.col + q);
-                    if (cc < lim) cfma(acc, A.val[q], __ldca(x + cc));
-                }
-            } else if (ok) {
-                for (int64_t q = A.rp[row] + lane; q < A.rp[row + 1]; q += G) {
-                    int32_t cc = __ldg(A.col + q);
-                    if (cc < lim) cfma(acc, A.val[q], __ldca(x + cc));
-                }
-            }
-        }
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) {
-            acc.x += __shfl_down_sync(0xffffffffu, acc.x, o, G);
-            acc.y += __shfl_down_sync(0xffffffffu, acc.y, o, G);
-        }
-        if (ok && lane == 0) {
-            C bb = (k == 0) ? pb : b[row];
-            R d = (R)1 / ((k == 0) ? pd : diag[row]);
-            x[row] = mk((bb.x - acc.x) * d, (bb.y - acc.y) * d);
-        }
-    }
-};
-
-template <int G, typename C, typename R>
-__global__ void __launch_bounds__(coop_threads<R>()) k_sgs_coop(CsrGView<C> A, const R *__restrict__ diag,
-                                                                const int64_t *__restrict__ cstart, int ncolors,
-                                                                const C *__restrict__ b, C *x, int zero_start,
-                                                                unsigned *bar, const unsigned long long *extra_p,
-                                                                int *err, int *stop) {
-    if (sweep_halted(stop, err)) return;
-    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(bar) + (sizeof(R) == 4 ? 0 : 1);
-    unsigned long long base = 0;
-    const unsigned long long extra = threadIdx.x == 0 ? *extra_p : 0ull;
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t grp = t / G, ngroups = (int64_t)gridDim.x * blockDim.x / G;
-    SweepRows<G, C, R> S(A, diag, b, x, (int)(t % G));
-    int nphase = 2 * ncolors - 1;
-    auto colour_of = [&](int ph) { return ph < ncolors ? ph : 2 * ncolors - 2 - ph; };
-    {
-        int c = colour_of(0);
-        S.prefetch(cstart[c] + grp, cstart[c] + grp < cstart[c + 1]);
-    }
-    for (int ph = 0; ph < nphase; ++ph) {
-        int c = colour_of(ph);
-        bool first = zero_start && ph < ncolors;
-        int64_t lo = cstart[c], hi = cstart[c + 1];
-        int64_t lim = first ? lo : INT64_MAX;
-        int64_t rounds = (hi - lo + ngroups - 1) / ngroups;
-        for (int64_t k = 0; k < rounds; ++k) {
-            int64_t row = lo + k * ngroups + grp;
-            S.relax(row, row < hi, k, lim, first && lo == 0);
-        }
-        if (ph + 1 < nphase) {
-            // arrive, load the next colour's x-independent data, then wait
-            grid_arrive(cnt, (unsigned)ph, base);
-            int cn = colour_of(ph + 1);
-            S.prefetch(cstart[cn] + grp, cstart[cn] + grp < cstart[cn + 1]);
-            if (!grid_wait(cnt, (unsigned)ph, base, extra, err, stop)) return;
-        }
-    }
-}
-
-// The same symmetric step with neighbour flags instead of the grid barrier.
-// CTA b owns a chunk of every colour's rows (FlagPlan) and after each
-// phase publishes, with a release store, the number of phases it has
-// completed; before phase ph (colour c) it waits, with acquiring loads, only
-// until every CTA owning a column of its colour-c rows has completed phase
-// ph - 1.  That CTA's last write of any such column came in a phase <= ph - 1,
-// and its reads of b's colour-c rows since their previous relaxation also lie
-// in phases <= ph - 1, so every row reads exactly the values the grid-barrier
-// sweep gives it: the two forms are bit-identical for the same G.  CTAs far
-// apart may then run several phases apart.  Counters only grow: a launch adds
-// 2 nc - 1 to each, so all CTAs of a launch start from the same value (a CTA
-// reads its own at the start); a CTA without rows in a colour only counts the
-// phase.
-//
-// The phase is a chain of latencies (the hand-off from the CTAs it reads, the
-// gathers of their x, the fence behind this CTA's writes), so the kernel keeps
-// everything else off it: warp 0 holds no rows and only publishes and polls,
-// starting its poll right after the release; the other warps relax the rows
-// and, before the phase is published, issue the loads of the next phase's
-// x-independent data (columns, values, b, diagonal) with row pointers from
-// shared memory, where the CTA's row pointers of all colours sit for the whole
-// launch, so no load waits on another.
-template <int G, typename C, typename R>
-__global__ void __launch_bounds__(coop_threads<R>()) k_sgs_flags(CsrGView<C> A, const R *__restrict__ diag,
-                                                                 const int64_t *__restrict__ cstart, int ncolors,
-                                                                 FlagView F, const C *__restrict__ b, C *x,
-                                                                 int zero_start, unsigned long long *flags,
-                                                                 const unsigned long long *extra_p, int *err,
-                                                                 int *stop) {
-    if (sweep_halted(stop, err)) return;
-    constexpr int NT = coop_threads<R>();
-    constexpr int GPB = (NT - 32) / G;  // row groups (rows per round) of the worker warps
-    // dynamic shared memory: this CTA's rows [s_lo[c], s_hi[c]) of every colour,
-    // the offsets s_roff[c] of their row pointers in s_rp, and the row pointers
-    extern __shared__ int64_t s_dyn[];
-    int64_t *s_lo = s_dyn, *s_hi = s_dyn + ncolors;
-    int32_t *s_roff = reinterpret_cast<int32_t *>(s_dyn + 2 * ncolors);
-    int64_t *s_rp = s_dyn + 2 * ncolors + (ncolors + 2) / 2;
-    const int nb = gridDim.x, cta = blockIdx.x;
-    const bool worker = threadIdx.x >= 32;
-    const int grp = worker ? (int)(threadIdx.x - 32) / G : 0;
-    unsigned long long *mine = flags + (size_t)cta * FLAG_STRIDE;
-    // the launch's starting count, and the offset of every wait target (nonzero
-    // only when a test asks for waits that cannot end), kept in shared memory
-    __shared__ unsigned long long s_base, s_target0;
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        s_base = *(volatile unsigned long long *)mine;
-        s_target0 = s_base + *extra_p;
-    }
-    for (int c = threadIdx.x; c <= ncolors; c += NT) {
-        s_roff[c] = F.roff[(int64_t)cta * (ncolors + 1) + c];
-        if (c < ncolors) {
-            s_lo[c] = F.rstart[(int64_t)c * (nb + 1) + cta];
-            s_hi[c] = F.rstart[(int64_t)c * (nb + 1) + cta + 1];
-        }
-    }
-    __syncthreads();
-    {
-        const int64_t *src = F.rpl + F.rbase[cta];
-        const int total = s_roff[ncolors];
-        for (int i0 = threadIdx.x; i0 < total; i0 += 4 * NT) {
-            int64_t v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + u * NT < total) v[u] = __ldg(src + i0 + u * NT);
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (i0 + u * NT < total) s_rp[i0 + u * NT] = v[u];
-        }
-    }
-    __syncthreads();
-    SweepRows<G, C, R> S(A, diag, b, x, (int)(threadIdx.x % G));
-    const int nphase = 2 * ncolors - 1;
-    auto colour_of = [&](int ph) { return ph < ncolors ? ph : 2 * ncolors - 2 - ph; };
-    auto rows_of = [&](int c, int64_t &lo, int64_t &hi) {
-        lo = s_lo[c];
-        hi = s_hi[c];
-    };
-    // the x-independent data of this group's first row of colour c (later rounds
-    // of a phase, rare, load their own)
-    auto prefetch = [&](int c) {
-        int64_t lo, hi;
-        rows_of(c, lo, hi);
-        const bool ok = lo + grp < hi;
-        const int32_t i = s_roff[c] + grp;
-        S.prefetch_q(lo + grp, ok, ok ? s_rp[i] : 0, ok ? s_rp[i + 1] : 0);
-    };
-    if (worker) prefetch(colour_of(0));
-    for (int ph = 0; ph < nphase; ++ph) {
-        const int c = colour_of(ph);
-        const bool first = zero_start && ph < ncolors;
-        const int64_t clo = cstart[c];
-        const int64_t lim = first ? clo : INT64_MAX;
-        int64_t lo, hi;
-        rows_of(c, lo, hi);
-        if (ph > 0 && hi > lo) {
-            if (!worker) {
-                const int64_t li = (int64_t)cta * ncolors + c;
-                const int cnt = F.nbrc[li];
-                bool ok = true;
-                if ((int)threadIdx.x < cnt)
-                    ok = spin_geq(flags + (size_t)F.nbr[li * FLAG_MAXN + threadIdx.x] * FLAG_STRIDE,
-                                  s_target0 + (unsigned long long)ph);
-                ok = __all_sync(0xffffffffu, ok);
-                if (threadIdx.x == 0) {
-                    s_ok = ok ? 1 : 0;
-                    if (!ok) report_timeout(err, stop);
-                }
-            }
-            __syncthreads();
-            if (!s_ok) return;
-        }
-        if (worker) {
-            const int64_t rounds = (hi - lo + GPB - 1) / GPB;
-            for (int64_t k = 0; k < rounds; ++k) {
-                const int64_t row = lo + k * GPB + grp;
-                S.relax(row, row < hi, k, lim, first && clo == 0);
-            }
-            // the next phase's x-independent data, before this phase is published
-            if (ph + 1 < nphase) prefetch(colour_of(ph + 1));
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) st_release_u64(mine, s_base + (unsigned long long)ph + 1);
-    }
-}
-
-// ---- partition of the neighbour-flag sweep
-// Each colour's positions are split into nb equal contiguous chunks: CTA b owns
-// positions [cstart[c] + floor(b m_c / nb), cstart[c] + floor((b + 1) m_c / nb))
-// of colour c (m_c its size).  The positions of a colour hold ascending node
-// ids, so chunk b of every colour covers about the same part of the level
-// (node ids follow space), and no CTA has more than ceil(m_c / nb) rows of a
-// colour, which keeps every phase to one round of rows where a partition by
-// node id would give some CTAs a second one.
-__device__ __forceinline__ int64_t chunk_start(int64_t m, int nb, int b) { return m * b / nb; }
-// owner CTA of solve position q
-__device__ __forceinline__ int flag_owner(int64_t q, const int64_t *__restrict__ cstart, int ncolors, int nb) {
-    int lo = 0, hi = ncolors - 1;  // colour c with cstart[c] <= q < cstart[c + 1]
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) / 2;
-        if (cstart[mid] <= q)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    const int64_t m = cstart[lo + 1] - cstart[lo], r = q - cstart[lo];
-    int64_t o = m > 0 ? r * nb / m : 0;
-    while (o + 1 < nb && chunk_start(m, nb, (int)o + 1) <= r) ++o;
-    while (o > 0 && chunk_start(m, nb, (int)o) > r) --o;
-    return (int)o;
-}
-// rstart[c (nb + 1) + b] = first position of CTA b's chunk of colour c
-__global__ void k_flag_rstart(int nb, int ncolors, const int64_t *__restrict__ cstart,
-                              int64_t *__restrict__ rstart) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= (int64_t)ncolors * (nb + 1)) return;
-    const int c = (int)(i / (nb + 1));
-    const int bb = (int)(i % (nb + 1));
-    rstart[i] = cstart[c] + chunk_start(cstart[c + 1] - cstart[c], nb, bb);
-}
-// the CTAs owning a column of CTA b's colour-c rows (b itself left out); the
-// list length is stored even when it exceeds FLAG_MAXN (the host then drops
-// the plan)
-template <typename C>
-__global__ void __launch_bounds__(256) k_flag_nbrs(CsrGView<C> A, int nb, int ncolors,
-                                                   const int64_t *__restrict__ cstart,
-                                                   const int64_t *__restrict__ rstart, int32_t *__restrict__ nbr,
-                                                   int32_t *__restrict__ nbrc) {
-    __shared__ unsigned bits[MAX_FLAG_CTAS / 32];
-    const int bb = blockIdx.x, c = blockIdx.y;
-    for (int w = threadIdx.x; w < MAX_FLAG_CTAS / 32; w += blockDim.x) bits[w] = 0u;
-    __syncthreads();
-    const int64_t lo = rstart[(int64_t)c * (nb + 1) + bb], hi = rstart[(int64_t)c * (nb + 1) + bb + 1];
-    for (int64_t row = lo + threadIdx.x; row < hi; row += blockDim.x)
-        for (int64_t q = A.rp[row]; q < A.rp[row + 1]; ++q) {
-            const int o = flag_owner(A.col[q], cstart, ncolors, nb);
-            if (o != bb) atomicOr(&bits[o >> 5], 1u << (o & 31));
-        }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int64_t li = (int64_t)bb * ncolors + c;
-        int cnt = 0;
-        for (int w = 0; w < MAX_FLAG_CTAS / 32; ++w) {
-            unsigned m = bits[w];
-            while (m) {
-                const int o = w * 32 + __ffs(m) - 1;
-                m &= m - 1;
-                if (cnt < FLAG_MAXN) nbr[li * FLAG_MAXN + cnt] = o;
-                ++cnt;
-            }
-        }
-        nbrc[li] = cnt;
-    }
-}
-
-// rpl[rbase[b] + roff[b][c] + i] = A.rp[lo + i], i = 0 .. hi - lo, for CTA b's
-// rows [lo, hi) of colour c
-template <typename C>
-__global__ void __launch_bounds__(256) k_flag_rpl(CsrGView<C> A, int nb, int ncolors,
-                                                  const int64_t *__restrict__ rstart, const int32_t *__restrict__ roff,
-                                                  const int64_t *__restrict__ rbase, int64_t *__restrict__ rpl) {
-    const int bb = blockIdx.x, c = blockIdx.y;
-    const int64_t lo = rstart[(int64_t)c * (nb + 1) + bb], hi = rstart[(int64_t)c * (nb + 1) + bb + 1];
-    int64_t *dst = rpl + rbase[bb] + roff[(int64_t)bb * (ncolors + 1) + c];
-    for (int64_t i = threadIdx.x; i <= hi - lo; i += blockDim.x) dst[i] = A.rp[lo + i];
-}
-
-// resident CTAs per SM of a sweep kernel and the SM count (queried once per kernel)
-template <typename K>
-static void sweep_residency(K kern, int threads, int &per_sm, int &nsm, size_t smem = 0) {
-    int dev = 0;
-    GL_CUDA(cudaGetDevice(&dev));
-    GL_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    GL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
-    GL_REQUIRE(per_sm > 0, GL_ERR_CUDA, "cooperative sweep kernel cannot be resident");
-}
-
-template <typename K, typename... Args>
-static void launch_coop_smem(K kern, int grid, int threads, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    GL_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
-}
-template <typename K, typename... Args>
-static void launch_coop(K kern, int grid, int threads, cudaStream_t s, Args... args) {
-    launch_coop_smem(kern, grid, threads, 0, s, args...);
-}
-
-template <int G, typename C, typename R>
-static void launch_sgs_coop(const CsrG<C> &A, const R *diag, const int64_t *cstart, int nc, const C *b, C *x,
-                            int zero_start, unsigned *bar, const unsigned long long *extra, int *err, int *stop,
-                            int64_t max_colour, cudaStream_t s) {
-    static int per_sm = -1, nsm = 0;
-    const int threads = coop_threads<R>();
-    if (per_sm < 0) sweep_residency(k_sgs_coop<G, C, R>, threads, per_sm, nsm);
-    int64_t want = (max_colour * G + threads - 1) / threads;
-    int grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), (int64_t)per_sm * nsm);
-    launch_coop(k_sgs_coop<G, C, R>, grid, threads, s, A.view(), diag, cstart, nc, b, x, zero_start, bar, extra, err,
-                stop);
-}
-
-// most CTAs a neighbour-flag sweep of G lanes per row may use (all resident,
-// with the largest shared memory a plan may ask for)
-template <int G, typename C, typename R>
-static int flags_max_ctas() {
-    static int per_sm = -1, nsm = 0;
-    if (per_sm < 0) sweep_residency(k_sgs_flags<G, C, R>, coop_threads<R>(), per_sm, nsm, FLAG_SMEM_MAX);
-    return std::min(per_sm * nsm, MAX_FLAG_CTAS);
-}
-
-template <int G, typename C, typename R>
-static void launch_sgs_flags(const CsrG<C> &A, const R *diag, const int64_t *cstart, int nc, const FlagPlan &F,
-                             const C *b, C *x, int zero_start, unsigned long long *flags,
-                             const unsigned long long *extra, int *err, int *stop, cudaStream_t s) {
-    const bool matches = F.nb > 0 && F.nb <= flags_max_ctas<G, C, R>() && F.G == G && F.smem <= FLAG_SMEM_MAX;
-    GL_REQUIRE(matches, GL_ERR_ARG, "neighbour-flag sweep without a matching partition");
-    launch_coop_smem(k_sgs_flags<G, C, R>, F.nb, coop_threads<R>(), (size_t)F.smem, s, A.view(), diag, cstart, nc,
-                     flag_view(F), b, x, zero_start, flags, extra, err, stop);
-}
-
-// Builds the neighbour-flag partition of a coarse level for nb CTAs of G lanes
-// per row.  Returns the longest neighbour list (the plan is usable if it is at
-// most FLAG_MAXN); synchronises s.
-template <typename C>
-static int build_flag_plan(const Level &L, const CsrG<C> &A, int G, int nb, FlagPlan &F, cudaStream_t s) {
-    F.nb = 0;
-    F.G = G;
-    GL_REQUIRE(nb >= 1 && nb <= MAX_FLAG_CTAS, GL_ERR_ARG, "neighbour-flag sweep: bad CTA count");
-    const int nc = L.ncolors;
-    F.rstart.alloc((size_t)nc * (nb + 1));
-    F.nbr.alloc((size_t)nb * nc * FLAG_MAXN);
-    F.nbrc.alloc((size_t)nb * nc);
-    k_flag_rstart<<<grid_for((int64_t)nc * (nb + 1), 256), 256, 0, s>>>(nb, nc, L.cstart_dev.get(), F.rstart.get());
-    GL_LAUNCH_CHECK();
-    k_flag_nbrs<C><<<dim3(nb, nc), 256, 0, s>>>(A.view(), nb, nc, L.cstart_dev.get(), F.rstart.get(), F.nbr.get(),
-                                                F.nbrc.get());
-    GL_LAUNCH_CHECK();
-    std::vector<int32_t> cnt((size_t)nb * nc);
-    std::vector<int64_t> rs((size_t)nc * (nb + 1));
-    GL_CUDA(cudaMemcpyAsync(cnt.data(), F.nbrc.get(), cnt.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    GL_CUDA(cudaMemcpyAsync(rs.data(), F.rstart.get(), rs.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    GL_CUDA(cudaStreamSynchronize(s));
-    int mx = 0;
-    for (int32_t v : cnt) mx = std::max(mx, (int)v);
-    // each CTA's row pointers, colour after colour: its rows of colour c and their end
-    std::vector<int32_t> roff((size_t)nb * (nc + 1));
-    std::vector<int64_t> rbase(nb + 1);
-    int64_t most = 0;
-    rbase[0] = 0;
-    for (int bb = 0; bb < nb; ++bb) {
-        int32_t o = 0;
-        for (int c = 0; c < nc; ++c) {
-            roff[(size_t)bb * (nc + 1) + c] = o;
-            o += (int32_t)(rs[(size_t)c * (nb + 1) + bb + 1] - rs[(size_t)c * (nb + 1) + bb]) + 1;
-        }
-        roff[(size_t)bb * (nc + 1) + nc] = o;
-        rbase[bb + 1] = rbase[bb] + o;
-        most = std::max<int64_t>(most, o);
-    }
-    // the kernel's layout: lo and hi per colour, nc + 1 offsets (int32), the row pointers
-    F.smem = (int)std::min<int64_t>((2 * nc + (nc + 2) / 2 + most) * (int64_t)sizeof(int64_t), INT32_MAX);
-    F.roff.alloc(roff.size());
-    F.rbase.alloc(nb + 1);
-    F.rpl.alloc((size_t)std::max<int64_t>(rbase[nb], 1));
-    GL_CUDA(cudaMemcpyAsync(F.roff.get(), roff.data(), roff.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    GL_CUDA(cudaMemcpyAsync(F.rbase.get(), rbase.data(), rbase.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    k_flag_rpl<<<dim3(nb, nc), 256, 0, s>>>(A.view(), nb, nc, F.rstart.get(), F.roff.get(), F.rbase.get(), F.rpl.get());
-    GL_LAUNCH_CHECK();
-    GL_CUDA(cudaStreamSynchronize(s));
-    if (mx <= FLAG_MAXN && F.smem <= FLAG_SMEM_MAX) F.nb = nb;
-    return F.smem <= FLAG_SMEM_MAX ? mx : FLAG_MAXN + 1;
-}
-
-// ---------------------------------------------------------------- cluster sweeps
-// One thread-block cluster runs a whole symmetric Gauss-Seidel step of a coarse
-// level in FP32.  The level's x lives in the distributed shared memory of the
-// cluster: CTA r holds positions [r chunk, (r + 1) chunk).  Rows of a colour are
-// spread over all the cluster's threads (G lanes per row); neighbour values are
-// read from the owning CTA's shared memory and new values written there, and
-// consecutive colours are separated by the cluster's hardware barrier, split
-// into arrive and wait so that the next colour's x-independent data (row
-// bounds, columns, values, b, diagonal) is loaded in between.  The same colour
-// order and the same first-sweep rule (from x = 0, later colours are still 0) as
-// the cooperative kernel.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
-constexpr int CLUSTER_THREADS = 1024;
-
-template <int G>
-__global__ void __launch_bounds__(CLUSTER_THREADS) k_sgs_cluster(CsrGView<float2> A, const float *__restrict__ diag,
-                                                                 const int64_t *__restrict__ cstart, int ncolors,
-                                                                 const float2 *__restrict__ b, float2 *x,
-                                                                 int zero_start, int chunk, float inv_chunk,
-                                                                 const int *__restrict__ stop) {
-    extern __shared__ float2 xs[];
-    if (stop && *stop) return;
-    namespace cgs = cooperative_groups;
-    cgs::cluster_group cl = cgs::this_cluster();
-    const int rank = (int)cl.block_rank();
-    const int nblk = (int)cl.num_blocks();
-    const int64_t n = A.nrows;
-    const int64_t base = (int64_t)rank * chunk;
-    const int64_t mine = std::max<int64_t>(0, std::min<int64_t>(chunk, n - base));
-    for (int64_t i = threadIdx.x; i < mine; i += blockDim.x) xs[i] = zero_start ? make_float2(0.f, 0.f) : x[base + i];
-    // owning CTA and offset of position c
-    auto owner_of = [&](int32_t c) {
-        int o = (int)((float)c * inv_chunk);
-        if ((int64_t)o * chunk > c) --o;
-        else if ((int64_t)(o + 1) * chunk <= c) ++o;
-        return o;
-    };
-    auto xget = [&](int32_t c) {
-        const int o = owner_of(c);
-        return cl.map_shared_rank(xs, o)[c - (int64_t)o * chunk];
-    };
-    const int64_t t = (int64_t)rank * blockDim.x + threadIdx.x;
-    const int64_t grp = t / G, ngroups = (int64_t)nblk * blockDim.x / G;
-    const int lane = (int)(t % G);
-    const int nphase = 2 * ncolors - 1;
-    int32_t pcol[PF];
-    float2 pval[PF];
-    float2 pb = make_float2(0.f, 0.f);
-    float pd = 1.f;
-    int64_t pq0 = 0, pq1 = 0;
-    auto colour_of = [&](int ph) { return ph < ncolors ? ph : 2 * ncolors - 2 - ph; };
-    auto prefetch = [&](int64_t row, bool ok) {
-        pq0 = pq1 = 0;
-        if (ok) {
-            pq0 = A.rp[row];
-            pq1 = A.rp[row + 1];
-            pb = b[row];
-            pd = diag[row];
-        }
-#pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            int64_t q = pq0 + lane + (int64_t)k * G;
-            if (q < pq1) {
-                pcol[k] = __ldg(A.col + q);
-                pval[k] = A.val[q];
-            }
-        }
-    };
-    cluster_arrive();
-    {
-        int c = colour_of(0);
-        prefetch(cstart[c] + grp, cstart[c] + grp < cstart[c + 1]);
-    }
-    cluster_wait();
-    for (int ph = 0; ph < nphase; ++ph) {
-        const int c = colour_of(ph);
-        const bool first = zero_start && ph < ncolors;
-        const int64_t lo = cstart[c], hi = cstart[c + 1];
-        const int64_t rounds = (hi - lo + ngroups - 1) / ngroups;
-        for (int64_t k = 0; k < rounds; ++k) {
-            const int64_t row = lo + k * ngroups + grp;
-            const bool ok = row < hi;
-            float2 acc = make_float2(0.f, 0.f);
-            if (!(first && lo == 0)) {
-                if (k == 0) {
-#pragma unroll
-                    for (int e = 0; e < PF; ++e) {
-                        int64_t q = pq0 + lane + (int64_t)e * G;
-                        if (q < pq1) cfma(acc, pval[e], xget(pcol[e]));
-                    }
-                    for (int64_t q = pq0 + lane + (int64_t)PF * G; q < pq1; q += G)
-                        cfma(acc, A.val[q], xget(__ldg(A.col + q)));
-                } else if (ok) {
-                    for (int64_t q = A.rp[row] + lane; q < A.rp[row + 1]; q += G)
-                        cfma(acc, A.val[q], xget(__ldg(A.col + q)));
-                }
-            }
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                acc.x += __shfl_down_sync(0xffffffffu, acc.x, o, G);
-                acc.y += __shfl_down_sync(0xffffffffu, acc.y, o, G);
-            }
-            if (ok && lane == 0) {
-                const float2 bb = (k == 0) ? pb : b[row];
-                const float d = 1.f / ((k == 0) ? pd : diag[row]);
-                const int o = owner_of((int32_t)row);
-                cl.map_shared_rank(xs, o)[row - (int64_t)o * chunk] =
-                    make_float2((bb.x - acc.x) * d, (bb.y - acc.y) * d);
-            }
-        }
-        cluster_arrive();
-        if (ph + 1 < nphase) {
-            const int cn = colour_of(ph + 1);
-            prefetch(cstart[cn] + grp, cstart[cn] + grp < cstart[cn + 1]);
-        }
-        cluster_wait();
-    }
-    for (int64_t i = threadIdx.x; i < mine; i += blockDim.x) x[base + i] = xs[i];
-}
-
-// cluster size (16 with the non-portable opt-in, else 8) and chunk for a level
-// of n rows whose x fits the cluster's shared memory; size 0 if none fits
-template <int G>
-static void plan_sgs_cluster(int64_t n, int &size, int &chunk) {
-    size = 0;
-    chunk = 0;
-    if (n <= 0) return;
-    GL_CUDA(cudaFuncSetAttribute(k_sgs_cluster<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    for (int cs : {16, 8}) {
-        int64_t ch = (n + cs - 1) / cs;
-        int64_t smem = ch * (int64_t)sizeof(float2);
-        if (smem > 200 * 1024) continue;
-        GL_CUDA(cudaFuncSetAttribute(k_sgs_cluster<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cs);
-        cfg.blockDim = dim3(CLUSTER_THREADS);
-        cfg.dynamicSmemBytes = (size_t)smem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cs;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int nclusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&nclusters, k_sgs_cluster<G>, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
-        if (nclusters >= 1) {
-            size = cs;
-            chunk = (int)ch;
-            return;
-        }
-    }
-}
-
-template <int G>
-static void launch_sgs_cluster(const CsrG<float2> &A, const float *diag, const int64_t *cstart, int nc,
-                               const float2 *b, float2 *x, int zero_start, int size, int chunk, const int *stop,
-                               cudaStream_t s) {
-    const size_t smem = (size_t)chunk * sizeof(float2);
-    GL_CUDA(cudaFuncSetAttribute(k_sgs_cluster<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    GL_CUDA(cudaFuncSetAttribute(k_sgs_cluster<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(size);
-    cfg.blockDim = dim3(CLUSTER_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = size;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    GL_CUDA(cudaLaunchKernelEx(&cfg, k_sgs_cluster<G>, A.view(), diag, cstart, nc, b, x, zero_start, chunk,
-                               1.0f / (float)chunk, stop));
-}
-
 // dispatch on the group width
 #define GL_DISPATCH_G(G_, CALL)                       \
     switch (G_) {                                     \
@@ -1113,10 +368,8 @@ void autotune_levels(gl_prec_s *p, bool fp32, cudaStream_t s) {
     for (int l = 0; l + 1 < p->nlev; ++l) {
         Level &L = p->L[l], &Lc = p->L[l + 1];
         if (fp32) {
-            if (l > 0) tune_groups<float2>(L.Ag32, L.x32.get(), L.r32.get(), s);
             tune_groups<float2>(L.PHg32, L.r32.get(), Lc.b32.get(), s);
         } else {
-            if (l > 0) tune_groups<double2>(L.Ag, L.x.get(), L.r.get(), s);
             tune_groups<double2>(L.PHg, L.r.get(), Lc.b.get(), s);
         }
     }
@@ -1348,60 +601,14 @@ static bool lattice_for(const gl_prec_s *p, LatticeView &v) {
     return false;
 }
 
-// pre- or post-smoothing on level l: per-colour launches on the lattice level
-// (two colours, large sweeps), one cooperative launch on coarse levels
+// pre- or post-smoothing on the finest level: per-colour launches (two colours,
+// large sweeps, on a lattice)
 template <typename T>
-static void smooth(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typename LevelOps<T>::C *x, bool zero_start,
-                   const int *stop, cudaStream_t s) {
-    using O = LevelOps<T>;
-    using C = typename O::C;
-    Level &L = p->L[l];
-    if (l == 0) {
-        LatticeView lv;
-        bool lat = lattice_for<T>(p, lv);
-        sgs<T>(L, l, b, x, zero_start, stop, s, lat ? &lv : nullptr);
-        return;
-    }
-    const CsrG<C> &A = O::Ag(L);
-    int64_t maxc = 0;
-    for (int c = 0; c < L.ncolors; ++c) maxc = std::max(maxc, L.cstart[c + 1] - L.cstart[c]);
-    // algorithmic bytes of one symmetric step: every visit of a colour reads its
-    // rows' stored entries (value + column) and b, diagonal and writes x; the
-    // first colour from a zero guess reads no entries
-    double bytes = 0, flops = 0;
-    for (int ph = 0; ph < 2 * L.ncolors - 1; ++ph) {
-        int c = ph < L.ncolors ? ph : 2 * L.ncolors - 2 - ph;
-        double rows = (double)(L.cstart[c + 1] - L.cstart[c]);
-        bytes += rows * (2 * sizeof(C) + sizeof(T));
-        flops += 6.0 * rows;
-        if (!(zero_start && ph == 0)) {
-            bytes += (double)L.cnnz[c] * (sizeof(C) + 4);
-            flops += 8.0 * (double)L.cnnz[c];
-        }
-    }
-    ProfScope ps("gs", bytes, s, flops);
-    const int sG = sizeof(T) == 4 ? L.sgs_G32 : L.sgs_G64;
-    if constexpr (sizeof(T) == 4) {
-        if (L.cl_size > 0 && p->cluster_sweeps) {
-            GL_DISPATCH_G(sG, (launch_sgs_cluster<GG>(A, O::diag(L), L.cstart_dev.get(), L.ncolors, b, x,
-                                                       zero_start ? 1 : 0, L.cl_size, L.cl_chunk, stop, s)));
-            return;
-        }
-    }
-    // the status word of the solve this sweep belongs to: a wait that runs out writes it
-    int *status = const_cast<int *>(stop);
-    const int sync = sizeof(T) == 4 ? L.sync32 : L.sync64;
-    if (sync == 1) {
-        const FlagPlan &F = sizeof(T) == 4 ? L.fl32 : L.fl64;
-        unsigned long long *flags = L.flags.get() + (sizeof(T) == 4 ? 0 : (size_t)MAX_FLAG_CTAS * FLAG_STRIDE);
-        GL_DISPATCH_G(sG, (launch_sgs_flags<GG, C, T>(A, O::diag(L), L.cstart_dev.get(), L.ncolors, F, b, x,
-                                                       zero_start ? 1 : 0, flags, p->wait_extra.get(), p->err.get(),
-                                                       status, s)));
-        return;
-    }
-    GL_DISPATCH_G(sG, (launch_sgs_coop<GG, C, T>(A, O::diag(L), L.cstart_dev.get(), L.ncolors, b, x,
-                                                  zero_start ? 1 : 0, L.barrier.get(), p->wait_extra.get(),
-                                                  p->err.get(), status, maxc, s)));
+static void smooth_finest(gl_prec_s *p, const typename LevelOps<T>::C *b, typename LevelOps<T>::C *x, bool zero_start,
+                          const int *stop, cudaStream_t s) {
+    LatticeView lv;
+    const bool lat = lattice_for<T>(p, lv);
+    sgs<T>(p->L[0], 0, b, x, zero_start, stop, s, lat ? &lv : nullptr);
 }
 
 template <typename T>
@@ -1415,10 +622,12 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         return;
     }
     Level &Lc = p->L[l + 1];
-    smooth<T>(p, l, b, x, true, stop, s);
     C *r = O::r(L);
     bool restrict_black = false;
-    if (l == 0) {
+    if (l > 0) {
+        sweep_step<T>(p, l, b, x, true, r, nullptr, stop, s);  // and the residual
+    } else {
+        smooth_finest<T>(p, b, x, true, stop, s);
         const T *scale;
         if constexpr (sizeof(T) == 8)
             scale = p->mesh->volp.get();
@@ -1441,11 +650,6 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         if (!lat)
             k_resid<C, T><<<grid_for(L.n, 256), 256, 0, s>>>(L.n, O::A(L).view(), O::diag(L), b, x, scale, r, stop);
         restrict_black = lat && sizeof(T) == 4 && L.PHg32b.nrows > 0;
-    } else {
-        const CsrG<C> &A = O::Ag(L);
-        ProfScope ps("resid", 0, s);
-        GL_DISPATCH_G(A.G, (k_resid_g<GG, C, T><<<grid_for(L.n * GG, 256), 256, 0, s>>>(A.view(), O::diag(L), b, x,
-                                                                                        r, stop)));
     }
     {
         ProfScope ps("restrict", 0, s);
@@ -1469,7 +673,10 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         ProfScope ps("prolong", 0, s);
         k_spmv<C><<<grid_for(L.n - lo, 256), 256, 0, s>>>(lo, L.n, O::P(L).view(), O::x(Lc), x, 1, stop);
     }
-    smooth<T>(p, l, b, x, false, stop, s);
+    if (l > 0)
+        sweep_step<T>(p, l, b, x, false, nullptr, nullptr, stop, s);
+    else
+        smooth_finest<T>(p, b, x, false, stop, s);
     GL_LAUNCH_CHECK();
 }
 
@@ -1695,236 +902,6 @@ void precond_apply_p64_via32(gl_prec_s *p, const double2 *v, double2 *z, const i
     precond_apply_t<float>(p, p->mp_in.get(), p->mp_out.get(), stop, s);
     k_f2d<<<grid_for(n, 256), 256, 0, s>>>(n, p->mp_out.get(), z, stop);
     GL_LAUNCH_CHECK();
-}
-
-// CTAs of a neighbour-flag sweep by default: about 3/4 of a round of rows per
-// CTA in the largest colour (the node-range partition spreads a colour unevenly)
-template <typename T>
-static int flags_default_nb(const Level &L, int G, int max_ctas) {
-    int64_t maxc = 0;
-    for (int c = 0; c < L.ncolors; ++c) maxc = std::max(maxc, L.cstart[c + 1] - L.cstart[c]);
-    // rows per round of the flag sweep (its warp 0 only synchronises), three quarters full
-    const int64_t per = std::max<int64_t>(1, (int64_t)((coop_threads<T>() - 32) / G) * 3 / 4);
-    return (int)std::min<int64_t>(std::max<int64_t>((maxc + per - 1) / per, 1), max_ctas);
-}
-
-template <typename T>
-static int flags_max_ctas_g(int G) {
-    using C = typename LevelOps<T>::C;
-    int r = 0;
-    GL_DISPATCH_G(G, (r = flags_max_ctas<GG, C, T>()));
-    return r;
-}
-
-static void zero_flags(Level &L, bool fp32, cudaStream_t s) {
-    const size_t words = (size_t)MAX_FLAG_CTAS * FLAG_STRIDE;
-    GL_CUDA(cudaMemsetAsync(L.flags.get() + (fp32 ? 0 : words), 0, words * sizeof(unsigned long long), s));
-}
-
-// chooses how every coarse level runs its symmetric Gauss-Seidel steps: the
-// lanes-per-row width G (a latency-bound kernel wants more lanes per row than
-// the throughput-bound SpMV that set the operator's own G), the synchronisation
-// between colours (grid barrier, or neighbour flags with nb CTAs) and, in FP32,
-// the thread-block-cluster sweep for levels whose vector fits a cluster.  With
-// autotuning every candidate (G = 2, 4, 8, 16; the flags with CTAs in
-// proportion to the level's largest colour) is timed on this GPU (best of two after
-// a warm-up launch, on zero vectors) and the fastest kept; without it the
-// operator's G, the flags where their partition fits (else the grid barrier),
-// and the cluster sweep wherever it fits.  options.sweep_sync = 1 or 2 keeps
-// only the grid-barrier or only the flag candidates (the flags fall back to the
-// barrier where no partition fits).  All of them give the same rows for the
-// same G.
-template <typename T>
-static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
-    using O = LevelOps<T>;
-    using C = typename O::C;
-    constexpr bool fp32 = sizeof(T) == 4;
-    cudaEvent_t e0, e1;
-    GL_CUDA(cudaEventCreate(&e0));
-    GL_CUDA(cudaEventCreate(&e1));
-    const bool try_grid = p->sweep_sync != 2, try_flags = p->sweep_sync != 1;
-    for (int l = 1; l < p->nlev - 1; ++l) {
-        Level &L = p->L[l];
-        const CsrG<C> &A = O::Ag(L);
-        int &sG = fp32 ? L.sgs_G32 : L.sgs_G64;
-        int &sync = fp32 ? L.sync32 : L.sync64;
-        FlagPlan &F = fp32 ? L.fl32 : L.fl64;
-        sG = A.G;
-        sync = 0;
-        F = FlagPlan{};
-        if constexpr (fp32) {
-            L.cl_size = 0;
-            L.cl_chunk = 0;
-        }
-        int size = 0, chunk = 0;
-        if constexpr (fp32) {
-            if (p->cluster_sweeps && p->sweep_sync == 0 && L.n <= INT32_MAX)
-                GL_DISPATCH_G(A.G, (plan_sgs_cluster<GG>(L.n, size, chunk)));
-        }
-        if (!p->autotune) {
-            if (try_flags) {
-                const int nb = flags_default_nb<T>(L, sG, flags_max_ctas_g<T>(sG));
-                if (build_flag_plan<C>(L, A, sG, nb, F, s) <= FLAG_MAXN)
-                    sync = 1;
-                else
-                    F = FlagPlan{};
-            }
-            if constexpr (fp32) {
-                L.cl_size = size;
-                L.cl_chunk = chunk;
-            }
-            zero_flags(L, fp32, s);
-            continue;
-        }
-        int64_t maxc = 0;
-        for (int c = 0; c < L.ncolors; ++c) maxc = std::max(maxc, L.cstart[c + 1] - L.cstart[c]);
-        C *b = O::b(L), *x = O::x(L);
-        GL_CUDA(cudaMemsetAsync(b, 0, L.n * sizeof(C), s));
-        GL_CUDA(cudaMemsetAsync(x, 0, L.n * sizeof(C), s));
-        auto time_it = [&](auto &&launch) {
-            float best = 1e30f;
-            for (int rep = 0; rep < 3; ++rep) {
-                GL_CUDA(cudaEventRecord(e0, s));
-                launch();
-                GL_CUDA(cudaEventRecord(e1, s));
-                GL_CUDA(cudaEventSynchronize(e1));
-                float ms = 0;
-                GL_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-                if (rep > 0) best = std::min(best, ms);
-            }
-            return best;
-        };
-        float best = 1e30f;
-        int bestG = A.G, best_sync = 0, best_nb = 0;
-        bool best_cluster = false;
-        unsigned long long *flags = L.flags.get() + (fp32 ? 0 : (size_t)MAX_FLAG_CTAS * FLAG_STRIDE);
-        for (int g : {2, 4, 8, 16}) {
-            if (try_grid) {
-                // a new grid size on this level's barrier counter: start it from zero
-                GL_CUDA(cudaMemsetAsync(L.barrier.get(), 0, GRID_BARRIER_WORDS * sizeof(unsigned), s));
-                float t = time_it([&] {
-                    GL_DISPATCH_G(g, (launch_sgs_coop<GG, C, T>(A, O::diag(L), L.cstart_dev.get(), L.ncolors, b, x,
-                                                                 0, L.barrier.get(), p->wait_extra.get(),
-                                                                 p->err.get(), nullptr, maxc, s)));
-                });
-                if (t < best) best = t, bestG = g, best_sync = 0, best_cluster = false;
-                if (verbose()) fprintf(stderr, "gl: level %d (n %lld, %d colours, %s) sweep G %d grid: %.1f us\n", l,
-                                       (long long)L.n, L.ncolors, fp32 ? "FP32" : "FP64", g, 1e3 * t);
-            }
-            if (try_flags) {
-                // CTAs in proportion to the level (never the whole GPU for a small
-                // level: in a batch, instances' sweeps run side by side)
-                const int nb0 = flags_default_nb<T>(L, g, flags_max_ctas_g<T>(g));
-                for (int nb : {nb0}) {
-                    FlagPlan cand;
-                    const int longest = build_flag_plan<C>(L, A, g, nb, cand, s);
-                    if (longest > FLAG_MAXN) {
-                        if (verbose()) fprintf(stderr, "gl: level %d flags G %d nb %d: %d neighbours, too many\n", l,
-                                               g, nb, longest);
-                        continue;
-                    }
-                    zero_flags(L, fp32, s);
-                    float t = time_it([&] {
-                        GL_DISPATCH_G(g, (launch_sgs_flags<GG, C, T>(A, O::diag(L), L.cstart_dev.get(), L.ncolors,
-                                                                      cand, b, x, 0, flags, p->wait_extra.get(),
-                                                                      p->err.get(), nullptr, s)));
-                    });
-                    if (verbose())
-                        fprintf(stderr, "gl: level %d sweep G %d flags nb %d (<= %d neighbours): %.1f us\n", l, g,
-                                nb, longest, 1e3 * t);
-                    if (t < best) {
-                        best = t, bestG = g, best_sync = 1, best_nb = nb, best_cluster = false;
-                        F = std::move(cand);
-                    }
-                }
-            }
-            if constexpr (fp32) {
-                if (size > 0) {
-                    float tc = time_it([&] {
-                        GL_DISPATCH_G(g, (launch_sgs_cluster<GG>(A, O::diag(L), L.cstart_dev.get(), L.ncolors, b, x, 0,
-                                                                  size, chunk, nullptr, s)));
-                    });
-                    if (tc < best) best = tc, bestG = g, best_cluster = true, best_sync = 0;
-                    if (verbose()) fprintf(stderr, "gl: level %d cluster sweep G %d: %.1f us\n", l, g, 1e3 * tc);
-                }
-            }
-        }
-        sG = bestG;
-        sync = best_sync;
-        if (sync != 1) F = FlagPlan{};
-        if (verbose())
-            fprintf(stderr, "gl: level %d %s sweep: G %d%s%s (largest colour %lld rows)\n", l, fp32 ? "FP32" : "FP64",
-                    bestG, best_cluster ? ", cluster" : "",
-                    best_sync == 1 ? (std::string(", flags nb ") + std::to_string(best_nb)).c_str() : "",
-                    (long long)maxc);
-        // the timing ran other launch shapes on this level's counters
-        GL_CUDA(cudaMemsetAsync(L.barrier.get(), 0, GRID_BARRIER_WORDS * sizeof(unsigned), s));
-        zero_flags(L, fp32, s);
-        GL_CUDA(cudaMemsetAsync(p->err.get(), 0, sizeof(int), s));
-        if constexpr (fp32) {
-            if (best_cluster) {
-                L.cl_size = size;
-                L.cl_chunk = chunk;
-            }
-        }
-    }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-}
-
-// the partitions of sweep choices taken over from a template (same sparsity)
-template <typename T>
-static void rebuild_flag_plans_t(gl_prec_s *p, const int *nbs, cudaStream_t s) {
-    using O = LevelOps<T>;
-    using C = typename O::C;
-    constexpr bool fp32 = sizeof(T) == 4;
-    for (int l = 1; l < p->nlev - 1; ++l) {
-        Level &L = p->L[l];
-        int &sync = fp32 ? L.sync32 : L.sync64;
-        FlagPlan &F = fp32 ? L.fl32 : L.fl64;
-        F = FlagPlan{};
-        if (sync == 1) {
-            const int G = fp32 ? L.sgs_G32 : L.sgs_G64;
-            if (nbs[l] < 1 || nbs[l] > flags_max_ctas_g<T>(G) || build_flag_plan<C>(L, O::Ag(L), G, nbs[l], F, s) > FLAG_MAXN) {
-                F = FlagPlan{};
-                sync = 0;
-            }
-        }
-        zero_flags(L, fp32, s);
-    }
-}
-
-void rebuild_flag_plans(gl_prec_s *p, bool fp32, cudaStream_t s) {
-    int nbs[MAX_LEVELS];
-    for (int l = 0; l < MAX_LEVELS; ++l) nbs[l] = fp32 ? p->tuned[l].nb32 : p->tuned[l].nb64;
-    if (fp32)
-        rebuild_flag_plans_t<float>(p, nbs, s);
-    else
-        rebuild_flag_plans_t<double>(p, nbs, s);
-}
-
-void sweeps_reset(gl_prec_s *p, cudaStream_t s) {
-    for (int l = 1; l < p->nlev - 1; ++l) {
-        Level &L = p->L[l];
-        if (L.barrier.get()) GL_CUDA(cudaMemsetAsync(L.barrier.get(), 0, GRID_BARRIER_WORDS * sizeof(unsigned), s));
-        if (L.flags.get()) GL_CUDA(cudaMemsetAsync(L.flags.get(), 0, L.flags.bytes(), s));
-    }
-    GL_CUDA(cudaMemsetAsync(p->err.get(), 0, sizeof(int), s));
-    GL_CUDA(cudaMemsetAsync(p->wait_extra.get(), 0, sizeof(unsigned long long), s));
-}
-
-int sweeps_failed(gl_prec_s *p, cudaStream_t s) {
-    int h = 0;
-    GL_CUDA(cudaMemcpyAsync(&h, p->err.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
-    GL_CUDA(cudaStreamSynchronize(s));
-    return h;
-}
-
-void plan_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s) {
-    if (fp32)
-        plan_sweeps_t<float>(p, s);
-    else
-        plan_sweeps_t<double>(p, s);
 }
 
 }  // namespace gl
