@@ -12,7 +12,7 @@
 //   * Galerkin A_c = P^H A P by a two-phase row-wise SpGEMM (hash symbolic pass,
 //     deterministic numeric pass), made exactly Hermitian as (A_c + A_c^H)/2
 //   * colours: red-black on the lattice level, Jones-Plassmann below
-//   * coarsest level: dense FP64 inverse by Gauss-Jordan elimination
+//   * coarsest level: dense FP64 inverse by the blocked Hermitian sweep operator
 #include <atomic>
 
 #include <chrono>
@@ -877,61 +877,194 @@ __global__ void k_to_dense(int64_t n, const int64_t *rp, const int32_t *ci, cons
     if (i >= n) return;
     for (int64_t q = rp[i]; q < rp[i + 1]; ++q) M[i * n + ci[q]] = v[q];
 }
-// the pivot row scaled by 1 / pivot and the pivot column, as they are before
-// step k (the pivot of an HPD matrix stays real positive; a non-positive one is
-// reported)
-__global__ void k_gj_snap(int64_t n, int64_t k, const double2 *M, double2 *rowk, double2 *colk, double *ipiv,
-                          int *err) {
-    const double piv = M[k * n + k].x;
-    const double ip = 1.0 / piv;
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t < n) {
-        const double2 r = M[k * n + t];
-        rowk[t] = make_double2(r.x * ip, r.y * ip);
-        colk[t] = M[t * n + k];
+// The inverse by the Hermitian sweep operator in blocks of INV_B rows: sweeping the
+// pivot block K maps M_KK -> -P with P = M_KK^-1, M_iK -> W_i = M_iK P and M_ij ->
+// M_ij - W_i M_jK^H; M stays Hermitian (only its lower triangle is kept and updated)
+// and is -A^-1 once every block has been swept.  M_KK is a Schur complement of A when
+// its turn comes, so its pivots are positive exactly if A is positive definite.
+//
+// The n^3 / 2 complex products are bound by this GPU's FP64 rate (1.06 TFLOP/s measured:
+// 76 ms at n = 2720), so shared memory and HBM have time to spare and small blocks cost
+// nothing: with 16 rows a step still computes for 0.45 ms on 60 MB, while the chain in
+// front of it (the inverse of one 16 x 16 block, which every CTA of the panel kernel
+// forms for itself, and a 16-column panel) stays short.  The update's 32 x 32 tiles
+// have eight warps of 2 x 2 entries a thread, so a small matrix's few tiles still keep
+// every sub-core's FP64 unit busy.  Measured at n = 2720 (128^3 cube): 322 ms as
+// n rank-one Gauss-Jordan steps over all n^2 entries, 83 ms now (0.92 of the FP64 rate);
+// n = 362 (1024^2 square): 4.0 and 1.2 ms.
+constexpr int INV_B = 16;     // rows of a pivot block
+constexpr int INV_T = 32;     // tile of the update
+constexpr int INV_UT = 256;   // its threads, 2 x 2 entries each
+
+// entry (i, j) of the Hermitian matrix whose lower triangle is stored
+__device__ __forceinline__ double2 inv_entry(const double2 *__restrict__ M, int64_t n, int64_t i, int64_t j) {
+    if (i >= j) return M[i * n + j];
+    const double2 v = M[j * n + i];
+    return make_double2(v.x, -v.y);
+}
+
+// P = M_KK^-1 for the rows [k0, k0 + INV_B) (every CTA; CTA 0 stores it) and, for the
+// CTA's INV_B rows i, U_i = M_iK and W_i = U_i P
+__global__ void __launch_bounds__(INV_B *INV_B) k_inv_panel(int64_t n, int64_t k0, const double2 *__restrict__ M,
+                                                           double2 *__restrict__ U, double2 *__restrict__ W,
+                                                           double2 *__restrict__ P, int *err) {
+    __shared__ double2 D[INV_B][INV_B + 1], S[INV_B][INV_B + 1];
+    const int r = threadIdx.x / INV_B, c = threadIdx.x % INV_B;
+    const int64_t i0 = (int64_t)blockIdx.x * INV_B;
+    {
+        const int64_t i = k0 + r, j = k0 + c;
+        D[r][c] = i < n && j < n ? inv_entry(M, n, i, j) : make_double2(r == c ? 1.0 : 0.0, 0.0);
     }
-    if (t == 0) {
-        *ipiv = ip;
-        if (!(piv > 0)) atomicExch(err, 1);
+    if (i0 >= k0) {
+        const int64_t i = i0 + r, j = k0 + c;
+        S[r][c] = i < n && j < n && i0 != k0 ? M[i * n + j] : make_double2(0.0, 0.0);
+    } else {  // the block's rows hold these entries: consecutive threads read along a row
+        const int64_t i = i0 + c, j = k0 + r;
+        const double2 v = j < n ? M[j * n + i] : make_double2(0.0, 0.0);
+        S[c][r] = make_double2(v.x, -v.y);
+    }
+    // Gauss-Jordan in place, one entry a thread; the next pivot's thread alone divides
+    // (a division by all eight warps would keep the FP64 pipe for most of a step)
+    __shared__ double ipiv;
+    if (threadIdx.x == 0) {
+        ipiv = 1.0 / D[0][0].x;
+        if (!(D[0][0].x > 0)) atomicExch(err, 1);
+    }
+    for (int p = 0; p < INV_B; ++p) {
+        __syncthreads();
+        const double ip = ipiv;
+        const double2 row = D[p][c], col = D[r][p];
+        double2 v = D[r][c];
+        if (r == p) {
+            v = c == p ? make_double2(ip, 0.0) : make_double2(row.x * ip, row.y * ip);
+        } else if (c == p) {
+            v = make_double2(-col.x * ip, -col.y * ip);
+        } else {
+            const double2 t = cmul(col, row);
+            v = make_double2(v.x - t.x * ip, v.y - t.y * ip);
+        }
+        __syncthreads();
+        D[r][c] = v;
+        if (r == p + 1 && c == p + 1) {
+            ipiv = 1.0 / v.x;
+            if (!(v.x > 0)) atomicExch(err, 1);
+        }
+    }
+    __syncthreads();
+    if (blockIdx.x == 0) P[threadIdx.x] = D[r][c];
+    if (i0 + r < n) {
+        double2 w = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int k = 0; k < INV_B; ++k) cfma(w, S[r][k], D[k][c]);
+        U[i0 * INV_B + threadIdx.x] = S[r][c];
+        W[i0 * INV_B + threadIdx.x] = w;
     }
 }
-// one Gauss-Jordan step on pivot k (in-place inversion, no pivoting: A is HPD):
-// row i = blockIdx.y, columns blockIdx.x * blockDim.x + threadIdx.x; one complex
-// product per entry off the pivot row and column
-__global__ void __launch_bounds__(256) k_gj_step(int64_t n, int64_t k, double2 *M, const double2 *__restrict__ rowk,
-                                                 const double2 *__restrict__ colk, const double *__restrict__ ipiv) {
-    const int64_t i = blockIdx.y;
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int64_t t = i * n + j;
-    double2 r;
-    if (i == k) {
-        r = (j == k) ? make_double2(*ipiv, 0.0) : rowk[j];
-    } else if (j == k) {
-        const double ip = *ipiv;
-        r = make_double2(-colk[i].x * ip, -colk[i].y * ip);
-    } else {
-        const double2 cr = cmul(colk[i], rowk[j]);
-        r = make_double2(M[t].x - cr.x, M[t].y - cr.y);
+
+// the swept lower triangle, one tile a CTA: M_ij - W_i U_j^H outside the pivot block's
+// rows and columns, W and -P in them
+__global__ void __launch_bounds__(INV_UT) k_inv_update(int64_t n, int64_t k0, double2 *__restrict__ M,
+                                                   const double2 *__restrict__ U, const double2 *__restrict__ W,
+                                                   const double2 *__restrict__ P) {
+    __shared__ double2 sW[INV_B][INV_T + 1], sU[INV_B][INV_T + 1];
+    // tile (I, J), J <= I, from the CTA's number in the triangle
+    int I = (int)((sqrt(8.0 * blockIdx.x + 1.0) - 1.0) * 0.5);
+    while ((I + 1) * (I + 2) / 2 <= (int)blockIdx.x) ++I;
+    while (I * (I + 1) / 2 > (int)blockIdx.x) --I;
+    const int J = (int)blockIdx.x - I * (I + 1) / 2;
+    const int64_t i0 = (int64_t)I * INV_T, j0 = (int64_t)J * INV_T;
+    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+    for (int t = threadIdx.x; t < INV_T * INV_B; t += INV_UT) {
+        const int r = t / INV_B, k = t % INV_B;
+        const double2 z = make_double2(0.0, 0.0);
+        sW[k][r] = i0 + r < n ? W[(i0 + r) * INV_B + k] : z;
+        sU[k][r] = j0 + r < n ? U[(j0 + r) * INV_B + k] : z;
     }
-    M[t] = r;
+    __syncthreads();
+    double2 acc[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) acc[a][b] = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int k = 0; k < INV_B; ++k) {
+        double2 w[2], u[2];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            w[a] = sW[k][ty + 16 * a];
+            u[a] = sU[k][tx + 16 * a];
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {  // acc += w conj(u)
+                acc[a][b].x = fma(w[a].x, u[b].x, acc[a][b].x);
+                acc[a][b].x = fma(w[a].y, u[b].y, acc[a][b].x);
+                acc[a][b].y = fma(w[a].y, u[b].x, acc[a][b].y);
+                acc[a][b].y = fma(-w[a].x, u[b].y, acc[a][b].y);
+            }
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int64_t i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+            if (i >= n || j > i) continue;
+            const bool ik = i >= k0 && i < k0 + INV_B, jk = j >= k0 && j < k0 + INV_B;
+            double2 v;
+            if (ik && jk) {
+                v = P[(i - k0) * INV_B + (j - k0)];
+                v = make_double2(-v.x, -v.y);
+            } else if (jk) {
+                v = W[i * INV_B + (j - k0)];
+            } else if (ik) {
+                v = W[j * INV_B + (i - k0)];
+                v.y = -v.y;
+            } else {
+                const double2 m = M[i * n + j];
+                v = make_double2(m.x - acc[a][b].x, m.y - acc[a][b].y);
+            }
+            M[i * n + j] = v;
+        }
+}
+
+// A^-1 = -M from the lower triangle into both
+__global__ void __launch_bounds__(256) k_inv_finish(int64_t n, double2 *__restrict__ M) {
+    __shared__ double2 T[INV_T][INV_T + 1];
+    if (blockIdx.y > blockIdx.x) return;
+    const int64_t i0 = (int64_t)blockIdx.x * INV_T, j0 = (int64_t)blockIdx.y * INV_T;
+    const int c = threadIdx.x % INV_T;
+    for (int r = threadIdx.x / INV_T; r < INV_T; r += 8) {
+        const int64_t i = i0 + r, j = j0 + c;
+        if (i < n && j <= i) {
+            const double2 v = M[i * n + j];
+            T[r][c] = make_double2(-v.x, i == j ? 0.0 : -v.y);
+            M[i * n + j] = T[r][c];
+        }
+    }
+    __syncthreads();
+    for (int r = threadIdx.x / INV_T; r < INV_T; r += 8) {  // row j0 + r of the upper triangle
+        const int64_t j = j0 + r, i = i0 + c;
+        if (i < n && j < i) M[j * n + i] = make_double2(T[c][r].x, -T[c][r].y);
+    }
 }
 
 static void dense_inverse(const CsrDev &A, DBuf<double2> &Ainv, cudaStream_t s) {
     int64_t n = A.n;
     GL_REQUIRE(n <= MAX_COARSE_DENSE, GL_ERR_CAPACITY, "coarsest level too large for the dense solve");
     Ainv.alloc(n * n);
-    DBuf<double2> rowk(n), colk(n);
-    DBuf<double> ipiv(1);
+    DBuf<double2> work((size_t)(2 * n + INV_B) * INV_B);
+    double2 *U = work.get(), *W = U + n * INV_B, *P = W + n * INV_B;
     DBuf<int> err(1);
     GL_CUDA(cudaMemsetAsync(err.get(), 0, sizeof(int), s));
     GL_CUDA(cudaMemsetAsync(Ainv.get(), 0, (size_t)n * n * sizeof(double2), s));
     k_to_dense<<<grid_for(n, 128), 128, 0, s>>>(n, A.rp.get(), A.ci.get(), A.v.get(), Ainv.get());
-    const dim3 step_grid((unsigned)((n + 255) / 256), (unsigned)n);
-    for (int64_t k = 0; k < n; ++k) {
-        k_gj_snap<<<grid_for(n, 256), 256, 0, s>>>(n, k, Ainv.get(), rowk.get(), colk.get(), ipiv.get(), err.get());
-        k_gj_step<<<step_grid, 256, 0, s>>>(n, k, Ainv.get(), rowk.get(), colk.get(), ipiv.get());
+    const unsigned T = (unsigned)((n + INV_T - 1) / INV_T);
+    for (int64_t k0 = 0; k0 < n; k0 += INV_B) {
+        k_inv_panel<<<(unsigned)((n + INV_B - 1) / INV_B), INV_B * INV_B, 0, s>>>(n, k0, Ainv.get(), U, W, P, err.get());
+        k_inv_update<<<T * (T + 1) / 2, INV_UT, 0, s>>>(n, k0, Ainv.get(), U, W, P);
     }
+    k_inv_finish<<<dim3(T, T), 256, 0, s>>>(n, Ainv.get());
     GL_LAUNCH_CHECK();
     int herr = 0;
     GL_CUDA(cudaMemcpyAsync(&herr, err.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
