@@ -278,14 +278,9 @@ GL_API gl_status gl_jacobian_apply(gl_mesh mesh, const void *psi_dev, const void
  * can fail or fragment it), and latency-critical loops (cudaMalloc/cudaFree may
  * synchronise the device).  The paper has no counterpart; this is an interface
  * convenience.
- * It allocates nothing: its working buffers live in one static device array of
- * GL_NOALLOC_MAX_NODES = 262144 nodes x 3 complex doubles (12 MiB) that every
- * GPU loading the library holds until exit.  Meshes with more nodes are rejected
- * with GL_ERR_CAPACITY.  All calls on a device share that array (it keeps the
- * last call's contents; nothing needs to start at zero), so calls whose work
- * overlaps on the GPU race.  The first call on each device looks up the array's
- * device address with that device current; that first call should come before
- * any stream capture.
+ * It allocates nothing and holds nothing: it runs the kernel of gl_jacobian_apply
+ * on the caller's vectors.  Meshes with more than GL_NOALLOC_MAX_NODES = 262144
+ * nodes are rejected with GL_ERR_CAPACITY.
  * Arguments and layouts as gl_jacobian_apply. */
 GL_API gl_status gl_jacobian_apply_noalloc(gl_mesh mesh, const void *psi_dev, const void *phi_dev, void *y_dev,
                                            void *stream);

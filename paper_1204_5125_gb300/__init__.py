@@ -372,7 +372,7 @@ def gl_jacobian_apply(mesh, psi, phi, y, precision=GL_FP64, stream=None):
 
 
 def gl_jacobian_apply_noalloc(mesh, psi, phi, y, stream=None):
-    """FP64 Jacobian apply that allocates no device memory (static scratch; see gl.h)."""
+    """FP64 Jacobian apply that allocates no device memory (the kernel of gl_jacobian_apply)."""
     _check(library().gl_jacobian_apply_noalloc(mesh, _ptr(psi), _ptr(phi), _ptr(y), _stream(stream)))
 
 

@@ -210,11 +210,7 @@ gl_status gl_residual(gl_mesh m, const void *psi, void *r, void *stream) {
     return guard([&] {
         GL_REQUIRE(m && psi && r, GL_ERR_ARG, "NULL argument");
         GL_REQUIRE(psi != r, GL_ERR_ARG, "psi and r must not alias");
-        cudaStream_t s = as_stream(stream);
-        ensure_tmp(m);
-        permute_in(m->n, m->perm.get(), (const double2 *)psi, m->t0.get(), s);
-        residual_p(m, m->t0.get(), m->t1.get(), s);
-        permute_out(m->n, m->perm.get(), m->t1.get(), (double2 *)r, s);
+        residual_nodes(m, (const double2 *)psi, (double2 *)r, as_stream(stream));
         return GL_OK;
     });
 }
@@ -227,6 +223,10 @@ gl_status gl_jacobian_apply(gl_mesh m, const void *psi, const void *phi, void *y
                        precision == GL_APPLY_FP64_TABLES,
                    GL_ERR_ARG, "unknown precision");
         cudaStream_t s = as_stream(stream);
+        if (precision == GL_FP64) {
+            jacobian_apply_nodes(m, (const double2 *)psi, (const double2 *)phi, (double2 *)y, s);
+            return GL_OK;
+        }
         ensure_tmp(m);
         permute_in(m->n, m->perm.get(), (const double2 *)psi, m->t0.get(), s);
         permute_in(m->n, m->perm.get(), (const double2 *)phi, m->t1.get(), s);
@@ -235,10 +235,8 @@ gl_status gl_jacobian_apply(gl_mesh m, const void *psi, const void *phi, void *y
         } else if (precision == GL_MIXED) {
             mesh_ensure_fp32(m, s);
             jacobian_apply_p32(m, m->t0.get(), m->t1.get(), m->t2.get(), s);
-        } else if (precision == GL_APPLY_FP64_TABLES) {
-            jacobian_apply_lat64_p(m, m->t0.get(), m->t1.get(), m->t2.get(), s);
         } else {
-            jacobian_apply_p(m, m->t0.get(), m->t1.get(), m->t2.get(), s);
+            jacobian_apply_lat64_p(m, m->t0.get(), m->t1.get(), m->t2.get(), s);
         }
         permute_out(m->n, m->perm.get(), m->t2.get(), (double2 *)y, s);
         return GL_OK;

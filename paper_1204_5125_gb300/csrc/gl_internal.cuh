@@ -27,6 +27,7 @@ struct gl_mesh_s {
     std::vector<int64_t> cstart0;
     gl::DBuf<int32_t> perm, iperm;
     gl::Sell<double2> K;                  // off-diagonals of K = D^-1 K-hat (solve ordering)
+    gl::DBuf<int32_t> kcoln;              // the same entries' columns as node numbers
     gl::DBuf<double> kdiag, volp;         // K_ii and |V_i| (solve ordering)
     bool has32 = false;
     gl::Sell<float2> K32;
@@ -298,7 +299,11 @@ void jacobian_apply_p32(const gl_mesh_s *m, const double2 *psi, const double2 *p
 // gl_solve.cu: the double-float lattice Jacobian of the GL_MIXED_PRECOND solve on
 // phi rounded to FP32 (solve ordering; GL_ERR_ARG without a lattice stencil)
 void jacobian_apply_pdf(gl_mesh_s *m, const double2 *psi, const double2 *phi, double2 *y, cudaStream_t s);
-void residual_p(const gl_mesh_s *m, const double2 *psi, double2 *r, cudaStream_t s);
+// the FP64 Jacobian and residual on node-order vectors (no reordering)
+void jacobian_apply_nodes(const gl_mesh_s *m, const double2 *psi, const double2 *phi, double2 *y, cudaStream_t s);
+void residual_nodes(const gl_mesh_s *m, const double2 *psi, double2 *r, cudaStream_t s);
+// fills m->kcoln once K is built
+void mesh_node_columns(gl_mesh_s *m, cudaStream_t s);
 // node order: r <- -r, returns ||r||_R (part: RED_BLOCKS doubles, scal: 1 double)
 double newton_rhs(const gl_mesh_s *m, double2 *r, double *part, double *scal, cudaStream_t s);
 void newton_update(int64_t n, const double2 *d, double2 *psi, cudaStream_t s);

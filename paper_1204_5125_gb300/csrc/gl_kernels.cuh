@@ -85,15 +85,16 @@ __device__ __forceinline__ C sell_row_before(const SellView<C> &A, int64_t p, co
     return acc;
 }
 
-// Jacobian row given the off-diagonal sum: acc + (K_ii - 1 + 2|psi|^2) phi + psi^2 conj(phi)
+// Jacobian row given the off-diagonal sum: acc + (K_ii - 1 + 2|psi|^2) phi + psi^2 conj(phi).
+// With s = Re(conj(psi) phi) the terms without K are psi (2 s) + |psi|^2 phi: eleven
+// operations instead of sixteen, in kernels that the FP64 pipe bounds.
 template <typename C, typename R>
 __device__ __forceinline__ C jacobian_epilogue(C acc, R kd, C ps, C ph) {
-    R a2 = ps.x * ps.x + ps.y * ps.y;
-    R d = kd - (R)1 + (R)2 * a2;
-    C p2 = mk(ps.x * ps.x - ps.y * ps.y, (R)2 * ps.x * ps.y);  // psi^2
+    const R d = kd - (R)1 + (ps.x * ps.x + ps.y * ps.y);
+    const R s2 = (R)2 * (ps.x * ph.x + ps.y * ph.y);
     C r;
-    r.x = acc.x + d * ph.x + (p2.x * ph.x + p2.y * ph.y);  // psi^2 conj(phi): (a+ib)(c-id)
-    r.y = acc.y + d * ph.y + (p2.y * ph.x - p2.x * ph.y);
+    r.x = acc.x + d * ph.x + s2 * ps.x;
+    r.y = acc.y + d * ph.y + s2 * ps.y;
     return r;
 }
 

@@ -728,6 +728,7 @@ void mesh_create(gl_mesh_s *m, int dim, int N, double edge, double mu, const dou
     // K = D^-1 K-hat, off-diagonals as sliced ELL in the solve ordering
     m->kdiag.alloc(n);
     build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s);
+    mesh_node_columns(m, s);
     m->volp.alloc(n);
     k_permute_real<<<grid_for(n, 256), 256, 0, s>>>(n, m->perm.get(), m->vol.get(), m->volp.get());
     GL_LAUNCH_CHECK();
@@ -1213,6 +1214,7 @@ void mesh_create_simplicial(gl_mesh_s *m, int dim, int64_t n, const double *xyz_
     // K = D^-1 K-hat, off-diagonals as sliced ELL in the solve ordering
     m->kdiag.alloc(n);
     build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s);
+    mesh_node_columns(m, s);
     m->volp.alloc(n);
     k_permute_real<<<grid_for(n, 256), 256, 0, s>>>(n, m->perm.get(), m->vol.get(), m->volp.get());
     GL_LAUNCH_CHECK();
