@@ -119,7 +119,7 @@ struct Level {
     DBuf<double> diag;              // level 0: K_ii + 2|psi_i|^2; else A_ii
     Sell<double2> P;                // permuted prolongator
     CsrG<double2> PHg;              // its adjoint, grouped CSR
-    SweepData<double2, double> sw64;  // coarse levels: the operator in the form of the sweeps
+    SweepData<double2, double> sw64;  // many-coloured levels: the operator in the form of the sweeps
     SweepData<float2, float> sw32;
     DBuf<int64_t> cstart_dev;       // cstart on the device (cooperative sweeps)
     DBuf<double2> b, x, r;          // level vectors (solve ordering)
@@ -157,6 +157,9 @@ struct gl_prec_s {
     gl::DBuf<unsigned long long> wait_extra;  // added to every sweep wait target: 0, or huge after
                                       // gl_precond_debug(GL_DEBUG_STALL_SWEEPS) (reset with the error word)
     int nlev = 0;
+    // level l's Gauss-Seidel steps are k_sweep launches (gl_sweep.cu): the levels between
+    // the finest and the coarsest, and a finest level with more than two colours
+    bool swept(int l) const { return l < nlev - 1 && (l > 0 || L[0].ncolors > 2); }
     int cycles = 1;
     bool has32 = false;
     bool autotune = true;
@@ -315,10 +318,11 @@ void precond_apply_p32(gl_prec_s *p, const float2 *v, float2 *z, const int *stop
 // autotuner: picks the lanes-per-row width of every grouped-CSR operator by timing
 void autotune_levels(gl_prec_s *p, bool fp32, cudaStream_t s);
 // gl_sweep.cu: the operator of a many-coloured level in the sweeps' form (and its
-// diagonal), in the solve ordering given by perm / iperm
+// diagonal), in the solve ordering given by perm / iperm, the rows divided by
+// row_scale (nullable)
 template <typename C>
-void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const CsrDev &A, SplitCsr<C> &out,
-                 double *diag_out, cudaStream_t s);
+void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const CsrDev &A, const double *row_scale,
+                 SplitCsr<C> &out, double *diag_out, cudaStream_t s);
 // one symmetric Gauss-Seidel step on level l, from x = 0 (zero_start) or from x;
 // r (nullable, zero_start only) receives the residual b - A x times scale (nullable)
 template <typename T>

@@ -1332,8 +1332,11 @@ void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_
         if (k == 0) {
             k_pdiag<<<grid_for(n, 256), 256, 0, s>>>(n, m->kdiag.get(), p->psi_p.get(), L.diag.get());
             GL_LAUNCH_CHECK();
-        } else if (!coarsest) {
-            build_split<double2>(L.n, L.perm, L.iperm, L.A_can, L.sw64.A, L.diag.get(), s);
+        }
+        if (p->swept(k)) {
+            // (the finest level's operator is the row-scaled one, whose diagonal is above)
+            build_split<double2>(L.n, L.perm, L.iperm, L.A_can, k == 0 ? m->vol.get() : nullptr, L.sw64.A,
+                                 k == 0 ? nullptr : L.diag.get(), s);
             L.cstart_dev.alloc(L.ncolors + 1);
             GL_CUDA(cudaMemcpyAsync(L.cstart_dev.get(), L.cstart.data(), (L.ncolors + 1) * sizeof(int64_t),
                                     cudaMemcpyHostToDevice, s));
@@ -1453,9 +1456,9 @@ void precond_ensure_fp32(gl_prec_s *p, cudaStream_t s) {
         to_float(L.diag.get(), L.diag32.get(), L.n, s);
         if (k == 0) {
             L.A32 = &m->K32;
-        } else if (!coarsest) {
-            build_split<float2>(L.n, L.perm, L.iperm, L.A_can, L.sw32.A, nullptr, s);
         }
+        if (p->swept(k))
+            build_split<float2>(L.n, L.perm, L.iperm, L.A_can, k == 0 ? m->vol.get() : nullptr, L.sw32.A, nullptr, s);
         if (!coarsest) {
             Level &Lc = p->L[k + 1];
             build_sell<float2>(L.n, Lc.n, L.perm, Lc.iperm, L.P_can, nullptr, false, L.P32, nullptr, s);

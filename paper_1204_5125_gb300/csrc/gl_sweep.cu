@@ -1,6 +1,8 @@
 // gl_sweep.cu -- the multicolour symmetric Gauss-Seidel steps of the V-cycle's
 // many-coloured levels (Sec. 4: one pre- and one post-step per level), each a
-// single launch, with the residual that follows the pre-step.
+// single launch, with the residual that follows the pre-step: the coarse levels,
+// and the finest level of a general simplicial mesh (on a lattice the finest level
+// is red-black: three large launches, gl_vcycle.cu).
 //
 // A level's operator is stored by rows with the entries of lower colours (solve
 // positions below the row's own) first and those of higher colours behind them.
@@ -37,6 +39,8 @@
 //   1024^2 square, FP32: level 1 (146,813 rows, 9 colours) 122 -> 59 us, level 2 (8,707
 //     rows, 10 colours) 123 -> 47 us
 //   64^2 square, level 1 (592 rows, 8 colours): FP64 198 -> 43 us, FP32 80 -> 29 us
+//   triangulation of 150^2 nodes, finest level (FP64; one launch per colour and a
+//     residual before): 101 -> 35 us
 // A phase takes 0.75 us on small levels (a store seen by another SM's poll takes 0.5 to
 // 0.75 us by itself) and 2.5 us on the 128^3 level, where the slowest of many
 // dependencies counts.  Carrying a tag beside every value instead of the empty slots
@@ -551,17 +555,18 @@ __global__ void k_split_len(int64_t nrows, const int32_t *perm, const int32_t *i
 }
 template <typename C>
 __global__ void k_split_fill(int64_t nrows, const int32_t *perm, const int32_t *iperm, const int64_t *rp,
-                             const int32_t *ci, const double2 *v, const int64_t *off, RowSplit *rows, int32_t *ocol,
-                             C *oval, double *diag_out) {
+                             const int32_t *ci, const double2 *v, const double *row_scale, const int64_t *off,
+                             RowSplit *rows, int32_t *ocol, C *oval, double *diag_out) {
     const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= nrows) return;
     const int64_t r = perm[p];
     int64_t lo = off[p], up = lo + rows[p].nl;
     rows[p].q0 = lo;
     double dg = 0;
+    const double sc = row_scale ? 1.0 / row_scale[r] : 1.0;
     for (int64_t q = rp[r]; q < rp[r + 1]; ++q) {
         const int32_t c = iperm[ci[q]];
-        const double2 a = v[q];
+        const double2 a = make_double2(v[q].x * sc, v[q].y * sc);
         if (c == p) {
             dg = a.x;
             continue;
@@ -577,8 +582,8 @@ __global__ void k_split_fill(int64_t nrows, const int32_t *perm, const int32_t *
 }
 
 template <typename C>
-void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const CsrDev &A, SplitCsr<C> &out,
-                 double *diag_out, cudaStream_t s) {
+void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const CsrDev &A, const double *row_scale,
+                 SplitCsr<C> &out, double *diag_out, cudaStream_t s) {
     out.nrows = n;
     out.nnz = A.nnz - n;  // every row stores its diagonal
     GL_REQUIRE(out.nnz < 0xffffffffll, GL_ERR_CAPACITY, "level operator has too many entries");
@@ -592,18 +597,19 @@ void build_split(int64_t n, const int32_t *perm, const int32_t *iperm, const Csr
     scan_exclusive(len.get(), len.get(), n, true, s);
     out.col.alloc(out.nnz > 0 ? out.nnz : 1);
     out.val.alloc(out.nnz > 0 ? out.nnz : 1);
-    k_split_fill<C><<<grid_for(n, 256), 256, 0, s>>>(n, perm, iperm, A.rp.get(), A.ci.get(), A.v.get(), len.get(),
-                                                     out.rows.get(), out.col.get(), out.val.get(), diag_out);
+    k_split_fill<C><<<grid_for(n, 256), 256, 0, s>>>(n, perm, iperm, A.rp.get(), A.ci.get(), A.v.get(), row_scale,
+                                                     len.get(), out.rows.get(), out.col.get(), out.val.get(),
+                                                     diag_out);
     GL_LAUNCH_CHECK();
     int herr = 0;
     GL_CUDA(cudaMemcpyAsync(&herr, err.get(), sizeof(int), cudaMemcpyDeviceToHost, s));
     GL_CUDA(cudaStreamSynchronize(s));
     GL_REQUIRE(herr == 0, GL_ERR_CAPACITY, "level operator row too long");
 }
-template void build_split<double2>(int64_t, const int32_t *, const int32_t *, const CsrDev &, SplitCsr<double2> &,
-                                   double *, cudaStream_t);
-template void build_split<float2>(int64_t, const int32_t *, const int32_t *, const CsrDev &, SplitCsr<float2> &,
-                                  double *, cudaStream_t);
+template void build_split<double2>(int64_t, const int32_t *, const int32_t *, const CsrDev &, const double *,
+                                   SplitCsr<double2> &, double *, cudaStream_t);
+template void build_split<float2>(int64_t, const int32_t *, const int32_t *, const CsrDev &, const double *,
+                                  SplitCsr<float2> &, double *, cudaStream_t);
 
 template <typename R>
 __global__ void k_inverse(int64_t n, const R *__restrict__ d, R *__restrict__ id) {
@@ -830,7 +836,8 @@ static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
         GL_CUDA(cudaEventCreate(&e0));
         GL_CUDA(cudaEventCreate(&e1));
     }
-    for (int l = 1; l < p->nlev - 1; ++l) {
+    for (int l = 0; l < p->nlev - 1; ++l) {
+        if (!p->swept(l)) continue;
         Level &L = p->L[l];
         auto &D = O::data(L);
         sweep_alloc<T>(L, s);
@@ -884,7 +891,8 @@ void plan_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s) {
 // the choices of a template preconditioner of the same sparsity
 template <typename T>
 static void adopt_sweeps_t(gl_prec_s *p, const int *lanes, const int *shifts, const int *sync, cudaStream_t s) {
-    for (int l = 1; l < p->nlev - 1; ++l) {
+    for (int l = 0; l < p->nlev - 1; ++l) {
+        if (!p->swept(l)) continue;
         Level &L = p->L[l];
         sweep_alloc<T>(L, s);
         sweep_shape<T>(L, sync[l], lanes[l], shifts[l], s);
@@ -904,7 +912,7 @@ void adopt_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s) {
 }
 
 void sweeps_reset(gl_prec_s *p, cudaStream_t s) {
-    for (int l = 1; l < p->nlev - 1; ++l) {
+    for (int l = 0; l < p->nlev - 1; ++l) {
         sweep_zero(p->L[l].sw32, s);
         sweep_zero(p->L[l].sw64, s);
     }

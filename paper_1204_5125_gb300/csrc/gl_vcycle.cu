@@ -624,15 +624,15 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
     Level &Lc = p->L[l + 1];
     C *r = O::r(L);
     bool restrict_black = false;
-    if (l > 0) {
-        sweep_step<T>(p, l, b, x, true, r, nullptr, stop, s);  // and the residual
+    const T *scale;  // of the residual handed to the restriction
+    if constexpr (sizeof(T) == 8)
+        scale = l == 0 ? p->mesh->volp.get() : nullptr;
+    else
+        scale = l == 0 ? p->mesh->volp32.get() : nullptr;
+    if (p->swept(l)) {
+        sweep_step<T>(p, l, b, x, true, r, scale, stop, s);  // and the residual
     } else {
         smooth_finest<T>(p, b, x, true, stop, s);
-        const T *scale;
-        if constexpr (sizeof(T) == 8)
-            scale = p->mesh->volp.get();
-        else
-            scale = p->mesh->volp32.get();
         ProfScope ps("resid0", 0, s);
         LatticeView lv;
         bool lat = lattice_for<T>(p, lv);
@@ -673,7 +673,7 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         ProfScope ps("prolong", 0, s);
         k_spmv<C><<<grid_for(L.n - lo, 256), 256, 0, s>>>(lo, L.n, O::P(L).view(), O::x(Lc), x, 1, stop);
     }
-    if (l > 0)
+    if (p->swept(l))
         sweep_step<T>(p, l, b, x, false, nullptr, nullptr, stop, s);
     else
         smooth_finest<T>(p, b, x, false, stop, s);

@@ -52,3 +52,30 @@ def test_dataflow_matches_grid_barrier(dim, N, max_coarse, precision):
         for p in P.values():
             gl.gl_precond_destroy(p)
         gl.gl_mesh_destroy(m)
+
+
+@pytest.mark.parametrize("precision", [gl.GL_FP64, gl.GL_MIXED_PRECOND], ids=["fp64", "fp32vc"])
+@pytest.mark.parametrize("domain,h", [("circ", 0.35), ("ball", 1.1)])
+def test_finest_level_of_a_triangulation(domain, h, precision):
+    """On a general mesh the finest level has many colours and takes the same sweeps,
+    with the residual scaled by the control volumes."""
+    pytest.importorskip("scipy")
+    dim, x, simplices = gi.delaunay_domain(domain, h)
+    m = gl.gl_mesh_create_simplicial(dim, x, simplices, 1.0)
+    n, _ = gl.gl_mesh_info(m)
+    psi, v = (torch.from_numpy(a).to(DEV) for a in (gi.disk(n, 46), gi.complex_normal(n, 47)))
+    z = []
+    try:
+        for sync in (1, 2):
+            P = gl.gl_precond_setup(m, psi, gl.options(max_coarse=64, sweep_sync=sync, autotune=0,
+                                                       precision=precision))
+            try:
+                assert gl.gl_precond_levels(P) >= 2
+                assert gl.gl_precond_level_sweep(P, 0, precision)["sync"] == sync - 1
+                z.append(torch.empty_like(v))
+                gl.gl_precond_apply_precision(P, v, z[-1], precision)
+            finally:
+                gl.gl_precond_destroy(P)
+        assert torch.equal(z[0], z[1])
+    finally:
+        gl.gl_mesh_destroy(m)
