@@ -154,7 +154,8 @@ __device__ __forceinline__ float2 lattice_row_f(const LatticeView &L, int64_t p,
 // sum_{k != p} K_pk x_k in FP64 from the FP64 tables (same layout, edge order and
 // conjugation as lattice_row_f), the row scaled by 1 / |V_p| = 2^b / h^d (b the
 // node's boundary coordinates; no division: this kernel is bound by the FP64 pipe)
-__device__ __forceinline__ double2 lattice_row64(const LatticeView64 &L, int64_t p, const double2 *__restrict__ x) {
+template <typename X>
+__device__ __forceinline__ double2 lattice_row64(const LatticeView64 &L, int64_t p, const X *__restrict__ x) {
     const uint32_t c = p >= L.nred ? 1u : 0u;
     const uint32_t N = (uint32_t)L.N;
     uint32_t v = 2u * (uint32_t)(p - (c ? L.nred : 0));
@@ -168,7 +169,8 @@ __device__ __forceinline__ double2 lattice_row64(const LatticeView64 &L, int64_t
     const int64_t other = c ? 0 : L.nred;
     double2 acc = make_double2(0.0, 0.0);
     auto edge = [&](double2 t, uint32_t u, bool plus) {
-        const double2 xv = x[(int64_t)(u >> 1) + other];
+        const X xs = x[(int64_t)(u >> 1) + other];
+        const double2 xv = make_double2(xs.x, xs.y);
         const double ty = plus ? t.y : -t.y;
         acc.x += t.x * xv.x - ty * xv.y;
         acc.y += t.x * xv.y + ty * xv.x;

@@ -29,7 +29,12 @@ struct MinresDev {
     double delta, a1, a2, a3, c_new, eta_prev, gamma_cur;
     double bnorm, tol, est, true_rel;
     double rho0;      // ||b - J x0||_D / ||b||_D: scales the recurrence's estimate to be relative to b
+    // factors of the vector kernels, formed once by the scalar steps (an FP64 division a
+    // thread kept the FP64 pipe for longer than a small vector's own work)
+    double ig, dg, go;        // v_new = ig q - dg v - go v_old
+    double sz, s3, s2, ce;    // w_new = sz z - s3 w_old - s2 w ; x += ce w_new
     int it, maxit, check_true, status, lucky, use_true, replays;
+    unsigned done;    // blocks of the current reduction that have written their partials
     double stall;     // > 0: stop with ST_STALL once the estimate is below stall * tol while the true
                       // residual is still above tol (0: never)
 };
@@ -58,12 +63,155 @@ __device__ __forceinline__ double redot(C a, C b) {  // Re(conj(a) b)
     return (double)a.x * (double)b.x + (double)a.y * (double)b.y;
 }
 
+// ------------------------------------------------------------------ scalar steps
+// A reduction writes one partial per block of its fixed grid; the block that finishes
+// last sums the partials in index order and takes the scalar step that follows, so a
+// reduction and its scalars are one launch (a one-block kernel behind each reduction
+// took 4 to 6 us, as long as a small system's vector kernels).
+__device__ double sum_parts(const double *part, double *sh) {
+    double a = 0;
+    for (int i = threadIdx.x; i < RED_BLOCKS; i += blockDim.x) a += __ldcg(part + i);
+    return block_sum(a, sh);
+}
+// true in every thread of the last block to get here (its partials are written)
+__device__ bool last_block(MinresDev *S) {
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&S->done, 1u) == gridDim.x - 1;
+        if (last) S->done = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return last;
+}
+
+// Conditional-node handles of the device-side MINRES loop (all unused when n = 0):
+// h[0] the WHILE node around a body of ITER_UNROLL iterations, h[k] (k >= 1) the
+// IF node around iteration k of the body.
+struct Gates {
+    cudaGraphConditionalHandle h[6];
+    int n;
+};
+
+// after iteration k of a loop body: the IF nodes of the body's later iterations
+// open only while the solve runs; every gate this iteration can reach is
+// written, so no value is left from an earlier body
+__device__ void set_gates(MinresDev *S, const Gates &g, int k) {
+    const unsigned run = S->status == ST_RUN ? 1u : 0u;
+    for (int j = k + 1; j < g.n; ++j) cudaGraphSetConditional(g.h[j], run);
+}
+
+// bb = <b, b>_R, vv = ||b - J x0||_D^2
+__device__ void scal_init(MinresDev *S, double bb, double vv) {
+    double tol = S->tol;
+    int use_true = S->use_true;
+    S->it = 0;
+    S->replays = 0;
+    S->status = ST_RUN;
+    S->check_true = 0;
+    S->lucky = 0;
+    S->bnorm = sqrt(bb);
+    S->true_rel = (S->bnorm > 0) ? sqrt(vv) / S->bnorm : 0.0;
+    // the tolerance is relative to b, the recurrence's estimate to r0 = b - J x0:
+    // scaled by ||r0||_D / ||b||_D (exactly 1 from x0 = 0)
+    S->rho0 = S->true_rel;
+    S->est = 1.0;
+    if (!(S->bnorm > 0)) {
+        S->status = ST_CONV;
+        S->est = 0;
+    } else if (use_true && S->true_rel <= tol) {
+        S->status = ST_CONV;
+    } else if (!isfinite(S->true_rel)) {
+        S->status = ST_NAN;
+    } else if (S->maxit <= 0) {
+        S->status = ST_MAXIT;
+    }
+}
+// g2 = <v_1, z_1>_R
+__device__ void scal_gamma0(MinresDev *S, double g2) {
+    if (!isfinite(g2)) {
+        S->status = ST_NAN;
+        return;
+    }
+    if (g2 < 0) {
+        S->status = ST_BREAK;
+        return;
+    }
+    double g = sqrt(g2);
+    S->gamma = g;
+    S->gamma_old = 1.0;
+    S->eta = S->eta0 = g;
+    S->c = S->c_old = 1.0;
+    S->s = S->s_old = 0.0;
+    if (g == 0) S->status = ST_CONV;
+}
+// d = <J z, z>_R
+__device__ void scal_delta(MinresDev *S, double d) {
+    S->delta = d / (S->gamma * S->gamma);
+    S->ig = 1.0 / S->gamma;
+    S->dg = S->delta / S->gamma;
+    S->go = S->gamma / S->gamma_old;
+}
+// g2 = <v_new, z_new>_R
+__device__ void scal_givens(MinresDev *S, double g2) {
+    if (!isfinite(g2) || !isfinite(S->delta)) {
+        S->status = ST_NAN;
+        return;
+    }
+    if (g2 < 0) {
+        S->status = ST_BREAK;
+        return;
+    }
+    double gn = sqrt(g2);
+    double g = S->gamma, d = S->delta;
+    double a0 = S->c * d - S->c_old * S->s * g;
+    double a1 = sqrt(a0 * a0 + gn * gn);
+    double a2 = S->s * d + S->c_old * S->c * g;
+    double a3 = S->s_old * g;
+    double cn = a0 / a1, sn = gn / a1;
+    const double ia1 = 1.0 / a1;
+    S->sz = ia1 / g;
+    S->s3 = a3 * ia1;
+    S->s2 = a2 * ia1;
+    S->ce = cn * S->eta;
+    S->eta = -sn * S->eta;
+    S->gamma_old = g;
+    S->gamma = gn;
+    S->c_old = S->c;
+    S->c = cn;
+    S->s_old = S->s;
+    S->s = sn;
+    S->it += 1;
+    S->est = S->rho0 * fabs(S->eta) / S->eta0;
+    S->lucky = (gn == 0);
+    S->check_true = (S->est <= S->tol) || S->lucky;
+}
+// the end of an iteration; r2 = ||b - J x||_D^2 when a check was asked for
+__device__ void scal_true(MinresDev *S, double r2) {
+    if (S->check_true) {
+        if (S->use_true) {
+            S->true_rel = sqrt(r2) / S->bnorm;
+            if (!isfinite(S->true_rel))
+                S->status = ST_NAN;
+            else if (S->true_rel <= S->tol)
+                S->status = ST_CONV;
+            else if (S->stall > 0 && S->est <= S->stall * S->tol)
+                S->status = ST_STALL;  // the recurrence has run far past what the true residual shows
+        } else {
+            S->status = ST_CONV;  // inner solves stop on the estimate alone
+        }
+        if (!S->status && S->lucky) S->status = ST_MAXIT;  // Krylov space exhausted above tol
+    }
+    if (!S->status && S->it >= S->maxit) S->status = ST_MAXIT;
+}
+
 // ------------------------------------------------------------------ vector kernels
-// v = b - J x ; partials of <b, b>_R and <v, v>_R
+// v = b - J x ; <b, b>_R and <v, v>_R
 template <typename C, typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_init_resid(int64_t n, SellView<C> K, const R *kd, const R *vol,
                                                             const C *psi, const C *b, const C *x, C *v,
-                                                            double *part) {
+                                                            double *part, MinresDev *S) {
     __shared__ double sh[32];
     double ab = 0, av = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
@@ -81,55 +229,92 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_resid(int64_t n, SellView<
         part[blockIdx.x] = t;
         part[RED_BLOCKS + blockIdx.x] = u;
     }
+    if (!last_block(S)) return;
+    const double bb = sum_parts(part, sh), vv = sum_parts(part + RED_BLOCKS, sh);
+    if (threadIdx.x == 0) scal_init(S, bb, vv);
 }
 
-// partials of <x, y>_R
-template <typename C, typename R>
-__global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t n, const R *vol, const C *x, const C *y, double *part,
-                                                     const int *stop) {
+// <x, y>_R and the scalar step behind it (0: gamma_1, 1: Givens); y may be the FP32
+// vector of a mixed-precision solve, whose FP64 image it stands for
+template <typename C, typename R, typename Y>
+__global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t n, const R *vol, const C *x, const Y *y, double *part,
+                                                     MinresDev *S, int givens) {
     __shared__ double sh[32];
-    if (*stop) return;
+    if (S->status) return;
     double a = 0;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-        a += (double)vol[p] * redot(x[p], y[p]);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto term = [](R w, C u, Y v) { return (double)w * ((double)u.x * (double)v.x + (double)u.y * (double)v.y); };
+    // four rows per step, every load issued before the first use
+    for (; p + 3 * stride < n; p += 4 * stride) {
+        C u[4];
+        Y v[4];
+        R w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            u[k] = x[p + k * stride];
+            v[k] = y[p + k * stride];
+            w[k] = vol[p + k * stride];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a += term(w[k], u[k], v[k]);
+    }
+    for (; p < n; p += stride) a += term(vol[p], x[p], y[p]);
     double t = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
+    if (!last_block(S)) return;
+    const double g2 = sum_parts(part, sh);
+    if (threadIdx.x) return;
+    if (givens)
+        scal_givens(S, g2);
+    else
+        scal_gamma0(S, g2);
 }
 
-// q = J z (z not yet normalised) ; partials of <J z, z>_R
-template <typename C, typename R>
+// q = J z (z not yet normalised) ; <J z, z>_R and delta.  Z: float2 when z is the FP32
+// V-cycle's output in a mixed-precision solve.
+template <typename C, typename R, typename Z>
 __global__ void __launch_bounds__(RED_THREADS) k_jz(int64_t n, SellView<C> K, const R *kd, const R *vol, const C *psi,
-                                                    const C *z, C *q, double *part, const int *stop) {
+                                                    const Z *z, C *q, double *part, MinresDev *S) {
     __shared__ double sh[32];
-    if (*stop) return;
+    if (S->status) return;
     double a = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        C acc = sell_row<C, C>(K, p, z);
-        C zz = z[p];
+        C acc = sell_row<C, Z>(K, p, z);
+        const Z zp = z[p];
+        C zz = mk((R)zp.x, (R)zp.y);
         C jz = jacobian_epilogue(acc, kd[p], psi[p], zz);
         q[p] = jz;
         a += (double)vol[p] * redot(jz, zz);
     }
     double t = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
+    if (!last_block(S)) return;
+    const double d = sum_parts(part, sh);
+    if (threadIdx.x == 0) scal_delta(S, d);
 }
 
 // the same from the FP64 lattice tables (the matrix-free stencil of a lattice mesh)
+template <typename Z>
 __global__ void __launch_bounds__(RED_THREADS) k_jz_lat64(int64_t n, LatticeView64 L, const double *kd,
-                                                          const double2 *psi, const double2 *z, double2 *q,
-                                                          double *part, const int *stop) {
+                                                          const double2 *psi, const Z *z, double2 *q,
+                                                          double *part, MinresDev *S) {
     __shared__ double sh[32];
-    if (*stop) return;
+    if (S->status) return;
     double a = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         const double2 acc = lattice_row64(L, p, z);
-        const double2 zz = z[p];
+        const Z zp = z[p];
+        const double2 zz = make_double2(zp.x, zp.y);
         const double2 jz = jacobian_epilogue(acc, kd[p], psi[p], zz);
         q[p] = jz;
         a += L.vol[p] * redot(jz, zz);
     }
     double t = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
+    if (!last_block(S)) return;
+    const double d = sum_parts(part, sh);
+    if (threadIdx.x == 0) scal_delta(S, d);
 }
 
 // ------------------------------------------------------------------ double-float Jacobian apply
@@ -146,7 +331,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_jz_lat64(int64_t n, LatticeView
 // accumulate in the compensated form of Ogita, Rump and Oishi's Dot2 (an FP32
 // running sum and an FP32 compensation collecting the exact rounding errors):
 // about 48 significant bits, against 53 in FP64.  The solve watches for the
-// consequence (see k_scal_true) and finishes with the FP64 apply if it stalls.
+// consequence (see scal_true) and finishes with the FP64 apply if it stalls.
 // per-solve coefficients of the local part: d = r - 1 + 2|psi|^2 and psi^2
 __global__ void k_jz_coef(int64_t n, const double *__restrict__ rem, const double2 *__restrict__ psi,
                           float2 *__restrict__ d, float4 *__restrict__ p2) {
@@ -158,13 +343,13 @@ __global__ void k_jz_coef(int64_t n, const double *__restrict__ rem, const doubl
     p2[i] = make_float4(re.x, re.y, im.x, im.y);
 }
 
-// q = J z from the exact FP32 copy z of the V-cycle output; partials of <J z, z>_R
+// q = J z from the FP32 V-cycle output z; <J z, z>_R and delta (S null: q alone)
 __global__ void __launch_bounds__(RED_THREADS) k_jz_latdf(int64_t n, LatticeDfView L, double hd,
                                                           const float2 *__restrict__ d, const float4 *__restrict__ p2,
                                                           const float2 *__restrict__ z, double2 *__restrict__ q,
-                                                          double *part, const int *stop) {
+                                                          double *part, MinresDev *S) {
     __shared__ double sh[32];
-    if (*stop) return;
+    if (S && S->status) return;
     float as = 0.f, ac = 0.f;
     const uint32_t N = (uint32_t)L.N;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
@@ -242,8 +427,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_jz_latdf(int64_t n, LatticeDfVi
         dot2_add(as, ac, ts * isb);
         ac = __fadd_rn(ac, tc * isb);
     }
+    if (!S) return;  // an apply outside a solve
     double t = block_sum(((double)as + (double)ac) * hd, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
+    if (!last_block(S)) return;
+    const double delta = sum_parts(part, sh);
+    if (threadIdx.x == 0) scal_delta(S, delta);
 }
 
 __global__ void k_round32(int64_t n, const double2 *a, float2 *b) {
@@ -261,28 +450,31 @@ void jacobian_apply_pdf(gl_mesh_s *m, const double2 *psi, const double2 *phi, do
     const int64_t n = m->n;
     DBuf<float2> d(n), z(n);
     DBuf<float4> p2(n);
-    DBuf<double> part(RED_BLOCKS);
-    DBuf<int> stop(1);
-    GL_CUDA(cudaMemsetAsync(stop.get(), 0, sizeof(int), s));
     const int G = grid_for(n, 256);
     note_launch(3);
     k_jz_coef<<<G, 256, 0, s>>>(n, m->lat_krem.get(), psi, d.get(), p2.get());
     k_round32<<<G, 256, 0, s>>>(n, phi, z.get());
     k_jz_latdf<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, lattice_df_view(m), m->lat_hd, d.get(), p2.get(), z.get(), y,
-                                                  part.get(), stop.get());
+                                                  nullptr, nullptr);
     GL_LAUNCH_CHECK();
     GL_CUDA(cudaStreamSynchronize(s));
 }
 
-// v_new = q / gamma - (delta / gamma) v - (gamma / gamma_old) v_old
-template <typename C, typename R>
-__global__ void k_vnew(int64_t n, const MinresDev *S, const C *q, const C *v, const C *v_old, C *v_new) {
+// v_new = q / gamma - (delta / gamma) v - (gamma / gamma_old) v_old; with v32 (the
+// mixed-precision form) also rounded to the FP32 V-cycle's input.  Four rows per step
+// with every load issued first.
+template <typename C, typename R, bool MP>
+__global__ void __launch_bounds__(RED_THREADS) k_vnew(int64_t n, const MinresDev *S, const C *q, const C *v,
+                                                      const C *v_old, C *v_new, float2 *v32) {
     if (S->status) return;
-    // the scalars once per thread (a fixed grid: FP64 divisions are costly here),
-    // four rows per step with every load issued first
-    R ig = (R)(1.0 / S->gamma), dg = (R)(S->delta / S->gamma), go = (R)(S->gamma / S->gamma_old);
+    const R ig = (R)S->ig, dg = (R)S->dg, go = (R)S->go;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    auto put = [&](int64_t i, C a, C b, C c) {
+        const C r = mk(a.x * ig - dg * b.x - go * c.x, a.y * ig - dg * b.y - go * c.y);
+        v_new[i] = r;
+        if (MP) v32[i] = make_float2((float)r.x, (float)r.y);
+    };
     for (; p + 3 * stride < n; p += 4 * stride) {
         C a[4], b[4], c[4];
 #pragma unroll
@@ -292,102 +484,29 @@ __global__ void k_vnew(int64_t n, const MinresDev *S, const C *q, const C *v, co
             c[u] = v_old[p + u * stride];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            v_new[p + u * stride] =
-                mk(a[u].x * ig - dg * b[u].x - go * c[u].x, a[u].y * ig - dg * b[u].y - go * c[u].y);
+        for (int u = 0; u < 4; ++u) put(p + u * stride, a[u], b[u], c[u]);
     }
-    for (; p < n; p += stride) {
-        C a = q[p], b = v[p], c = v_old[p];
-        v_new[p] = mk(a.x * ig - dg * b.x - go * c.x, a.y * ig - dg * b.y - go * c.y);
-    }
+    for (; p < n; p += stride) put(p, q[p], v[p], v_old[p]);
 }
 
-// the mixed-precision form's two passes around the FP32 V-cycle, each fused
-// with its neighbour: v_new of k_vnew also written as the V-cycle's FP32 input,
-// and the V-cycle's FP32 output widened to z_new inside the <v_new, z_new>_R dot
-__global__ void k_vnew_mp(int64_t n, const MinresDev *S, const double2 *q, const double2 *v, const double2 *v_old,
-                          double2 *v_new, float2 *v32) {
+// w_new = (z / gamma - a3 w_old - a2 w) / a1 ; x += c_new eta w_new, with the factors of
+// MinresDev (three FP64 operations per component; this stream is bound by GB300's FP64
+// pipe before HBM).  Z: float2 when z is the FP32 V-cycle's output.
+template <typename C, typename R, typename Z>
+__global__ void __launch_bounds__(RED_THREADS) k_update(int64_t n, const MinresDev *S, const Z *z, const C *w_old,
+                                                        const C *w, C *w_new, C *x) {
     if (S->status) return;
-    double ig = 1.0 / S->gamma, dg = S->delta / S->gamma, go = S->gamma / S->gamma_old;
+    const R sz = (R)S->sz, s3 = (R)S->s3, s2 = (R)S->s2, ce = (R)S->ce;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    for (; p + 3 * stride < n; p += 4 * stride) {
-        double2 a[4], b[4], c[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            a[u] = q[p + u * stride];
-            b[u] = v[p + u * stride];
-            c[u] = v_old[p + u * stride];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const double2 r =
-                make_double2(a[u].x * ig - dg * b[u].x - go * c[u].x, a[u].y * ig - dg * b[u].y - go * c[u].y);
-            v_new[p + u * stride] = r;
-            v32[p + u * stride] = to32(r);
-        }
-    }
-    for (; p < n; p += stride) {
-        double2 a = q[p], b = v[p], c = v_old[p];
-        double2 r = make_double2(a.x * ig - dg * b.x - go * c.x, a.y * ig - dg * b.y - go * c.y);
-        v_new[p] = r;
-        v32[p] = to32(r);
-    }
-}
-__global__ void __launch_bounds__(RED_THREADS) k_widen_dot(int64_t n, const double *vol, const double2 *v,
-                                                           const float2 *z32, double2 *z, double *part,
-                                                           const int *stop) {
-    __shared__ double sh[32];
-    if (*stop) return;
-    double a = 0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    // four rows per step, every load issued before the first use
-    for (; p + 3 * stride < n; p += 4 * stride) {
-        float2 zr[4];
-        double2 vv[4];
-        double vo[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            zr[u] = z32[p + u * stride];
-            vv[u] = v[p + u * stride];
-            vo[u] = vol[p + u * stride];
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const double2 zz = to64(zr[u]);
-            z[p + u * stride] = zz;
-            a += vo[u] * redot(vv[u], zz);
-        }
-    }
-    for (; p < n; p += stride) {
-        double2 zz = to64(z32[p]);
-        z[p] = zz;
-        a += vol[p] * redot(v[p], zz);
-    }
-    double t = block_sum(a, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-// w_new = (z / gamma - a3 w_old - a2 w) / a1 ; x += c_new eta w_new.  The
-// scalars are folded once per thread (z (1 / (gamma a1)) - (a3 / a1) w_old -
-// (a2 / a1) w): three FP64 operations per component instead of four, which
-// matters because this stream is bound by GB300's FP64 pipe, not by HBM.
-template <typename C, typename R>
-__global__ void k_update(int64_t n, const MinresDev *S, const C *z, const C *w_old, const C *w, C *w_new, C *x) {
-    if (S->status) return;
-    const double ia1 = 1.0 / S->a1;
-    const R sz = (R)(ia1 / S->gamma_cur), s3 = (R)(S->a3 * ia1), s2 = (R)(S->a2 * ia1);
-    const R ce = (R)(S->c_new * S->eta_prev);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    auto upd = [&](C zz, C wo, C ww, C xx, int64_t q) {
-        const C wn = mk(zz.x * sz - s3 * wo.x - s2 * ww.x, zz.y * sz - s3 * wo.y - s2 * ww.y);
+    auto upd = [&](Z zz, C wo, C ww, C xx, int64_t q) {
+        const C wn = mk((R)zz.x * sz - s3 * wo.x - s2 * ww.x, (R)zz.y * sz - s3 * wo.y - s2 * ww.y);
         w_new[q] = wn;
         x[q] = mk(xx.x + ce * wn.x, xx.y + ce * wn.y);
     };
     for (; p + 3 * stride < n; p += 4 * stride) {
-        C zz[4], wo[4], ww[4], xx[4];
+        Z zz[4];
+        C wo[4], ww[4], xx[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             zz[u] = z[p + u * stride];
@@ -401,13 +520,20 @@ __global__ void k_update(int64_t n, const MinresDev *S, const C *z, const C *w_o
     for (; p < n; p += stride) upd(z[p], w_old[p], w[p], x[p], p);
 }
 
-// partials of ||b - J x||_D^2, only when the scalar kernel asked for a check
+// ||b - J x||_D^2 when the Givens step asked for a check, and the end of iteration k of
+// a loop body; with `final` the true residual of the solve's result, whatever the status
 template <typename C, typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_true_resid(int64_t n, SellView<C> K, const R *kd, const R *vol,
                                                             const C *psi, const C *b, const C *x, double *part,
-                                                            const MinresDev *S, int force) {
+                                                            MinresDev *S, Gates g, int k, int final) {
     __shared__ double sh[32];
-    if (!force && (S->status || !S->check_true)) return;
+    if (!final && (S->status || !S->check_true)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (!S->status) scal_true(S, 0.0);
+            set_gates(S, g, k);
+        }
+        return;
+    }
     double a = 0;
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
         C acc = sell_row<C, C>(K, p, x);
@@ -417,43 +543,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_true_resid(int64_t n, SellView<
     }
     double t = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-// ------------------------------------------------------------------ scalar kernels (one block)
-__device__ double sum_parts(const double *part, double *sh) {
-    double a = 0;
-    for (int i = threadIdx.x; i < RED_BLOCKS; i += blockDim.x) a += part[i];
-    return block_sum(a, sh);
-}
-
-__global__ void k_scal_init(MinresDev *S, const double *part) {
-    __shared__ double sh[32];
-    double bb = sum_parts(part, sh);
-    double vv = sum_parts(part + RED_BLOCKS, sh);
+    if (!last_block(S)) return;
+    const double r2 = sum_parts(part, sh);
     if (threadIdx.x) return;
-    double tol = S->tol;
-    int use_true = S->use_true;
-    S->it = 0;
-    S->replays = 0;
-    S->status = ST_RUN;
-    S->check_true = 0;
-    S->lucky = 0;
-    S->bnorm = sqrt(bb);
-    S->true_rel = (S->bnorm > 0) ? sqrt(vv) / S->bnorm : 0.0;
-    // the tolerance is relative to b, the recurrence's estimate to r0 = b - J x0:
-    // scaled by ||r0||_D / ||b||_D (exactly 1 from x0 = 0)
-    S->rho0 = S->true_rel;
-    S->est = 1.0;
-    if (!(S->bnorm > 0)) {
-        S->status = ST_CONV;
-        S->est = 0;
-    } else if (use_true && S->true_rel <= tol) {
-        S->status = ST_CONV;
-    } else if (!isfinite(S->true_rel)) {
-        S->status = ST_NAN;
-    } else if (S->maxit <= 0) {
-        S->status = ST_MAXIT;
+    if (final) {
+        if (S->bnorm > 0) S->true_rel = sqrt(r2) / S->bnorm;
+        return;
     }
+    scal_true(S, r2);
+    set_gates(S, g, k);
 }
 
 // solve parameters, written before the captured init phase reads them
@@ -462,88 +560,7 @@ __global__ void k_set_params(MinresDev *S, double tol, int maxit, int use_true, 
     S->maxit = maxit;
     S->use_true = use_true;
     S->stall = stall;
-}
-
-__global__ void k_scal_gamma0(MinresDev *S, const double *part) {
-    __shared__ double sh[32];
-    double g2 = sum_parts(part, sh);
-    if (threadIdx.x || S->status) return;
-    if (!isfinite(g2)) {
-        S->status = ST_NAN;
-        return;
-    }
-    if (g2 < 0) {
-        S->status = ST_BREAK;
-        return;
-    }
-    double g = sqrt(g2);
-    S->gamma = g;
-    S->gamma_old = 1.0;
-    S->eta = S->eta0 = g;
-    S->c = S->c_old = 1.0;
-    S->s = S->s_old = 0.0;
-    if (g == 0) S->status = ST_CONV;
-}
-
-__global__ void k_scal_delta(MinresDev *S, const double *part) {
-    __shared__ double sh[32];
-    double d = sum_parts(part, sh);
-    if (threadIdx.x || S->status) return;
-    S->delta = d / (S->gamma * S->gamma);
-}
-
-__global__ void k_scal_givens(MinresDev *S, const double *part) {
-    __shared__ double sh[32];
-    double g2 = sum_parts(part, sh);
-    if (threadIdx.x || S->status) return;
-    if (!isfinite(g2) || !isfinite(S->delta)) {
-        S->status = ST_NAN;
-        return;
-    }
-    if (g2 < 0) {
-        S->status = ST_BREAK;
-        return;
-    }
-    double gn = sqrt(g2);
-    double g = S->gamma, d = S->delta;
-    double a0 = S->c * d - S->c_old * S->s * g;
-    double a1 = sqrt(a0 * a0 + gn * gn);
-    double a2 = S->s * d + S->c_old * S->c * g;
-    double a3 = S->s_old * g;
-    double cn = a0 / a1, sn = gn / a1;
-    S->a1 = a1;
-    S->a2 = a2;
-    S->a3 = a3;
-    S->c_new = cn;
-    S->eta_prev = S->eta;
-    S->gamma_cur = g;
-    S->eta = -sn * S->eta;
-    S->gamma_old = g;
-    S->gamma = gn;
-    S->c_old = S->c;
-    S->c = cn;
-    S->s_old = S->s;
-    S->s = sn;
-    S->it += 1;
-    S->est = S->rho0 * fabs(S->eta) / S->eta0;
-    S->lucky = (gn == 0);
-    S->check_true = (S->est <= S->tol) || S->lucky;
-}
-
-// Conditional-node handles of the device-side MINRES loop (all unused when n = 0):
-// h[0] the WHILE node around a body of ITER_UNROLL iterations, h[k] (k >= 1) the
-// IF node around iteration k of the body.
-struct Gates {
-    cudaGraphConditionalHandle h[6];
-    int n;
-};
-
-// after iteration k of a loop body: the IF nodes of the body's later iterations
-// open only while the solve runs; every gate this iteration can reach is
-// written, so no value is left from an earlier body
-__device__ void set_gates(MinresDev *S, const Gates &g, int k) {
-    const unsigned run = S->status == ST_RUN ? 1u : 0u;
-    for (int j = k + 1; j < g.n; ++j) cudaGraphSetConditional(g.h[j], run);
+    S->done = 0;
 }
 
 __global__ void k_loop_begin(cudaGraphConditionalHandle h, const MinresDev *S) {
@@ -560,39 +577,6 @@ __global__ void k_loop_next(cudaGraphConditionalHandle h, MinresDev *S) {
         run = false;
     }
     cudaGraphSetConditional(h, run ? 1u : 0u);
-}
-
-__global__ void k_scal_true(MinresDev *S, const double *part, Gates g, int k) {
-    __shared__ double sh[32];
-    double r2 = sum_parts(part, sh);
-    if (threadIdx.x) return;
-    if (S->status) {
-        set_gates(S, g, k);
-        return;
-    }
-    if (S->check_true) {
-        if (S->use_true) {
-            S->true_rel = sqrt(r2) / S->bnorm;
-            if (!isfinite(S->true_rel))
-                S->status = ST_NAN;
-            else if (S->true_rel <= S->tol)
-                S->status = ST_CONV;
-            else if (S->stall > 0 && S->est <= S->stall * S->tol)
-                S->status = ST_STALL;  // the recurrence has run far past what the true residual shows
-        } else {
-            S->status = ST_CONV;  // inner solves stop on the estimate alone
-        }
-        if (!S->status && S->lucky) S->status = ST_MAXIT;  // Krylov space exhausted above tol
-    }
-    if (!S->status && S->it >= S->maxit) S->status = ST_MAXIT;
-    set_gates(S, g, k);
-}
-
-__global__ void k_scal_final(MinresDev *S, const double *part) {
-    __shared__ double sh[32];
-    double r2 = sum_parts(part, sh);
-    if (threadIdx.x) return;
-    if (S->bnorm > 0) S->true_rel = sqrt(r2) / S->bnorm;
 }
 
 // ------------------------------------------------------------------ MINRES driver
@@ -631,6 +615,7 @@ template <typename T>
 struct MinresWork {
     using C = cplx_t<T>;
     DBuf<C> v[3], z[2], w[3], q;
+    DBuf<float2> z32[2];  // in place of z around an FP32 V-cycle
     DBuf<float2> jd;      // double-float Jacobian coefficients (mixed-precision solve)
     DBuf<float4> jp2;
     DBuf<double> part;
@@ -643,24 +628,31 @@ struct MinresWork {
     // phase and of one iteration (counted at capture)
     Graph loop;
     int64_t loop_init_launches = 0, loop_iter_launches = 0;
-    void ensure(int64_t nn) {
+    void ensure(int64_t nn, bool vc32) {
         if (!cap) GL_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         if (!cap_body) GL_CUDA(cudaStreamCreateWithFlags(&cap_body, cudaStreamNonBlocking));
         if (!cap_if) GL_CUDA(cudaStreamCreateWithFlags(&cap_if, cudaStreamNonBlocking));
-        if (n == nn) return;
-        init.reset();
-        body.reset();
-        loop.reset();
-        key = GraphKey{};
-        for (auto &b : v) b.alloc(nn);
-        for (auto &b : z) b.alloc(nn);
-        for (auto &b : w) b.alloc(nn);
-        q.alloc(nn);
-        part.alloc(2 * RED_BLOCKS);
-        S.alloc(1);
-        jd.release();
-        jp2.release();
-        n = nn;
+        if (n != nn) {
+            init.reset();
+            body.reset();
+            loop.reset();
+            key = GraphKey{};
+            for (auto &b : v) b.alloc(nn);
+            for (auto &b : z) b.release();
+            for (auto &b : z32) b.release();
+            for (auto &b : w) b.alloc(nn);
+            q.alloc(nn);
+            part.alloc(2 * RED_BLOCKS);
+            S.alloc(1);
+            jd.release();
+            jp2.release();
+            n = nn;
+        }
+        if (vc32) {
+            for (auto &b : z32) b.reserve(nn);
+        } else {
+            for (auto &b : z) b.reserve(nn);
+        }
     }
     void ensure_df() {
         if (jd.n != (size_t)n) {
@@ -675,20 +667,14 @@ struct MinresResult {
     double est, true_rel;
 };
 
-// vc32: run the V-cycle in FP32 even when the Krylov vectors are FP64
 template <typename T>
-static void precond_apply_any(gl_prec_s *p, const cplx_t<T> *v, cplx_t<T> *z, const int *stop, bool vc32,
-                              cudaStream_t s);
+static void precond_apply_any(gl_prec_s *p, const cplx_t<T> *v, cplx_t<T> *z, const int *stop, cudaStream_t s);
 template <>
-void precond_apply_any<double>(gl_prec_s *p, const double2 *v, double2 *z, const int *stop, bool vc32,
-                               cudaStream_t s) {
-    if (vc32)
-        precond_apply_p64_via32(p, v, z, stop, s);
-    else
-        precond_apply_p(p, v, z, stop, s);
+void precond_apply_any<double>(gl_prec_s *p, const double2 *v, double2 *z, const int *stop, cudaStream_t s) {
+    precond_apply_p(p, v, z, stop, s);
 }
 template <>
-void precond_apply_any<float>(gl_prec_s *p, const float2 *v, float2 *z, const int *stop, bool, cudaStream_t s) {
+void precond_apply_any<float>(gl_prec_s *p, const float2 *v, float2 *z, const int *stop, cudaStream_t s) {
     precond_apply_p32(p, v, z, stop, s);
 }
 
@@ -754,7 +740,7 @@ static void enqueue_init(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
     const int *stop = &S->status;
     double *part = W.part.get();
     int G = grid_for(n, 256);
-    C *v0 = W.v[0].get(), *v1 = W.v[1].get(), *z0 = W.z[0].get();
+    C *v0 = W.v[0].get(), *v1 = W.v[1].get();
     C *w0 = W.w[0].get(), *w1 = W.w[1].get();
     GL_CUDA(cudaMemsetAsync(v0, 0, n * sizeof(C), cs));
     GL_CUDA(cudaMemsetAsync(w0, 0, n * sizeof(C), cs));
@@ -765,20 +751,29 @@ static void enqueue_init(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
             k_jz_coef<<<G, 256, 0, cs>>>(n, m->lat_krem.get(), psi, W.jd.get(), W.jp2.get());
         }
     }
-    note_launch(3);
-    k_init_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, v1, part);
-    k_scal_init<<<1, 1024, 0, cs>>>(S, part);
+    note_launch(2);
+    k_init_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, v1, part, S);
     k_zero_if_bzero<C><<<G, 256, 0, cs>>>(n, S, x);
     GL_LAUNCH_CHECK();
+    if constexpr (std::is_same<T, double>::value) {
+        if (vc32 && p) {
+            note_launch(2);
+            k_round32<<<G, 256, 0, cs>>>(n, v1, p->mp_in.get());
+            precond_apply_p32(p, p->mp_in.get(), W.z32[0].get(), stop, cs);
+            k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v1, W.z32[0].get(), part, S, 0);
+            GL_LAUNCH_CHECK();
+            return;
+        }
+    }
+    C *z0 = W.z[0].get();
     if (p) {
-        precond_apply_any<T>(p, v1, z0, stop, vc32, cs);
+        precond_apply_any<T>(p, v1, z0, stop, cs);
     } else {
         note_launch();
         k_copy_if<C><<<G, 256, 0, cs>>>(n, v1, z0, stop);
     }
-    note_launch(2);
-    k_dot<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v1, z0, part, stop);
-    k_scal_gamma0<<<1, 1024, 0, cs>>>(S, part);
+    note_launch();
+    k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v1, z0, part, S, 0);
     GL_LAUNCH_CHECK();
 }
 
@@ -803,7 +798,10 @@ static void enqueue_body(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
     int G = grid_for(n, 256);
     C *v_old = W.v[0].get(), *v = W.v[1].get(), *v_new = W.v[2].get();
     C *z = W.z[0].get(), *z_new = W.z[1].get();
+    float2 *y = W.z32[0].get(), *y_new = W.z32[1].get();  // z around an FP32 V-cycle
     C *w_old = W.w[0].get(), *w = W.w[1].get(), *w_new = W.w[2].get();
+    bool mp = false;  // FP64 vectors around an FP32 V-cycle
+    if constexpr (std::is_same<T, double>::value) mp = vc32 && p;
     const Gates nog{{}, 0};
     const Gates &g = gates ? *gates : nog;
     for (int k = 0; k < ITER_UNROLL; ++k) {
@@ -833,69 +831,70 @@ static void enqueue_body(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
             // algorithmic bytes of the fused Jacobian + dot: off-diagonals, K_ii,
             // |V|, psi, z (own row; neighbours cached) and the written q
             int64_t nnz = (sizeof(T) == 8) ? m->K.nnz_real : m->K32.nnz_real;
-            bool use_df = false;
-            if constexpr (std::is_same<T, double>::value) use_df = df;
-            if (use_df) {
-                // z32 (8 B), d and psi^2 (24 B) and the written q (16 B) per row; the
-                // neighbours' z and the tables from cache
-                // FP32 operations of the error-free transformations, counted from the
-                // kernel: about 84 per stored neighbour and 100 per row, as flop
-                // equivalents (2 per operation: each takes an FMA issue slot)
-                ProfScope ps("jz", (double)n * (8 + 24 + 16), ks,
-                             2.0 * (84.0 * (double)m->K.nnz_real + 100.0 * (double)n));
-                k_jz_latdf<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_df_view(m), m->lat_hd, W.jd.get(),
-                                                               W.jp2.get(), p->mp_out.get(), (double2 *)W.q.get(),
-                                                               part, stop);
-            } else {
-                bool lat64 = false;
-                if constexpr (std::is_same<T, double>::value) lat64 = m->lat64_ok && p && p->lattice64;
-                if (lat64) {
+            bool done = false;
+            if constexpr (std::is_same<T, double>::value) {
+                if (df) {
+                    // z (8 B), d and psi^2 (24 B) and the written q (16 B) per row; the
+                    // neighbours' z and the tables from cache
+                    // FP32 operations of the error-free transformations, counted from the
+                    // kernel: about 84 per stored neighbour and 100 per row, as flop
+                    // equivalents (2 per operation: each takes an FMA issue slot)
+                    ProfScope ps("jz", (double)n * (8 + 24 + 16), ks,
+                                 2.0 * (84.0 * (double)m->K.nnz_real + 100.0 * (double)n));
+                    k_jz_latdf<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_df_view(m), m->lat_hd, W.jd.get(),
+                                                                   W.jp2.get(), y, W.q.get(), part, S);
+                    done = true;
+                } else if (m->lat64_ok && p && p->lattice64) {
                     // own z, K_ii, |V|, psi and the written q per row (48 + 16 B); the
                     // neighbours' z and the tables from cache; per row the six
                     // complex FMAs, the 1 / |V| scaling, the local terms and the dot
-                    if constexpr (std::is_same<T, double>::value) {
-                        ProfScope ps("jz", (double)n * (3 * sizeof(C) + 2 * sizeof(T)), ks,
-                                     8.0 * (double)nnz + 28.0 * (double)n);
+                    ProfScope ps("jz", (double)n * (3 * sizeof(C) + 2 * sizeof(T)), ks,
+                                 8.0 * (double)nnz + 28.0 * (double)n);
+                    if (mp)
+                        k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_view64(m), kd, psi, y, W.q.get(),
+                                                                       part, S);
+                    else
                         k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_view64(m), kd, psi, z, W.q.get(),
-                                                                      part, stop);
-                    }
-                } else {
-                    double jb = (double)nnz * (sizeof(C) + 4) + (double)n * (2 * sizeof(T) + 3 * sizeof(C));
-                    // a complex FMA (8 flops) per stored entry; per row the local terms
-                    // (K_ii - 1 + 2|psi|^2) z + psi^2 conj(z) (20) and the dot (5)
-                    ProfScope ps("jz", jb, ks, 8.0 * (double)nnz + 25.0 * (double)n);
-                    k_jz<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, z, W.q.get(), part, stop);
+                                                                       part, S);
+                    done = true;
                 }
             }
+            if (!done) {
+                double jb = (double)nnz * (sizeof(C) + 4) + (double)n * (2 * sizeof(T) + 3 * sizeof(C));
+                // a complex FMA (8 flops) per stored entry; per row the local terms (13)
+                // and the dot (5)
+                ProfScope ps("jz", jb, ks, 8.0 * (double)nnz + 18.0 * (double)n);
+                if constexpr (std::is_same<T, double>::value) {
+                    if (mp)
+                        k_jz<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, y, W.q.get(), part,
+                                                                               S);
+                }
+                if (!mp) k_jz<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, z, W.q.get(), part, S);
+            }
         }
-        note_launch(2);
-        k_scal_delta<<<1, 1024, 0, ks>>>(S, part);
-        bool fused = false;
-        if constexpr (std::is_same<T, double>::value) fused = vc32 && p;
-        if (fused) {
-            // FP32 V-cycle between the two fused passes
-            k_vnew_mp<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, (const double2 *)W.q.get(), (const double2 *)v,
-                                                          (const double2 *)v_old, (double2 *)v_new,
-                                                          p->mp_in.get());
-            precond_apply_p32(p, p->mp_in.get(), p->mp_out.get(), stop, ks);
-            note_launch(5);
-            k_widen_dot<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, m->volp.get(), (const double2 *)v_new,
-                                                            p->mp_out.get(), (double2 *)z_new, part, stop);
-        } else {
-            k_vnew<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, W.q.get(), v, v_old, v_new);
+        note_launch(4);
+        if constexpr (std::is_same<T, double>::value) {
+            if (mp) {
+                // FP32 V-cycle: its input is written beside v_new, its output read as it is
+                k_vnew<C, T, true><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, W.q.get(), v, v_old, v_new,
+                                                                       p->mp_in.get());
+                precond_apply_p32(p, p->mp_in.get(), y_new, stop, ks);
+                k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, vol, v_new, y_new, part, S, 1);
+                k_update<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, y, w_old, w, w_new, x);
+            }
+        }
+        if (!mp) {
+            k_vnew<C, T, false><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, W.q.get(), v, v_old, v_new, nullptr);
             if (p) {
-                precond_apply_any<T>(p, v_new, z_new, stop, vc32, ks);
+                precond_apply_any<T>(p, v_new, z_new, stop, ks);
             } else {
                 note_launch();
                 k_copy_if<C><<<G, 256, 0, ks>>>(n, v_new, z_new, stop);
             }
-            note_launch(5);
-            k_dot<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, vol, v_new, z_new, part, stop);
+            k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, vol, v_new, z_new, part, S, 1);
+            k_update<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, z, w_old, w, w_new, x);
         }
-        k_scal_givens<<<1, 1024, 0, ks>>>(S, part);
-        k_update<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, z, w_old, w, w_new, x);
-        k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, b, x, part, S, 0);
-        k_scal_true<<<1, 1024, 0, ks>>>(S, part, g, k);
+        k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, b, x, part, S, g, k, 0);
         GL_LAUNCH_CHECK();
         } catch (...) {
             if (child) {
@@ -909,9 +908,8 @@ static void enqueue_body(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
         v_old = v;
         v = v_new;
         v_new = t;
-        t = z;
-        z = z_new;
-        z_new = t;
+        std::swap(z, z_new);
+        std::swap(y, y_new);
         t = w_old;
         w_old = w;
         w = w_new;
@@ -928,7 +926,7 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
     using O = SolveOps<T>;
     using C = cplx_t<T>;
     int64_t n = m->n;
-    W.ensure(n);
+    W.ensure(n, std::is_same<T, double>::value && vc32 && p);
     if (df) W.ensure_df();
     MinresDev *S = W.S.get();
     double *part = W.part.get();
@@ -1027,10 +1025,9 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
     }
     }
     if (use_true) {
-        note_launch(2);
+        note_launch();
         k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, part, S,
-                                                              1);
-        k_scal_final<<<1, 1024, 0, s>>>(S, part);
+                                                              Gates{{}, 0}, 0, 1);
         GL_LAUNCH_CHECK();
         GL_CUDA(cudaMemcpyAsync(&h, S, sizeof(MinresDev), cudaMemcpyDeviceToHost, s));
         GL_CUDA(cudaStreamSynchronize(s));
@@ -1172,7 +1169,7 @@ void batch_create(gl_batch_s *B, int count, gl_mesh_s *const *meshes, const doub
         I->m = meshes[i];
         I->p = new gl_prec_s();
         precond_setup(I->p, I->m, psi[i], so, s);
-        I->W.ensure(I->m->n);
+        I->W.ensure(I->m->n, B->vc32);
         // as in a single mixed solve: the double-float Jacobian wherever the mesh
         // has the checked lattice stencil
         I->df = B->vc32 && I->p->lattice && I->m->lat_ok;
@@ -1241,8 +1238,7 @@ static void batch_build(gl_batch_s *B, const double2 *const *b, double2 *const *
             // final FP64 true residual, back to node order
             k_true_resid<double2, double><<<RED_BLOCKS, RED_THREADS, 0, si>>>(
                 n, I.m->K.view(), I.m->kdiag.get(), I.m->volp.get(), I.p->psi_p.get(), I.b.get(), I.x.get(),
-                I.W.part.get(), S, 1);
-            k_scal_final<<<1, 1024, 0, si>>>(S, I.W.part.get());
+                I.W.part.get(), S, Gates{{}, 0}, 0, 1);
             GL_LAUNCH_CHECK();
             permute_out(n, I.m->perm.get(), I.x.get(), x[i], si);
             GL_CUDA(cudaEventRecord(B->ev[i + 1], si));
