@@ -126,8 +126,8 @@ typedef struct {
                             value before its FP32 rounding, at the FP32 rate); 0 = FP64 arithmetic.  The
                             FP64 V-cycle always uses FP64 (default 1) */
     int device_loop;     /* 1: a solve runs as one CUDA graph whose MINRES iterations loop on the device
-                            (conditional WHILE / IF nodes; no kernel after convergence, one host wait);
-                            0: the same six-iteration body graph replayed by the host, which polls the
+                            (a conditional WHILE node; no kernel after convergence, one host wait);
+                            0: a body graph of six iterations replayed by the host, which polls the
                             status word between replays (for profilers that cannot see inside
                             conditional graphs).  Solves that time a kernel class with gl_profile_begin,
                             and R_inf, always use 0 (default 1) */

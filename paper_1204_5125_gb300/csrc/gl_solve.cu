@@ -7,10 +7,9 @@
 // partial per block of a fixed grid and is summed in index order, so results do
 // not depend on scheduling.  A device status word stops all kernels once the
 // solve has converged or failed.  A solve is one CUDA graph that loops on the
-// device (a WHILE conditional node over bodies of six iterations, the later
-// ones in IF nodes that the previous iteration's scalar kernel opens), so the
-// host waits once; options.device_loop = 0 replays the body graph from the host
-// instead, reading the status word between replays.
+// device (a WHILE conditional node over one iteration), so the host waits once;
+// options.device_loop = 0 replays a body of six iterations from the host instead,
+// reading the status word between replays.
 //
 // GL_MIXED: FP64 defect correction x <- x + e around inner MINRES solves of
 // J e = r whose vectors, Jacobian applies and V-cycles are FP32 (dots and
@@ -25,14 +24,17 @@
 namespace gl {
 
 struct MinresDev {
-    double gamma, gamma_old, eta, eta0, c, c_old, s, s_old;
-    double delta, a1, a2, a3, c_new, eta_prev, gamma_cur;
+    double gamma, eta, eta0, c, c_old, s, s_old, delta;
     double bnorm, tol, est, true_rel;
     double rho0;      // ||b - J x0||_D / ||b||_D: scales the recurrence's estimate to be relative to b
     // factors of the vector kernels, formed once by the scalar steps (an FP64 division a
     // thread kept the FP64 pipe for longer than a small vector's own work)
-    double ig, dg, go;        // v_new = ig q - dg v - go v_old
-    double sz, s3, s2, ce;    // w_new = sz z - s3 w_old - s2 w ; x += ce w_new
+    double ig, dg, go;        // v_new = ig q - dg v - go v_old; ig = 1 / gamma
+    double k2, k3;            // w_new = ig z - k3 w_old - k2 w; the direction is sig w
+    double sig, sig_old;
+    double tau;               // x += tau w_new
+    double est_scale;         // rho0 / eta0
+    double go_next, ig_next;  // go and ig of the next iteration
     int it, maxit, check_true, status, lucky, use_true, replays;
     unsigned done;    // blocks of the current reduction that have written their partials
     double stall;     // > 0: stop with ST_STALL once the estimate is below stall * tol while the true
@@ -86,20 +88,23 @@ __device__ bool last_block(MinresDev *S) {
     return last;
 }
 
-// Conditional-node handles of the device-side MINRES loop (all unused when n = 0):
-// h[0] the WHILE node around a body of ITER_UNROLL iterations, h[k] (k >= 1) the
-// IF node around iteration k of the body.
-struct Gates {
-    cudaGraphConditionalHandle h[6];
-    int n;
+// The WHILE node of a device-side MINRES loop; its condition is written by the last
+// kernel of a loop body (use != 0).
+struct LoopGate {
+    cudaGraphConditionalHandle h;
+    int use;
 };
-
-// after iteration k of a loop body: the IF nodes of the body's later iterations
-// open only while the solve runs; every gate this iteration can reach is
-// written, so no value is left from an earlier body
-__device__ void set_gates(MinresDev *S, const Gates &g, int k) {
-    const unsigned run = S->status == ST_RUN ? 1u : 0u;
-    for (int j = k + 1; j < g.n; ++j) cudaGraphSetConditional(g.h[j], run);
+// end of a loop body: another one while the solve runs, at most maxit + 2 (then
+// ST_MAXIT), so the loop ends whatever the state
+__device__ void loop_next(MinresDev *S, const LoopGate &g) {
+    if (!g.use) return;
+    S->replays += 1;
+    bool run = S->status == ST_RUN;
+    if (run && S->replays >= S->maxit + 2) {
+        S->status = ST_MAXIT;
+        run = false;
+    }
+    cudaGraphSetConditional(g.h, run ? 1u : 0u);
 }
 
 // bb = <b, b>_R, vv = ||b - J x0||_D^2
@@ -140,21 +145,36 @@ __device__ void scal_gamma0(MinresDev *S, double g2) {
     }
     double g = sqrt(g2);
     S->gamma = g;
-    S->gamma_old = 1.0;
+    S->ig_next = 1.0 / g;
+    S->go_next = g;  // v_0 = 0, with gamma_0 = 1
+    S->sig = S->sig_old = 1.0;
     S->eta = S->eta0 = g;
+    S->est_scale = S->rho0 / g;
     S->c = S->c_old = 1.0;
     S->s = S->s_old = 0.0;
     if (g == 0) S->status = ST_CONV;
 }
 // d = <J z, z>_R
 __device__ void scal_delta(MinresDev *S, double d) {
-    S->delta = d / (S->gamma * S->gamma);
-    S->ig = 1.0 / S->gamma;
-    S->dg = S->delta / S->gamma;
-    S->go = S->gamma / S->gamma_old;
+    const double ig = S->ig_next, g = S->gamma;
+    S->ig = ig;
+    S->go = S->go_next;
+    d = d * ig * ig;
+    S->delta = d;
+    S->dg = d * ig;
+    S->k3 = S->s_old * g * S->sig_old;
+    S->k2 = (S->s * d + S->c_old * S->c * g) * S->sig;
 }
-// g2 = <v_new, z_new>_R
-__device__ void scal_givens(MinresDev *S, double g2) {
+// g2 = <v_new, z_new>_R.  One thread takes the step, so its dependent FP64 divisions and
+// square roots are what it costs: two roots and two reciprocals, one of them in another
+// warp (`other`), where a division per scalar took 3 us more.
+__device__ void scal_givens(MinresDev *S, double g2, bool other) {
+    const double gn = sqrt(g2);
+    if (other) {  // the next iteration's own factors (unused unless it runs)
+        S->go_next = gn * S->ig;
+        S->ig_next = 1.0 / gn;
+        return;
+    }
     if (!isfinite(g2) || !isfinite(S->delta)) {
         S->status = ST_NAN;
         return;
@@ -163,27 +183,20 @@ __device__ void scal_givens(MinresDev *S, double g2) {
         S->status = ST_BREAK;
         return;
     }
-    double gn = sqrt(g2);
-    double g = S->gamma, d = S->delta;
-    double a0 = S->c * d - S->c_old * S->s * g;
-    double a1 = sqrt(a0 * a0 + gn * gn);
-    double a2 = S->s * d + S->c_old * S->c * g;
-    double a3 = S->s_old * g;
-    double cn = a0 / a1, sn = gn / a1;
-    const double ia1 = 1.0 / a1;
-    S->sz = ia1 / g;
-    S->s3 = a3 * ia1;
-    S->s2 = a2 * ia1;
-    S->ce = cn * S->eta;
+    const double a0 = S->c * S->delta - S->c_old * S->s * S->gamma;
+    const double a1 = sqrt(a0 * a0 + gn * gn);
+    const double ia1 = 1.0 / a1, cn = a0 * ia1, sn = gn * ia1;
+    S->sig_old = S->sig;
+    S->sig = ia1;
+    S->tau = cn * S->eta * ia1;
     S->eta = -sn * S->eta;
-    S->gamma_old = g;
     S->gamma = gn;
     S->c_old = S->c;
     S->c = cn;
     S->s_old = S->s;
     S->s = sn;
     S->it += 1;
-    S->est = S->rho0 * fabs(S->eta) / S->eta0;
+    S->est = S->est_scale * fabs(S->eta);
     S->lucky = (gn == 0);
     S->check_true = (S->est <= S->tol) || S->lucky;
 }
@@ -234,13 +247,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_resid(int64_t n, SellView<
     if (threadIdx.x == 0) scal_init(S, bb, vv);
 }
 
-// <x, y>_R and the scalar step behind it (0: gamma_1, 1: Givens); y may be the FP32
-// vector of a mixed-precision solve, whose FP64 image it stands for
+// <v, z>_R and the scalar step behind it: gamma_1 with v = v0, or (givens) Givens with
+// the vector that k_step wrote, v1 and v0 in turn.  z may be the FP32 vector of a
+// mixed-precision solve, whose FP64 image it stands for.
 template <typename C, typename R, typename Y>
-__global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t n, const R *vol, const C *x, const Y *y, double *part,
-                                                     MinresDev *S, int givens) {
+__global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t n, const R *vol, const C *v0, const C *v1, const Y *y,
+                                                     double *part, MinresDev *S, int givens) {
     __shared__ double sh[32];
     if (S->status) return;
+    const C *x = givens && !(S->it & 1) ? v1 : v0;
     double a = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -263,11 +278,14 @@ __global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t n, const R *vol, co
     double t = block_sum(a, sh);
     if (threadIdx.x == 0) part[blockIdx.x] = t;
     if (!last_block(S)) return;
-    const double g2 = sum_parts(part, sh);
-    if (threadIdx.x) return;
+    double g2 = sum_parts(part, sh);
+    if (threadIdx.x == 0) sh[0] = g2;
+    __syncthreads();
+    g2 = sh[0];
+    if (threadIdx.x != 0 && threadIdx.x != 32) return;
     if (givens)
-        scal_givens(S, g2);
-    else
+        scal_givens(S, g2, threadIdx.x == 32);
+    else if (threadIdx.x == 0)
         scal_gamma0(S, g2);
 }
 
@@ -460,77 +478,82 @@ void jacobian_apply_pdf(gl_mesh_s *m, const double2 *psi, const double2 *phi, do
     GL_CUDA(cudaStreamSynchronize(s));
 }
 
-// v_new = q / gamma - (delta / gamma) v - (gamma / gamma_old) v_old; with v32 (the
-// mixed-precision form) also rounded to the FP32 V-cycle's input.  Four rows per step
-// with every load issued first.
-template <typename C, typename R, bool MP>
-__global__ void __launch_bounds__(RED_THREADS) k_vnew(int64_t n, const MinresDev *S, const C *q, const C *v,
-                                                      const C *v_old, C *v_new, float2 *v32) {
+// The two recurrences that follow the Jacobian:
+//   v_new = q / gamma - (delta / gamma) v - (gamma / gamma_old) v_old
+//   w_new = z / gamma - a3 w_old - a2 w
+// (w_new without its factor 1 / a1, which the next scalar step knows and hands on as
+// sig), each written over its oldest vector; the two vectors of a pair change roles
+// with the iteration's parity, so one captured iteration serves all.  in: the V-cycle's
+// input, v_new as it is or (float2) rounded; Z: float2 when z is the FP32 V-cycle's
+// output.  Four rows per step with every load issued first.
+template <typename C, typename R, typename Z>
+__global__ void __launch_bounds__(RED_THREADS) k_step(int64_t n, const MinresDev *S, const C *q, C *v0, C *v1, C *w0,
+                                                      C *w1, const Z *z, Z *in) {
     if (S->status) return;
-    const R ig = (R)S->ig, dg = (R)S->dg, go = (R)S->go;
+    const R ig = (R)S->ig, dg = (R)S->dg, go = (R)S->go, k2 = (R)S->k2, k3 = (R)S->k3;
+    const bool odd = S->it & 1;
+    C *v = odd ? v1 : v0, *vo = odd ? v0 : v1, *w = odd ? w1 : w0, *wo = odd ? w0 : w1;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    auto put = [&](int64_t i, C a, C b, C c) {
+    auto put = [&](int64_t i, C a, C b, C c, Z zz, C ww, C wv) {
         const C r = mk(a.x * ig - dg * b.x - go * c.x, a.y * ig - dg * b.y - go * c.y);
-        v_new[i] = r;
-        if (MP) v32[i] = make_float2((float)r.x, (float)r.y);
+        vo[i] = r;
+        Z o;
+        o.x = r.x;
+        o.y = r.y;
+        in[i] = o;
+        wo[i] = mk((R)zz.x * ig - k3 * wv.x - k2 * ww.x, (R)zz.y * ig - k3 * wv.y - k2 * ww.y);
     };
-    for (; p + 3 * stride < n; p += 4 * stride) {
-        C a[4], b[4], c[4];
+    for (; p + stride < n; p += 2 * stride) {
+        C a[2], b[2], c[2], d[2], e[2];
+        Z f[2];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 2; ++u) {
             a[u] = q[p + u * stride];
             b[u] = v[p + u * stride];
-            c[u] = v_old[p + u * stride];
+            c[u] = vo[p + u * stride];
+            f[u] = z[p + u * stride];
+            d[u] = w[p + u * stride];
+            e[u] = wo[p + u * stride];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) put(p + u * stride, a[u], b[u], c[u]);
+        for (int u = 0; u < 2; ++u) put(p + u * stride, a[u], b[u], c[u], f[u], d[u], e[u]);
     }
-    for (; p < n; p += stride) put(p, q[p], v[p], v_old[p]);
+    if (p < n) put(p, q[p], v[p], vo[p], z[p], w[p], wo[p]);
 }
 
-// w_new = (z / gamma - a3 w_old - a2 w) / a1 ; x += c_new eta w_new, with the factors of
-// MinresDev (three FP64 operations per component; this stream is bound by GB300's FP64
-// pipe before HBM).  Z: float2 when z is the FP32 V-cycle's output.
-template <typename C, typename R, typename Z>
-__global__ void __launch_bounds__(RED_THREADS) k_update(int64_t n, const MinresDev *S, const Z *z, const C *w_old,
-                                                        const C *w, C *w_new, C *x) {
+// x += tau w_new (the vector that k_step wrote; the Givens step has counted the iteration)
+template <typename C, typename R>
+__global__ void __launch_bounds__(RED_THREADS) k_update(int64_t n, const MinresDev *S, const C *w0, const C *w1, C *x) {
     if (S->status) return;
-    const R sz = (R)S->sz, s3 = (R)S->s3, s2 = (R)S->s2, ce = (R)S->ce;
+    const R tau = (R)S->tau;
+    const C *w = S->it & 1 ? w1 : w0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    auto upd = [&](Z zz, C wo, C ww, C xx, int64_t q) {
-        const C wn = mk((R)zz.x * sz - s3 * wo.x - s2 * ww.x, (R)zz.y * sz - s3 * wo.y - s2 * ww.y);
-        w_new[q] = wn;
-        x[q] = mk(xx.x + ce * wn.x, xx.y + ce * wn.y);
-    };
     for (; p + 3 * stride < n; p += 4 * stride) {
-        Z zz[4];
-        C wo[4], ww[4], xx[4];
+        C ww[4], xx[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            zz[u] = z[p + u * stride];
-            wo[u] = w_old[p + u * stride];
             ww[u] = w[p + u * stride];
             xx[u] = x[p + u * stride];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) upd(zz[u], wo[u], ww[u], xx[u], p + u * stride);
+        for (int u = 0; u < 4; ++u) x[p + u * stride] = mk(xx[u].x + tau * ww[u].x, xx[u].y + tau * ww[u].y);
     }
-    for (; p < n; p += stride) upd(z[p], w_old[p], w[p], x[p], p);
+    for (; p < n; p += stride) x[p] = mk(x[p].x + tau * w[p].x, x[p].y + tau * w[p].y);
 }
 
-// ||b - J x||_D^2 when the Givens step asked for a check, and the end of iteration k of
-// a loop body; with `final` the true residual of the solve's result, whatever the status
+// ||b - J x||_D^2 when the Givens step asked for a check, and the end of the iteration;
+// with `final` the true residual of the solve's result, whatever the status
 template <typename C, typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_true_resid(int64_t n, SellView<C> K, const R *kd, const R *vol,
                                                             const C *psi, const C *b, const C *x, double *part,
-                                                            MinresDev *S, Gates g, int k, int final) {
+                                                            MinresDev *S, LoopGate g, int final) {
     __shared__ double sh[32];
     if (!final && (S->status || !S->check_true)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             if (!S->status) scal_true(S, 0.0);
-            set_gates(S, g, k);
+            loop_next(S, g);
         }
         return;
     }
@@ -551,7 +574,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_true_resid(int64_t n, SellView<
         return;
     }
     scal_true(S, r2);
-    set_gates(S, g, k);
+    loop_next(S, g);
 }
 
 // solve parameters, written before the captured init phase reads them
@@ -567,26 +590,15 @@ __global__ void k_loop_begin(cudaGraphConditionalHandle h, const MinresDev *S) {
     cudaGraphSetConditional(h, S->status == ST_RUN ? 1u : 0u);
 }
 
-// end of a loop body: another body while the solve runs, at most maxit / 6 + 2
-// bodies (then ST_MAXIT), so the loop ends whatever the state
-__global__ void k_loop_next(cudaGraphConditionalHandle h, MinresDev *S) {
-    S->replays += 1;
-    bool run = S->status == ST_RUN;
-    if (run && S->replays >= S->maxit / 6 + 2) {
-        S->status = ST_MAXIT;
-        run = false;
-    }
-    cudaGraphSetConditional(h, run ? 1u : 0u);
-}
-
 // ------------------------------------------------------------------ MINRES driver
-// The initial phase and a body of ITER_UNROLL iterations are captured once as
-// CUDA graphs and replayed; every kernel turns into a no-op once the status word
-// is set, so a replay past convergence costs only launch latency.  The three v,
-// two z and three w buffers rotate, so the body holds a multiple of 6 iterations
-// and starts every replay with the same buffer roles.
+// A solve is the initial phase and a WHILE node over one iteration, captured once per
+// (state, right-hand side, solution, preconditioner): the vectors of the recurrences
+// change roles by the iteration's parity on the device, so the body is one iteration
+// and the loop stops where the solve does.  (Six iterations in IF nodes, which the
+// rotation of the buffers needed before, took 0.29 ms more to capture and instantiate
+// for every new state.)  For profilers the host replays a body of ITER_UNROLL
+// iterations instead; kernels behind the end of the solve return at once.
 constexpr int ITER_UNROLL = 6;
-static_assert(ITER_UNROLL == 6, "k_loop_next bounds the device loop by maxit / 6 + 2 bodies");
 
 struct Graph {
     cudaGraphExec_t exec = nullptr;
@@ -614,14 +626,15 @@ struct GraphKey {
 template <typename T>
 struct MinresWork {
     using C = cplx_t<T>;
-    DBuf<C> v[3], z[2], w[3], q;
-    DBuf<float2> z32[2];  // in place of z around an FP32 V-cycle
+    DBuf<C> v[2], w[2], q;
+    DBuf<C> z, in;     // the V-cycle's output and input (FP32 V-cycles have the next two)
+    DBuf<float2> z32;
     DBuf<float2> jd;      // double-float Jacobian coefficients (mixed-precision solve)
     DBuf<float4> jp2;
     DBuf<double> part;
     DBuf<MinresDev> S;
     int64_t n = 0;
-    cudaStream_t cap = nullptr, cap_body = nullptr, cap_if = nullptr;
+    cudaStream_t cap = nullptr, cap_body = nullptr;
     GraphKey key;
     Graph init, body;
     // the device-side loop: the whole solve in one graph; launches of its initial
@@ -631,15 +644,15 @@ struct MinresWork {
     void ensure(int64_t nn, bool vc32) {
         if (!cap) GL_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
         if (!cap_body) GL_CUDA(cudaStreamCreateWithFlags(&cap_body, cudaStreamNonBlocking));
-        if (!cap_if) GL_CUDA(cudaStreamCreateWithFlags(&cap_if, cudaStreamNonBlocking));
         if (n != nn) {
             init.reset();
             body.reset();
             loop.reset();
             key = GraphKey{};
             for (auto &b : v) b.alloc(nn);
-            for (auto &b : z) b.release();
-            for (auto &b : z32) b.release();
+            z.release();
+            in.release();
+            z32.release();
             for (auto &b : w) b.alloc(nn);
             q.alloc(nn);
             part.alloc(2 * RED_BLOCKS);
@@ -649,9 +662,10 @@ struct MinresWork {
             n = nn;
         }
         if (vc32) {
-            for (auto &b : z32) b.reserve(nn);
+            z32.reserve(nn);
         } else {
-            for (auto &b : z) b.reserve(nn);
+            z.reserve(nn);
+            in.reserve(nn);
         }
     }
     void ensure_df() {
@@ -740,11 +754,9 @@ static void enqueue_init(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
     const int *stop = &S->status;
     double *part = W.part.get();
     int G = grid_for(n, 256);
-    C *v0 = W.v[0].get(), *v1 = W.v[1].get();
-    C *w0 = W.w[0].get(), *w1 = W.w[1].get();
-    GL_CUDA(cudaMemsetAsync(v0, 0, n * sizeof(C), cs));
-    GL_CUDA(cudaMemsetAsync(w0, 0, n * sizeof(C), cs));
-    GL_CUDA(cudaMemsetAsync(w1, 0, n * sizeof(C), cs));
+    C *v = W.v[0].get();
+    GL_CUDA(cudaMemsetAsync(W.v[1].get(), 0, n * sizeof(C), cs));
+    for (auto &w : W.w) GL_CUDA(cudaMemsetAsync(w.get(), 0, n * sizeof(C), cs));
     if constexpr (std::is_same<T, double>::value) {
         if (df) {
             note_launch();
@@ -752,40 +764,35 @@ static void enqueue_init(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
         }
     }
     note_launch(2);
-    k_init_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, v1, part, S);
+    k_init_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, v, part, S);
     k_zero_if_bzero<C><<<G, 256, 0, cs>>>(n, S, x);
     GL_LAUNCH_CHECK();
     if constexpr (std::is_same<T, double>::value) {
         if (vc32 && p) {
             note_launch(2);
-            k_round32<<<G, 256, 0, cs>>>(n, v1, p->mp_in.get());
-            precond_apply_p32(p, p->mp_in.get(), W.z32[0].get(), stop, cs);
-            k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v1, W.z32[0].get(), part, S, 0);
+            k_round32<<<G, 256, 0, cs>>>(n, v, p->mp_in.get());
+            precond_apply_p32(p, p->mp_in.get(), W.z32.get(), stop, cs);
+            k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v, v, W.z32.get(), part, S, 0);
             GL_LAUNCH_CHECK();
             return;
         }
     }
-    C *z0 = W.z[0].get();
     if (p) {
-        precond_apply_any<T>(p, v1, z0, stop, cs);
+        precond_apply_any<T>(p, v, W.z.get(), stop, cs);
     } else {
         note_launch();
-        k_copy_if<C><<<G, 256, 0, cs>>>(n, v1, z0, stop);
+        k_copy_if<C><<<G, 256, 0, cs>>>(n, v, W.z.get(), stop);
     }
     note_launch();
-    k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v1, z0, part, S, 0);
+    k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, O::vol(m), v, v, W.z.get(), part, S, 0);
     GL_LAUNCH_CHECK();
 }
 
-// Enqueues ITER_UNROLL MINRES iterations on `cs` (buffer roles rotate inside
-// and return to the starting roles at the end).  With `gates` (the device-side
-// loop; cs captures into the loop body) iterations 1.. each sit in an IF node,
-// captured on cs_child, which the previous iteration opens only while the solve
-// runs.
+// Enqueues one MINRES iteration on `cs`; with `gate` it ends a loop body.
 template <typename T>
-static void enqueue_body(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const cplx_t<T> *b, cplx_t<T> *x,
-                         bool vc32, bool df, MinresWork<T> &W, cudaStream_t cs, const Gates *gates = nullptr,
-                         cudaStream_t cs_child = nullptr) {
+static void enqueue_iteration(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const cplx_t<T> *b, cplx_t<T> *x,
+                              bool vc32, bool df, MinresWork<T> &W, cudaStream_t cs,
+                              const LoopGate &gate = LoopGate{{}, 0}) {
     using O = SolveOps<T>;
     using C = cplx_t<T>;
     int64_t n = m->n;
@@ -795,126 +802,103 @@ static void enqueue_body(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, const
     auto K = O::K(m);
     auto kd = O::kdiag(m);
     auto vol = O::vol(m);
-    int G = grid_for(n, 256);
-    C *v_old = W.v[0].get(), *v = W.v[1].get(), *v_new = W.v[2].get();
-    C *z = W.z[0].get(), *z_new = W.z[1].get();
-    float2 *y = W.z32[0].get(), *y_new = W.z32[1].get();  // z around an FP32 V-cycle
-    C *w_old = W.w[0].get(), *w = W.w[1].get(), *w_new = W.w[2].get();
-    bool mp = false;  // FP64 vectors around an FP32 V-cycle
+    C *v0 = W.v[0].get(), *v1 = W.v[1].get(), *w0 = W.w[0].get(), *w1 = W.w[1].get();
+    C *q = W.q.get(), *z = W.z.get();
+    float2 *y = W.z32.get();  // z around an FP32 V-cycle
+    bool mp = false;          // FP64 vectors around an FP32 V-cycle
     if constexpr (std::is_same<T, double>::value) mp = vc32 && p;
-    const Gates nog{{}, 0};
-    const Gates &g = gates ? *gates : nog;
-    for (int k = 0; k < ITER_UNROLL; ++k) {
-        cudaStream_t ks = cs;
-        cudaGraph_t child = nullptr;
-        if (gates && k > 0) {
-            cudaStreamCaptureStatus cst;
-            cudaGraph_t cg = nullptr;
-            const cudaGraphNode_t *deps = nullptr;
-            size_t ndeps = 0;
-            GL_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
-            cudaGraphNodeParams cp = {};
-            cp.type = cudaGraphNodeTypeConditional;
-            cp.conditional.handle = g.h[k];
-            cp.conditional.type = cudaGraphCondTypeIf;
-            cp.conditional.size = 1;
-            cudaGraphNode_t inode;
-            GL_CUDA(cudaGraphAddNode(&inode, cg, deps, nullptr, ndeps, &cp));
-            child = cp.conditional.phGraph_out[0];
-            GL_CUDA(cudaStreamUpdateCaptureDependencies(cs, &inode, nullptr, 1, cudaStreamSetCaptureDependencies));
-            GL_CUDA(cudaStreamBeginCaptureToGraph(cs_child, child, nullptr, nullptr, 0,
-                                                  cudaStreamCaptureModeThreadLocal));
-            ks = cs_child;
-        }
-        try {
-        {
-            // algorithmic bytes of the fused Jacobian + dot: off-diagonals, K_ii,
-            // |V|, psi, z (own row; neighbours cached) and the written q
-            int64_t nnz = (sizeof(T) == 8) ? m->K.nnz_real : m->K32.nnz_real;
-            bool done = false;
-            if constexpr (std::is_same<T, double>::value) {
-                if (df) {
-                    // z (8 B), d and psi^2 (24 B) and the written q (16 B) per row; the
-                    // neighbours' z and the tables from cache
-                    // FP32 operations of the error-free transformations, counted from the
-                    // kernel: about 84 per stored neighbour and 100 per row, as flop
-                    // equivalents (2 per operation: each takes an FMA issue slot)
-                    ProfScope ps("jz", (double)n * (8 + 24 + 16), ks,
-                                 2.0 * (84.0 * (double)m->K.nnz_real + 100.0 * (double)n));
-                    k_jz_latdf<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_df_view(m), m->lat_hd, W.jd.get(),
-                                                                   W.jp2.get(), y, W.q.get(), part, S);
-                    done = true;
-                } else if (m->lat64_ok && p && p->lattice64) {
-                    // own z, K_ii, |V|, psi and the written q per row (48 + 16 B); the
-                    // neighbours' z and the tables from cache; per row the six
-                    // complex FMAs, the 1 / |V| scaling, the local terms and the dot
-                    ProfScope ps("jz", (double)n * (3 * sizeof(C) + 2 * sizeof(T)), ks,
-                                 8.0 * (double)nnz + 28.0 * (double)n);
-                    if (mp)
-                        k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_view64(m), kd, psi, y, W.q.get(),
-                                                                       part, S);
-                    else
-                        k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, lattice_view64(m), kd, psi, z, W.q.get(),
-                                                                       part, S);
-                    done = true;
-                }
-            }
-            if (!done) {
-                double jb = (double)nnz * (sizeof(C) + 4) + (double)n * (2 * sizeof(T) + 3 * sizeof(C));
-                // a complex FMA (8 flops) per stored entry; per row the local terms (13)
-                // and the dot (5)
-                ProfScope ps("jz", jb, ks, 8.0 * (double)nnz + 18.0 * (double)n);
-                if constexpr (std::is_same<T, double>::value) {
-                    if (mp)
-                        k_jz<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, y, W.q.get(), part,
-                                                                               S);
-                }
-                if (!mp) k_jz<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, z, W.q.get(), part, S);
-            }
-        }
-        note_launch(4);
+    {
+        // algorithmic bytes of the fused Jacobian + dot: off-diagonals, K_ii,
+        // |V|, psi, z (own row; neighbours cached) and the written q
+        int64_t nnz = (sizeof(T) == 8) ? m->K.nnz_real : m->K32.nnz_real;
+        bool done = false;
         if constexpr (std::is_same<T, double>::value) {
-            if (mp) {
-                // FP32 V-cycle: its input is written beside v_new, its output read as it is
-                k_vnew<C, T, true><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, W.q.get(), v, v_old, v_new,
-                                                                       p->mp_in.get());
-                precond_apply_p32(p, p->mp_in.get(), y_new, stop, ks);
-                k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, vol, v_new, y_new, part, S, 1);
-                k_update<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, y, w_old, w, w_new, x);
+            if (df) {
+                // z (8 B), d and psi^2 (24 B) and the written q (16 B) per row; the
+                // neighbours' z and the tables from cache
+                // FP32 operations of the error-free transformations, counted from the
+                // kernel: about 84 per stored neighbour and 100 per row, as flop
+                // equivalents (2 per operation: each takes an FMA issue slot)
+                ProfScope ps("jz", (double)n * (8 + 24 + 16), cs,
+                             2.0 * (84.0 * (double)m->K.nnz_real + 100.0 * (double)n));
+                k_jz_latdf<<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, lattice_df_view(m), m->lat_hd, W.jd.get(),
+                                                               W.jp2.get(), y, q, part, S);
+                done = true;
+            } else if (m->lat64_ok && p && p->lattice64) {
+                // own z, K_ii, |V|, psi and the written q per row (48 + 16 B); the
+                // neighbours' z and the tables from cache; per row the six
+                // complex FMAs, the 1 / |V| scaling, the local terms and the dot
+                ProfScope ps("jz", (double)n * (3 * sizeof(C) + 2 * sizeof(T)), cs,
+                             8.0 * (double)nnz + 28.0 * (double)n);
+                if (mp)
+                    k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, lattice_view64(m), kd, psi, y, q, part, S);
+                else
+                    k_jz_lat64<<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, lattice_view64(m), kd, psi, z, q, part, S);
+                done = true;
             }
         }
-        if (!mp) {
-            k_vnew<C, T, false><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, W.q.get(), v, v_old, v_new, nullptr);
-            if (p) {
-                precond_apply_any<T>(p, v_new, z_new, stop, ks);
-            } else {
-                note_launch();
-                k_copy_if<C><<<G, 256, 0, ks>>>(n, v_new, z_new, stop);
+        if (!done) {
+            double jb = (double)nnz * (sizeof(C) + 4) + (double)n * (2 * sizeof(T) + 3 * sizeof(C));
+            // a complex FMA (8 flops) per stored entry; per row the local terms (13)
+            // and the dot (5)
+            ProfScope ps("jz", jb, cs, 8.0 * (double)nnz + 18.0 * (double)n);
+            if constexpr (std::is_same<T, double>::value) {
+                if (mp) k_jz<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, K, kd, vol, psi, y, q, part, S);
             }
-            k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, vol, v_new, z_new, part, S, 1);
-            k_update<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, S, z, w_old, w, w_new, x);
+            if (!mp) k_jz<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, K, kd, vol, psi, z, q, part, S);
         }
-        k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, ks>>>(n, K, kd, vol, psi, b, x, part, S, g, k, 0);
-        GL_LAUNCH_CHECK();
-        } catch (...) {
-            if (child) {
-                cudaGraph_t dummy = nullptr;
-                cudaStreamEndCapture(cs_child, &dummy);
-            }
-            throw;
-        }
-        if (child) GL_CUDA(cudaStreamEndCapture(cs_child, &child));
-        C *t = v_old;
-        v_old = v;
-        v = v_new;
-        v_new = t;
-        std::swap(z, z_new);
-        std::swap(y, y_new);
-        t = w_old;
-        w_old = w;
-        w = w_new;
-        w_new = t;
     }
+    note_launch(4);
+    if constexpr (std::is_same<T, double>::value) {
+        if (mp) {
+            k_step<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, S, q, v0, v1, w0, w1, y, p->mp_in.get());
+            precond_apply_p32(p, p->mp_in.get(), y, stop, cs);
+            k_dot<C, T, float2><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, vol, v0, v1, y, part, S, 1);
+        }
+    }
+    if (!mp) {
+        // without a preconditioner z = v
+        C *in = p ? W.in.get() : z;
+        k_step<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, S, q, v0, v1, w0, w1, z, in);
+        if (p) precond_apply_any<T>(p, in, z, stop, cs);
+        k_dot<C, T, C><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, vol, v0, v1, z, part, S, 1);
+    }
+    k_update<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, S, w0, w1, x);
+    k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, cs>>>(n, K, kd, vol, psi, b, x, part, S, gate, 0);
+    GL_LAUNCH_CHECK();
+}
+
+// Adds a WHILE node over `body` behind what `cs` has captured; `body` enqueues one
+// iteration on the stream it is given, ending with the gate.
+template <typename F>
+static void enqueue_loop(cudaStream_t cs, cudaStream_t body_stream, MinresDev *S, F &&body) {
+    cudaStreamCaptureStatus cst;
+    cudaGraph_t cg = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t ndeps = 0;
+    GL_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
+    LoopGate gate{{}, 1};
+    GL_CUDA(cudaGraphConditionalHandleCreate(&gate.h, cg, 0, cudaGraphCondAssignDefault));
+    k_loop_begin<<<1, 1, 0, cs>>>(gate.h, S);
+    GL_LAUNCH_CHECK();
+    GL_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
+    cudaGraphNodeParams cp = {};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = gate.h;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t wnode;
+    GL_CUDA(cudaGraphAddNode(&wnode, cg, deps, nullptr, ndeps, &cp));
+    cudaGraph_t graph = cp.conditional.phGraph_out[0];
+    GL_CUDA(cudaStreamUpdateCaptureDependencies(cs, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
+    GL_CUDA(cudaStreamBeginCaptureToGraph(body_stream, graph, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+    try {
+        body(body_stream, gate);
+    } catch (...) {
+        cudaStreamEndCapture(body_stream, &graph);
+        throw;
+    }
+    GL_CUDA(cudaStreamEndCapture(body_stream, &graph));
 }
 
 // Runs MINRES on J x = b with x as the initial guess (overwritten).  use_true:
@@ -931,9 +915,9 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
     MinresDev *S = W.S.get();
     double *part = W.part.get();
     // The device-side loop (the whole solve in one graph: the initial phase, then a
-    // WHILE node over bodies of ITER_UNROLL iterations whose later iterations sit in
-    // IF nodes) whenever no kernel class is being timed (the profiler's event
-    // nodes cannot sit in conditional bodies) and R_inf does not nest its own loop.
+    // WHILE node over one iteration) whenever no kernel class is being timed (the
+    // profiler's event nodes cannot sit in conditional bodies) and R_inf does not nest
+    // its own loop.
     const bool timing_class = profiler().active && !profiler().name.empty();
     const bool loop = device_loop && !timing_class && !(p && p->rinf);
     GraphKey key{m, psi, b, x, p ? p->uid : -1, profiler().generation, m->version, vc32 ? 1 : 0, df ? 1 : 0,
@@ -946,47 +930,17 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
                 const int64_t l0 = pr.launches.load();
                 enqueue_init<T>(m, p, psi, b, x, vc32, df, W, cs);
                 const int64_t l1 = pr.launches.load();
-                cudaStreamCaptureStatus cst;
-                cudaGraph_t cg = nullptr;
-                const cudaGraphNode_t *deps = nullptr;
-                size_t ndeps = 0;
-                GL_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
-                Gates g{};
-                g.n = ITER_UNROLL;
-                GL_CUDA(cudaGraphConditionalHandleCreate(&g.h[0], cg, 0, cudaGraphCondAssignDefault));
-                note_launch();
-                k_loop_begin<<<1, 1, 0, cs>>>(g.h[0], S);
-                GL_LAUNCH_CHECK();
-                GL_CUDA(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
-                cudaGraphNodeParams cp = {};
-                cp.type = cudaGraphNodeTypeConditional;
-                cp.conditional.handle = g.h[0];
-                cp.conditional.type = cudaGraphCondTypeWhile;
-                cp.conditional.size = 1;
-                cudaGraphNode_t wnode;
-                GL_CUDA(cudaGraphAddNode(&wnode, cg, deps, nullptr, ndeps, &cp));
-                cudaGraph_t body = cp.conditional.phGraph_out[0];
-                GL_CUDA(cudaStreamUpdateCaptureDependencies(cs, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-                for (int k = 1; k < ITER_UNROLL; ++k)
-                    GL_CUDA(cudaGraphConditionalHandleCreate(&g.h[k], body, 0, cudaGraphCondAssignDefault));
-                GL_CUDA(cudaStreamBeginCaptureToGraph(W.cap_body, body, nullptr, nullptr, 0,
-                                                      cudaStreamCaptureModeThreadLocal));
-                const int64_t l2 = pr.launches.load();
-                try {
-                    enqueue_body<T>(m, p, psi, b, x, vc32, df, W, W.cap_body, &g, W.cap_if);
-                    k_loop_next<<<1, 1, 0, W.cap_body>>>(g.h[0], S);
-                    GL_LAUNCH_CHECK();
-                } catch (...) {
-                    cudaStreamEndCapture(W.cap_body, &body);
-                    throw;
-                }
-                GL_CUDA(cudaStreamEndCapture(W.cap_body, &body));
+                enqueue_loop(cs, W.cap_body, S, [&](cudaStream_t bs, const LoopGate &gate) {
+                    enqueue_iteration<T>(m, p, psi, b, x, vc32, df, W, bs, gate);
+                });
                 W.loop_init_launches = l1 - l0 + 1;  // + k_loop_begin
-                W.loop_iter_launches = (pr.launches.load() - l2) / ITER_UNROLL;
+                W.loop_iter_launches = pr.launches.load() - l1;
             });
         } else {
             capture(W.init, W.cap, [&](cudaStream_t cs) { enqueue_init<T>(m, p, psi, b, x, vc32, df, W, cs); });
-            capture(W.body, W.cap, [&](cudaStream_t cs) { enqueue_body<T>(m, p, psi, b, x, vc32, df, W, cs); });
+            capture(W.body, W.cap, [&](cudaStream_t cs) {
+                for (int k = 0; k < ITER_UNROLL; ++k) enqueue_iteration<T>(m, p, psi, b, x, vc32, df, W, cs);
+            });
         }
     }
     // Stall test: with the double-FP32 Jacobian the ~48-bit apply limits the true
@@ -1002,7 +956,7 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
         GL_CUDA(cudaMemcpyAsync(&h, S, sizeof(MinresDev), cudaMemcpyDeviceToHost, s));
         GL_CUDA(cudaStreamSynchronize(s));
         // the kernels that ran: the initial phase and one iteration's launches per iteration
-        note_launch((int)(W.loop_init_launches + (int64_t)h.it * W.loop_iter_launches + h.replays));
+        note_launch((int)(W.loop_init_launches + (int64_t)h.it * W.loop_iter_launches));
         GL_REQUIRE(h.status != ST_RUN, GL_ERR_TIMEOUT, "MINRES status word was not updated");
     } else {
     replay(W.init, s);
@@ -1027,7 +981,7 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
     if (use_true) {
         note_launch();
         k_true_resid<C, T><<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, O::K(m), O::kdiag(m), O::vol(m), psi, b, x, part, S,
-                                                              Gates{{}, 0}, 0, 1);
+                                                              LoopGate{{}, 0}, 1);
         GL_LAUNCH_CHECK();
         GL_CUDA(cudaMemcpyAsync(&h, S, sizeof(MinresDev), cudaMemcpyDeviceToHost, s));
         GL_CUDA(cudaStreamSynchronize(s));
@@ -1111,16 +1065,9 @@ static SolveWork &solve_work() {
 // ------------------------------------------------------------------ batched solves
 // Many independent systems J(psi_s) x_s = b_s in ONE CUDA-graph launch: each
 // instance is a branch of the graph (its own buffers and preconditioner), and
-// its MINRES iterations run inside a WHILE conditional node whose condition a
-// kernel sets from the instance's status word, so the whole batch runs on the
-// device without host round trips.  The loop is bounded by a replay count.
-__global__ void k_set_cond(cudaGraphConditionalHandle h, MinresDev *S, int max_replays) {
-    int go = (S->status == ST_RUN) && (S->replays < max_replays);
-    S->replays += 1;
-    if (!go && S->status == ST_RUN) S->status = ST_MAXIT;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-
+// its MINRES iterations run inside a WHILE conditional node whose condition the
+// iteration's last kernel sets from the instance's status word, so the whole batch runs
+// on the device without host round trips.
 struct BatchInst {
     gl_mesh_s *m = nullptr;
     gl_prec_s *p = nullptr;
@@ -1209,36 +1156,14 @@ static void batch_build(gl_batch_s *B, const double2 *const *b, double2 *const *
             // the double-float Jacobian's stall test, as in a single solve
             k_set_params<<<1, 1, 0, si>>>(S, B->o.tol, B->o.maxit, 1, I.df ? 1e-3 : 0.0);
             enqueue_init<double>(I.m, I.p, I.p->psi_p.get(), I.b.get(), I.x.get(), B->vc32, I.df, I.W, si);
-            // the WHILE node: its handle lives in the graph being captured
-            cudaStreamCaptureStatus cst;
-            cudaGraph_t cg = nullptr;
-            const cudaGraphNode_t *deps = nullptr;
-            size_t ndeps = 0;
-            GL_CUDA(cudaStreamGetCaptureInfo(si, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
-            cudaGraphConditionalHandle h;
-            GL_CUDA(cudaGraphConditionalHandleCreate(&h, cg, 1, cudaGraphCondAssignDefault));
-            int max_replays = B->o.maxit / ITER_UNROLL + 2;
-            k_set_cond<<<1, 1, 0, si>>>(h, S, max_replays);
-            GL_LAUNCH_CHECK();
-            GL_CUDA(cudaStreamGetCaptureInfo(si, &cst, nullptr, &cg, &deps, nullptr, &ndeps));
-            cudaGraphNodeParams cp = {};
-            cp.type = cudaGraphNodeTypeConditional;
-            cp.conditional.handle = h;
-            cp.conditional.type = cudaGraphCondTypeWhile;
-            cp.conditional.size = 1;
-            cudaGraphNode_t wnode;
-            GL_CUDA(cudaGraphAddNode(&wnode, cg, deps, nullptr, ndeps, &cp));
-            cudaGraph_t body = cp.conditional.phGraph_out[0];
-            GL_CUDA(cudaStreamUpdateCaptureDependencies(si, &wnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-            GL_CUDA(cudaStreamBeginCaptureToGraph(B->sb, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-            enqueue_body<double>(I.m, I.p, I.p->psi_p.get(), I.b.get(), I.x.get(), B->vc32, I.df, I.W, B->sb);
-            k_set_cond<<<1, 1, 0, B->sb>>>(h, S, max_replays);
-            GL_LAUNCH_CHECK();
-            GL_CUDA(cudaStreamEndCapture(B->sb, &body));
+            enqueue_loop(si, B->sb, S, [&](cudaStream_t bs, const LoopGate &gate) {
+                enqueue_iteration<double>(I.m, I.p, I.p->psi_p.get(), I.b.get(), I.x.get(), B->vc32, I.df, I.W, bs,
+                                          gate);
+            });
             // final FP64 true residual, back to node order
             k_true_resid<double2, double><<<RED_BLOCKS, RED_THREADS, 0, si>>>(
                 n, I.m->K.view(), I.m->kdiag.get(), I.m->volp.get(), I.p->psi_p.get(), I.b.get(), I.x.get(),
-                I.W.part.get(), S, Gates{{}, 0}, 0, 1);
+                I.W.part.get(), S, LoopGate{{}, 0}, 1);
             GL_LAUNCH_CHECK();
             permute_out(n, I.m->perm.get(), I.x.get(), x[i], si);
             GL_CUDA(cudaEventRecord(B->ev[i + 1], si));
