@@ -19,7 +19,8 @@
 //   * activations h^l are n x 64 BF16, node-major (128 B per node);
 //   * the dense layers are tcgen05 MMAs (kind::f16, BF16 operands, FP32
 //     accumulators in tensor memory), one 128-node tile per MMA group.  Operands
-//     are staged in shared memory as K-major tiles of 8-row x 16-byte core
+//     are staged in shared memory as K-major tiles: the forward activations as rows of
+//     128 bytes with swizzled chunks (SWIZZLE_128B), the others of 8-row x 16-byte core
 //     matrices without swizzle: leading-dimension offset 128 B (next core matrix
 //     along K), stride-dimension offset 16 K bytes (next 8-row group);
 //   * forward: one persistent kernel per layer builds [h, S h] for its tile
@@ -51,7 +52,6 @@ constexpr int WSZ = CH * CIN;        // one W^l
 constexpr int NPARAM = NL * WSZ + 2 * CH;
 constexpr int TILE = 128;            // nodes per MMA tile (= M)
 constexpr int THREADS = 128;         // one thread per node row of the tile
-constexpr int FWD_SMEM = TILE * CIN * 2 + CH * CIN * 2;            // a tile + W image
 constexpr int BWD_SMEM = TILE * CH * 2 + CIN * CH * 2 + CIN * TILE * 2 + CH * TILE * 2;
 constexpr int DU_BLOCKS = 2 * NUM_SMS_HINT;
 constexpr long long WAIT_CYCLES = 4000000000LL;   // about 2 s at the maximum SM clock
@@ -73,6 +73,13 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
            ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
 
+// the same for rows of 64 BF16 (128 bytes) whose 16-byte chunks are XOR-swizzled by the
+// row within groups of eight rows (SWIZZLE_128B): 1024 bytes from group to group
+__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
 // instruction descriptor of kind::f16: BF16 A and B, FP32 D, both K-major
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -90,17 +97,21 @@ __device__ __forceinline__ void mma_commit(uint64_t *mbar) {
 }
 
 // wait on an mbarrier phase for at most WAIT_CYCLES; returns false if that ran out
-__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity) {
-    uint32_t done = 0;
-    const long long t0 = clock64();
-    while (!done) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(smem_u32(mbar)), "r"(parity));
-        if (!done && clock64() - t0 > WAIT_CYCLES) break;
-    }
+__device__ __forceinline__ bool mbar_try(uint64_t *mbar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(smem_u32(mbar)), "r"(parity)
+        : "memory");
     return done != 0;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity) {
+    if (mbar_try(mbar, parity)) return true;
+    const long long t0 = clock64();
+    while (!mbar_try(mbar, parity))
+        if (clock64() - t0 > WAIT_CYCLES) return false;
+    return true;
 }
 
 // 16 consecutive FP32 columns of this thread's TMEM lane
@@ -128,6 +139,22 @@ __device__ __forceinline__ void tmem_free(uint32_t base, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols));
 }
 
+__device__ __forceinline__ void mbar_init_n(uint64_t *mbar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(mbar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_tx(uint64_t *mbar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(mbar)), "r"(bytes) : "memory");
+}
+// global -> shared, both 16-byte aligned, a multiple of 16 bytes
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+                 : "memory");
+}
 __device__ __forceinline__ void mbar_init(uint64_t *mbar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
     asm volatile("fence.mbarrier_init.release.cluster;");
@@ -184,8 +211,6 @@ __device__ __forceinline__ void aggregate_row(const SellView<float2> &K, const f
     for (int c = 0; c < CH; ++c) acc[c] *= sc;
 }
 
-constexpr int WMAX = 8;   // sliced-ELL entries per row staged in shared memory
-
 // accumulate K_pq h_q over one 16-byte chunk (four complex pairs) of h_q
 __device__ __forceinline__ void cacc4(float *acc, float2 v, uint4 r) {
     float f[8];
@@ -197,52 +222,22 @@ __device__ __forceinline__ void cacc4(float *acc, float2 v, uint4 r) {
     }
 }
 
-// (S h) for channels 8 j .. 8 j + 7 of two nodes rA, rB of the tile, with their
-// sliced-ELL entries staged in shared memory (entries beyond WMAX, which the
-// lattice meshes do not have, are read from global memory).  All neighbour
-// chunks of both nodes are requested before any is used.
-__device__ __forceinline__ void aggregate_pair(const SellView<float2> &K, const float *__restrict__ kdiag,
-                                               const uint4 *__restrict__ H, const int32_t *sCol,
-                                               const float2 *sVal, const int *sWid, int64_t base, int rA, int rB,
-                                               int j, int64_t n, uint4 &outA, uint4 &outB) {
-    float accA[8], accB[8];
+// The same sums two channel pairs at a time in packed FP32 arithmetic, rounding for rounding
+// what cacc4 compiles to: acc + fma(v.x, re, -(v.y im)) and acc + fma(v.x, im, v.y re).
+// Twelve packed instructions in place of 24; re/im of pairs (0, 1) and (2, 3).
+struct Acc4 {
+    float2 re[2], im[2];
+};
+__device__ __forceinline__ void cacc4_packed(Acc4 &acc, float2 v, uint4 r) {
+    const float2 vx = make_float2(v.x, v.x), vy = make_float2(v.y, v.y), ny = make_float2(-v.y, -v.y);
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-    for (int i = 0; i < 8; ++i) accA[i] = accB[i] = 0.f;
-    const int wA = (base + rA < n) ? sWid[rA >> 5] : 0, wB = (base + rB < n) ? sWid[rB >> 5] : 0;
-    uint4 ra[WMAX], rb[WMAX];
-#pragma unroll
-    for (int k = 0; k < WMAX; ++k) {
-        if (k < wA) ra[k] = __ldg(H + (int64_t)sCol[k * TILE + rA] * 8 + j);
-        if (k < wB) rb[k] = __ldg(H + (int64_t)sCol[k * TILE + rB] * 8 + j);
+    for (int t = 0; t < 2; ++t) {
+        const float2 re = make_float2(__uint_as_float(w[2 * t] << 16), __uint_as_float(w[2 * t + 1] << 16));
+        const float2 im = make_float2(__uint_as_float(w[2 * t] & 0xffff0000u), __uint_as_float(w[2 * t + 1] & 0xffff0000u));
+        acc.re[t] = __fadd2_rn(acc.re[t], __ffma2_rn(vx, re, __fmul2_rn(ny, im)));
+        acc.im[t] = __fadd2_rn(acc.im[t], __ffma2_rn(vx, im, __fmul2_rn(vy, re)));
     }
-#pragma unroll
-    for (int k = 0; k < WMAX; ++k) {
-        if (k < wA) cacc4(accA, sVal[k * TILE + rA], ra[k]);
-        if (k < wB) cacc4(accB, sVal[k * TILE + rB], rb[k]);
-    }
-    // rows wider than WMAX (not produced by the lattice meshes)
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        const int r = h ? rB : rA;
-        const int64_t p = base + r;
-        if (p >= n) continue;
-        const int64_t sl = p >> 5;
-        const int64_t beg = K.sptr[sl];
-        const int w = (int)((K.sptr[sl + 1] - beg) >> 5);
-        for (int k = WMAX; k < w; ++k) {
-            const int64_t e = beg + (int64_t)k * SELL_C + (p & 31);
-            cacc4(h ? accB : accA, K.val[e], __ldg(H + (int64_t)K.col[e] * 8 + j));
-        }
-    }
-    const float sa = base + rA < n ? -1.f / kdiag[base + rA] : 0.f;
-    const float sb = base + rB < n ? -1.f / kdiag[base + rB] : 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        accA[i] *= sa;
-        accB[i] *= sb;
-    }
-    outA = pack8(accA);
-    outB = pack8(accB);
 }
 
 // ------------------------------------------------------------------ small kernels
@@ -339,7 +334,7 @@ __global__ void k_hint_add(int64_t n, const double *__restrict__ hs, const doubl
 // (the hint a^ = a / ||a||_D as the complex channel pair (6, 7), zero without one)
 __global__ void k_features(int64_t n, const double2 *__restrict__ b, const double2 *__restrict__ psi,
                            const double *__restrict__ bn, const double2 *__restrict__ hint,
-                           const double *__restrict__ hs, uint4 *__restrict__ H0) {
+                           const double *__restrict__ hs, uint4 *__restrict__ H0, int compact) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= n) return;
     double inv = bn[1];
@@ -353,6 +348,11 @@ __global__ void k_features(int64_t n, const double2 *__restrict__ b, const doubl
     }
     float z[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float last[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 1.f};
+    if (compact) {  // only the chunks that hold anything
+        H0[2 * p] = pack8(f);
+        H0[2 * p + 1] = pack8(last);
+        return;
+    }
     uint4 *row = H0 + p * 8;
     row[0] = pack8(f);
 #pragma unroll
@@ -368,7 +368,7 @@ struct FwdArgs {
     int64_t ntiles;
     SellView<float2> K;
     const float *kdiag;
-    const uint4 *Hin;        // n x 8 uint4
+    const uint4 *Hin;        // n x 8 uint4 (compact: n x 2, the first and the last chunk)
     uint4 *Hout;             // n x 8 uint4 (hidden layers, and h^4 when training)
     const uint4 *Wimg;       // 64 x 128 BF16 operand image (1024 uint4)
     const float *U;          // 2 x 64 head (last layer)
@@ -378,122 +378,308 @@ struct FwdArgs {
     int *err;
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(THREADS) k_fwd(FwdArgs a) {
+// One layer.  Bound by the gathers: six neighbour rows of 128 bytes a node through L1 (1.6 GB
+// at 128^3 nodes, half of it from L2) around 0.7 GB of HBM traffic; the MMAs take a few
+// percent of the time.  Eight threads a node read one 16-byte chunk of every row each, so
+// the registers decide how many rows are in flight: one CTA per SM holds as many gathering
+// warps as its registers allow with two nodes a thread requested ahead, and nothing else
+// runs in those warps:
+//   * one warp brings the K entries, slice widths and -1 / K_pp of the tiles to come into
+//     shared memory (bulk copies; the offsets and diagonals they need are requested four
+//     tiles earlier, or their latency alone is 3 us a tile);
+//   * the gathering warps build operand tiles: their own rows by cp.async, S h from the
+//     neighbours' chunks, two channel pairs at a time in packed FP32.  Rows of 64 channels
+//     are 128 bytes with XOR-swizzled chunks (SWIZZLE_128B operands), so that a node's
+//     eight threads write different banks (eight-way conflicts without);
+//   * four warps take the finished tiles: one thread issues the MMAs of the next one into the
+//     other of two accumulators, then all take the current accumulator through relu (and
+//     head) to global memory.
+// Fewer operand tiles leave more L1 to the gathers: two take 365 us where three take 377
+// (K entries of four tiles ahead instead of three: 392).  The first layer's rows hold two
+// chunks that are not zero; only these are stored and gathered (COMPACT), and there the
+// third operand tile pays: 163 us against 190.
+// Every wait is bounded; a warp whose wait runs out leaves, the others follow.
+// 128^3 nodes: 365 us a layer, 163 the first, 357 the last (588 each with three CTAs an SM
+// going through staging, gathers, MMA and epilogue in turn); 63^3 nodes: 47 us (70).
+constexpr int FWD_KSTAGES = 3;                         // tiles whose K entries are in shared memory
+constexpr int FWD_K = 6;                               // staged K entries a row (further ones are read where used)
+constexpr int FWD_TILE_BYTES = TILE * CIN * 2;
+// gathering warps; + four epilogue warps + one for the K entries
+__host__ __device__ constexpr int fwd_gw(bool compact) { return compact ? 8 : 16; }
+__host__ __device__ constexpr int fwd_stages(bool compact) { return compact ? 3 : 2; }
+__host__ __device__ constexpr int fwd_smem(bool compact) {  // operand tiles, W image, output rows, K entries
+    return fwd_stages(compact) * FWD_TILE_BYTES + CH * CIN * 2 + TILE * CH * 2 + FWD_KSTAGES * FWD_K * TILE * 12;
+}
+__host__ __device__ constexpr int fwd_threads(bool compact) { return 32 * (fwd_gw(compact) + 5); }
+
+// 16 bytes global -> shared behind the thread's back (zeros if !ok); not through L1
+__device__ __forceinline__ void copy16(void *dst, const void *src, bool ok) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <int MODE, bool COMPACT>
+__global__ void __launch_bounds__(fwd_threads(COMPACT), 1) k_fwd(FwdArgs a) {
+    constexpr int GW = fwd_gw(COMPACT), NTHREADS = fwd_threads(COMPACT), STAGES = fwd_stages(COMPACT);
     extern __shared__ __align__(1024) unsigned char smem[];
-    __nv_bfloat16 *sA = reinterpret_cast<__nv_bfloat16 *>(smem);          // 128 x 128
-    uint4 *sW = reinterpret_cast<uint4 *>(smem + TILE * CIN * 2);          // 64 x 128 image
-    __shared__ int32_t sCol[WMAX * TILE];
-    __shared__ float2 sVal[WMAX * TILE];
-    __shared__ int sWid[TILE / SELL_C];
-    __shared__ __align__(8) uint64_t mbar;
+    unsigned char *sA = smem;                                                        // STAGES x [h, S h] x 128 x 64
+    uint4 *sW = reinterpret_cast<uint4 *>(smem + STAGES * FWD_TILE_BYTES);           // 64 x 128 image
+    uint4 *sOut = sW + CH * CIN / 8;                                                 // 128 rows of 8 chunks
+    float2 *sVal = reinterpret_cast<float2 *>(sOut + TILE * CH / 8);                 // FWD_KSTAGES x 4 slices x FWD_K x 32
+    int32_t *sCol = reinterpret_cast<int32_t *>(sVal + FWD_KSTAGES * FWD_K * TILE);
+    __shared__ float sSc[FWD_KSTAGES][TILE];             // -1 / K_pp
+    __shared__ int sWid[FWD_KSTAGES][TILE / SELL_C];     // entries a row of each slice
+    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2], kfull[FWD_KSTAGES],
+        kempty[FWD_KSTAGES];
     __shared__ uint32_t tslot;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    for (int i = tid; i < CH * CIN / 8; i += THREADS) sW[i] = a.Wimg[i];
-    if (warp == 0) tmem_alloc(&tslot, CH);
-    if (tid == 0) mbar_init(&mbar);
+    __shared__ float sU[2 * CH];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < CH * CIN / 8; i += NTHREADS) sW[i] = a.Wimg[i];
+    if (COMPACT)  // the chunks that are not stored are zero in every tile
+        for (int i = tid; i < STAGES * FWD_TILE_BYTES / 16; i += NTHREADS) reinterpret_cast<uint4 *>(sA)[i] = zero;
+    if (MODE != FWD_HIDDEN && tid < 2 * CH) sU[tid] = a.U[tid];
+    if (warp == GW) tmem_alloc(&tslot, 2 * CH);
+    if (tid == 0) {
+        for (int i = 0; i < STAGES; ++i) {
+            mbar_init_n(&full[i], GW);
+            mbar_init_n(&empty[i], 1);
+        }
+        for (int i = 0; i < FWD_KSTAGES; ++i) {
+            mbar_init_n(&kfull[i], 32);
+            mbar_init_n(&kempty[i], GW);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init_n(&tfull[i], 1);
+            mbar_init_n(&tempty[i], 4);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    proxy_fence();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tslot;
-    const uint32_t idesc = idesc_bf16(TILE, CH);
-    uint32_t phase = 0;
     bool failed = false;
-    __shared__ float sU[2 * CH];
-    if (MODE != FWD_HIDDEN) {
-        sU[tid] = a.U[tid];
-        __syncthreads();
-    }
-    for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-        const int64_t p = t * TILE + tid;
-        // ---- stage the tile's sliced-ELL rows (thread tid: node tid of the tile)
-        const int64_t base = t * TILE;
-        {
-            const int64_t sl = (base >> 5) + (tid >> 5);
-            int w = 0;
-            int64_t beg = 0;
-            if (sl * SELL_C < a.n) {
-                beg = a.K.sptr[sl];
-                w = (int)((a.K.sptr[sl + 1] - beg) >> 5);
-            }
-            if ((tid & 31) == 0) sWid[tid >> 5] = w;
+    if (warp < GW) {
+        // ---- operand tiles [h, S h] in BF16
+        constexpr int NI = COMPACT ? 1 : 2;     // nodes of a tile for each thread
+        constexpr int RS = COMPACT ? 2 : 8;     // chunks of a stored row
+        const int jc = COMPACT ? (lane & 1) : (lane & 7), j = COMPACT ? 7 * jc : jc;
+        const int r0 = COMPACT ? warp * 16 + (lane >> 1) : warp * 4 + (lane >> 3);
+        const uint4 *__restrict__ Hj = a.Hin + jc;
+        int st = 0, ks = 0;
+        uint32_t ph = 1, kph = 0;  // (the first round of the operand tiles is empty already)
+        // request a chunk of a node's own row (into the operand tile) and of its neighbours'
+        auto request = [&](uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
+            const int64_t p = t * TILE + r;
+            const bool ok = p < a.n;
+            copy16(sA + stage * FWD_TILE_BYTES + r * 128 + ((j ^ (r & 7)) << 4), ok ? Hj + p * RS : Hj, ok);
+            if (!ok) return;
+            const int w = sWid[kst][r >> 5];
+            const int32_t *c = sCol + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
 #pragma unroll
-            for (int k = 0; k < WMAX; ++k) {
-                if (k < w) {
-                    const int64_t e = beg + (int64_t)k * SELL_C + (tid & 31);
-                    sCol[k * TILE + tid] = a.K.col[e];
-                    sVal[k * TILE + tid] = a.K.val[e];
+            for (int e = 0; e < FWD_K; ++e)
+                if (e < w) nb[e] = __ldg(Hj + (int64_t)c[e * SELL_C] * RS);
+        };
+        // the chunk of S h
+        auto finish = [&](const uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
+            const int64_t p = t * TILE + r;
+            uint4 out = zero;
+            if (p < a.n) {
+                Acc4 acc;
+                acc.re[0] = acc.re[1] = acc.im[0] = acc.im[1] = make_float2(0.f, 0.f);
+                const int w = sWid[kst][r >> 5];
+                const float2 *v = sVal + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
+#pragma unroll
+                for (int e = 0; e < FWD_K; ++e)
+                    if (e < w) cacc4_packed(acc, v[e * SELL_C], nb[e]);
+                // rows wider than FWD_K (not produced by the lattice meshes)
+                for (int e = FWD_K; e < w; ++e) {
+                    const int64_t q = a.K.sptr[p >> 5] + (int64_t)e * SELL_C + (p & 31);
+                    cacc4_packed(acc, a.K.val[q], __ldg(Hj + (int64_t)a.K.col[q] * RS));
                 }
+                const float sc = sSc[kst][r];
+                const float f[8] = {acc.re[0].x * sc, acc.im[0].x * sc, acc.re[0].y * sc, acc.im[0].y * sc,
+                                    acc.re[1].x * sc, acc.im[1].x * sc, acc.re[1].y * sc, acc.im[1].y * sc};
+                out = pack8(f);
+            }
+            *reinterpret_cast<uint4 *>(sA + stage * FWD_TILE_BYTES + (TILE + r) * 128 + ((j ^ (r & 7)) << 4)) = out;
+        };
+        uint4 A[FWD_K], B[FWD_K];
+        bool more = blockIdx.x < a.ntiles;
+        if (more) {
+            failed = !__all_sync(0xffffffffu, mbar_wait(&kfull[0], 0));
+            if (!failed) request(A, blockIdx.x, 0, r0, 0);
+            if (NI == 1) copy_commit();
+        }
+        for (int64_t t = blockIdx.x; more && !failed; t += gridDim.x) {
+            more = t + gridDim.x < a.ntiles;
+            const int kn = ks + 1 == FWD_KSTAGES ? 0 : ks + 1, sn = st + 1 == STAGES ? 0 : st + 1;
+            const uint32_t kpn = kn ? kph : kph ^ 1, pn = sn ? ph : ph ^ 1;
+            if (NI == 2) {
+                request(B, t, ks, r0 + TILE / 2, st);
+                copy_commit();
+                finish(A, t, ks, r0, st);
+            }
+            if (more && !__all_sync(0xffffffffu, mbar_wait(&kfull[kn], kpn) && mbar_wait(&empty[sn], pn))) {
+                failed = true;
+                break;
+            }
+            if (NI == 2) {
+                if (more) request(A, t + gridDim.x, kn, r0, sn);
+                finish(B, t, ks, r0 + TILE / 2, st);
+                copy_wait<0>();
+            } else {
+                if (more) request(B, t + gridDim.x, kn, r0, sn);
+                copy_commit();
+                finish(A, t, ks, r0, st);
+                copy_wait<1>();
+#pragma unroll
+                for (int e = 0; e < FWD_K; ++e) A[e] = B[e];
+            }
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&full[st]);
+                mbar_arrive(&kempty[ks]);
+            }
+            st = sn;
+            ph = pn;
+            ks = kn;
+            kph = kpn;
+        }
+        copy_wait<0>();
+    } else if (warp == GW + 4) {
+        // ---- K entries of the tiles to come; slice offsets and diagonals are requested
+        // KPF tiles ahead of that
+        constexpr int KPF = 4, NS = TILE / SELL_C;
+        int64_t s0[KPF], s1[KPF];
+        float kd[KPF][NS];
+        auto fetch = [&](int u, int64_t t) {
+            const int64_t sl = t * NS + lane;
+            s0[u] = s1[u] = 0;
+            if (lane < NS && sl * SELL_C < a.n) {
+                s0[u] = __ldg(a.K.sptr + sl);
+                s1[u] = __ldg(a.K.sptr + sl + 1);
+            }
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                const int64_t p = t * TILE + SELL_C * q + lane;
+                kd[u][q] = p < a.n ? __ldg(a.kdiag + p) : 1.f;
+            }
+        };
+#pragma unroll
+        for (int u = 0; u < KPF; ++u) fetch(u, blockIdx.x + (int64_t)u * gridDim.x);
+        int i = 0, ks = 0;
+        uint32_t kph = 1;
+        for (int64_t t = blockIdx.x; t < a.ntiles && !failed;) {
+#pragma unroll
+            for (int u = 0; u < KPF; ++u) {
+                if (t >= a.ntiles || failed) break;
+                failed = !__all_sync(0xffffffffu, mbar_wait(&kempty[ks], kph));
+                if (failed) break;
+#pragma unroll
+                for (int q = 0; q < NS; ++q) sSc[ks][SELL_C * q + lane] = -1.f / kd[u][q];
+                if (lane < NS) {
+                    const int w = (int)((s1[u] - s0[u]) / SELL_C);
+                    const uint32_t ne = (uint32_t)min(w, FWD_K) * SELL_C;
+                    const int dst = (ks * NS + lane) * (FWD_K * SELL_C);
+                    sWid[ks][lane] = w;
+                    mbar_arrive_tx(&kfull[ks], ne * 12);
+                    if (ne) {
+                        bulk_load(sCol + dst, a.K.col + s0[u], ne * 4, &kfull[ks]);
+                        bulk_load(sVal + dst, a.K.val + s0[u], ne * 8, &kfull[ks]);
+                    }
+                } else {
+                    mbar_arrive(&kfull[ks]);
+                }
+                fetch(u, t + (int64_t)KPF * gridDim.x);
+                t += gridDim.x;
+                ++i;
+                if (++ks == FWD_KSTAGES) ks = 0, kph ^= 1;
             }
         }
-        __syncthreads();
-        // ---- operand rows [h, S h] in BF16: eight threads per node, one 16-byte chunk each
-        uint4 *rowA = reinterpret_cast<uint4 *>(sA);
-        {
-            const int j = tid & 7;
-#pragma unroll 1
-            for (int pass = 0; pass < TILE / 32; ++pass) {
-                const int rA = pass * 32 + (tid >> 3), rB = rA + 16;
-                uint4 hA = make_uint4(0, 0, 0, 0), hB = make_uint4(0, 0, 0, 0), sA4, sB4;
-                if (base + rA < a.n) hA = __ldg(a.Hin + (base + rA) * 8 + j);
-                if (base + rB < a.n) hB = __ldg(a.Hin + (base + rB) * 8 + j);
-                aggregate_pair(a.K, a.kdiag, a.Hin, sCol, sVal, sWid, base, rA, rB, j, a.n, sA4, sB4);
-                rowA[cm_off(rA, 8 * j, CIN) >> 3] = hA;
-                rowA[cm_off(rA, CH + 8 * j, CIN) >> 3] = sA4;
-                rowA[cm_off(rB, 8 * j, CIN) >> 3] = hB;
-                rowA[cm_off(rB, CH + 8 * j, CIN) >> 3] = sB4;
-            }
-        }
-        proxy_fence();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) {
-            uint32_t a0 = smem_u32(sA), b0 = smem_u32(sW);
+        // no copy may be in flight when the block ends
+        for (int q = max(0, i - FWD_KSTAGES); q < i; ++q) mbar_wait(&kfull[q % FWD_KSTAGES], (q / FWD_KSTAGES) & 1);
+    } else {
+        // ---- MMAs (one thread) and epilogue: warp quarter's 32 rows of the 128 x 64
+        // accumulator, one a thread
+        const int quarter = warp - GW;
+        const int r = quarter * 32 + lane;
+        const uint32_t idesc = idesc_bf16(TILE, CH);
+        uint4 *stage = sOut + quarter * 32 * 8;
+        int st = 0;
+        uint32_t ph = 0;
+        // the MMAs of the CTA's i-th tile, once it is built and its accumulator read out
+        auto issue = [&](int i) {
+            const int buf = i & 1;
+            if (!mbar_wait(&full[st], ph) || !mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1)) return false;
+            // the tile's generic writes, ordered before this thread by the barrier, before the
+            // MMA's reads (a fence in the gathering warps would wait for their rows in flight)
+            proxy_fence();
+            tc_fence_after();
+            const uint32_t a0 = smem_u32(sA + st * FWD_TILE_BYTES), b0 = smem_u32(sW);
 #pragma unroll
             for (int ks = 0; ks < CIN / 16; ++ks)
-                mma_bf16(tmem, sdesc(a0 + ks * 256, 128, CIN * 16), sdesc(b0 + ks * 256, 128, CIN * 16), idesc,
-                         ks > 0);
-            mma_commit(&mbar);
-        }
-        const bool done = mbar_wait(&mbar, phase);
-        if (__syncthreads_or(!done)) {
-            failed = true;
-            break;
-        }
-        phase ^= 1;
-        tc_fence_after();
-        // ---- epilogue: row tid of the 128 x 64 accumulator
-        float h[CH];
-        const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll
-        for (int c = 0; c < CH; c += 16) tmem_ld16(lane_base + c, h + c);
-        tc_fence_before();
-        if (p < a.n) {
-#pragma unroll
-            for (int c = 0; c < CH; ++c) h[c] = fmaxf(h[c], 0.f);
-            h[CH - 1] = 1.f;
-            uint4 packed[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) packed[j] = pack8(h + 8 * j);
-            if (MODE != FWD_LAST_PREDICT) {
-                // stage the row in shared memory (chunks XOR-swizzled by row) for coalesced stores
-                uint4 *stage = reinterpret_cast<uint4 *>(sA);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) stage[tid * 8 + (j ^ (tid & 7))] = packed[j];
+                mma_bf16(tmem + buf * CH, sdesc_sw128(a0 + (ks >> 2) * (TILE * 128) + (ks & 3) * 32),
+                         sdesc(b0 + ks * 256, 128, CIN * 16), idesc, ks > 0);
+            mma_commit(&empty[st]);
+            mma_commit(&tfull[buf]);
+            if (++st == STAGES) st = 0, ph ^= 1;
+            return true;
+        };
+        const bool issuer = quarter == 0 && lane == 0;
+        if (issuer && blockIdx.x < a.ntiles) failed = !issue(0);
+        int it = 0;
+        for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
+            const int buf = it & 1;
+            if (issuer && !failed && t + gridDim.x < a.ntiles) failed = !issue(it + 1);
+            __syncwarp();
+            if (!__all_sync(0xffffffffu, !failed && mbar_wait(&tfull[buf], (it >> 1) & 1))) {
+                failed = true;
+                break;
             }
-            if (MODE != FWD_HIDDEN) {
-                // head on the stored (BF16-rounded) h^4
-                float y0 = 0.f, y1 = 0.f;
+            tc_fence_after();
+            const uint32_t lane_base = tmem + buf * CH + ((uint32_t)(quarter * 32) << 16);
+            const int64_t p = t * TILE + r;
+            float y0 = 0.f, y1 = 0.f;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float f[8];
-                    unpack8(packed[j], f);
+            for (int c = 0; c < CH; c += 16) {
+                float h[16];
+                tmem_ld16(lane_base + c, h);
+                if (c == CH - 16) {  // the accumulator has been read
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[buf]);
+                }
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        y0 = fmaf(sU[8 * j + i], f[i], y0);
-                        y1 = fmaf(sU[CH + 8 * j + i], f[i], y1);
+                for (int i = 0; i < 16; ++i) h[i] = fmaxf(h[i], 0.f);
+                if (c == CH - 16) h[15] = 1.f;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int ch = (c >> 3) + u;
+                    const uint4 packed = pack8(h + 8 * u);
+                    // the warp's rows through shared memory (chunks XOR-swizzled by row), so
+                    // that its stores are whole lines
+                    if (MODE != FWD_LAST_PREDICT) stage[lane * 8 + (ch ^ (lane & 7))] = packed;
+                    if (MODE != FWD_HIDDEN) {
+                        // head on the stored (BF16-rounded) h^4
+                        float f[8];
+                        unpack8(packed, f);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            y0 = fmaf(sU[8 * ch + i], f[i], y0);
+                            y1 = fmaf(sU[CH + 8 * ch + i], f[i], y1);
+                        }
                     }
                 }
+            }
+            if (MODE != FWD_HIDDEN && p < a.n) {
                 float inv = 1.f / a.kdiag[p];
                 if (MODE == FWD_LAST_TRAIN) {
                     a.xhat[p] = make_float2(y0 * inv, y1 * inv);
@@ -502,22 +688,21 @@ __global__ void __launch_bounds__(THREADS) k_fwd(FwdArgs a) {
                     a.x0[p] = make_double2(s * (double)(y0 * inv), s * (double)(y1 * inv));
                 }
             }
-        }
-        if (MODE != FWD_LAST_PREDICT) {
-            __syncthreads();
-            const uint4 *stage = reinterpret_cast<const uint4 *>(sA);
+            if (MODE != FWD_LAST_PREDICT) {
+                __syncwarp();
 #pragma unroll
-            for (int it = 0; it < 8; ++it) {
-                const int idx = it * THREADS + tid, r = idx >> 3, c = idx & 7;
-                const int64_t node = t * TILE + r;
-                if (node < a.n) a.Hout[node * 8 + c] = stage[r * 8 + (c ^ (r & 7))];
+                for (int i = 0; i < 8; ++i) {
+                    const int idx = i * 32 + lane, rr = idx >> 3, c = idx & 7;
+                    const int64_t node = t * TILE + quarter * 32 + rr;
+                    if (node < a.n) a.Hout[node * 8 + c] = stage[rr * 8 + (c ^ (rr & 7))];
+                }
+                __syncwarp();
             }
         }
-        __syncthreads();
     }
+    if (failed) atomicExch(a.err, 1);
     __syncthreads();
-    if (warp == 0) tmem_free(tmem, CH);
-    if (failed && tid == 0) atomicExch(a.err, 1);
+    if (warp == GW) tmem_free(tmem, 2 * CH);
 }
 
 // ------------------------------------------------------------------ loss and its gradient in x^
@@ -979,16 +1164,14 @@ void ws_reserve(gl_warmstart_s *w, int64_t n) {
 
 void ws_setup_kernels(gl_warmstart_s *w) {
     if (w->fwd_grid) return;
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_HIDDEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM));
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_LAST_TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM));
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_LAST_PREDICT>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM));
+    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_HIDDEN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem(true)));
+    for (const void *fn : {(const void *)k_fwd<FWD_HIDDEN, false>, (const void *)k_fwd<FWD_LAST_TRAIN, false>,
+                           (const void *)k_fwd<FWD_LAST_PREDICT, false>})
+        GL_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem(false)));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
     // ask for the largest shared-memory carveout, or only one CTA fits an SM
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_HIDDEN>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_LAST_TRAIN>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_LAST_PREDICT>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     GL_CUDA(cudaFuncSetAttribute(k_bwd<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
@@ -1009,13 +1192,10 @@ void ws_setup_kernels(gl_warmstart_s *w) {
         int by_smem = smem_sm / (dyn + (int)fa.sharedSizeBytes + 1024);
         return std::max(1, std::min(cap, std::min(by_regs, by_smem)));
     };
-    int f = std::min(per_sm((const void *)k_fwd<FWD_HIDDEN>, FWD_SMEM, 8),
-                     std::min(per_sm((const void *)k_fwd<FWD_LAST_TRAIN>, FWD_SMEM, 8),
-                              per_sm((const void *)k_fwd<FWD_LAST_PREDICT>, FWD_SMEM, 8)));
     int b = std::min(per_sm((const void *)k_bwd<true, true>, BWD_SMEM, 2),
                      std::min(per_sm((const void *)k_bwd<false, true>, BWD_SMEM, 2),
                               per_sm((const void *)k_bwd<false, false>, BWD_SMEM, 2)));
-    w->fwd_grid = f * nsm;
+    w->fwd_grid = nsm;  // one CTA per SM
     w->bwd_grid = b * nsm;
     w->part.alloc(RED_BLOCKS);
     w->bn.alloc(2);
@@ -1055,7 +1235,7 @@ void ws_forward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const dou
     k_bnorm_part<<<RED_BLOCKS, RED_THREADS, 0, s>>>(n, m->volp.get(), b_p, w->part.get());
     k_bnorm_final<<<1, 1024, 0, s>>>(w->part.get(), RED_BLOCKS, w->bn.get());
     k_features<<<grid_for(n, 256), 256, 0, s>>>(n, b_p, psi_p, w->bn.get(), hint_p, w->hsc.get(),
-                                                reinterpret_cast<uint4 *>(Hbuf(w, 0)));
+                                                reinterpret_cast<uint4 *>(Hbuf(w, 0)), train ? 0 : 1);
     GL_LAUNCH_CHECK();
     note_launch(3);
     const int64_t ntiles = (n + TILE - 1) / TILE;
@@ -1082,12 +1262,14 @@ void ws_forward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const dou
         a.x0 = x0_p;
         a.bn = w->bn.get();
         a.err = w->err.get();
-        if (l < NL - 1)
-            k_fwd<FWD_HIDDEN><<<grid, THREADS, FWD_SMEM, s>>>(a);
+        if (l == 0 && !train)
+            k_fwd<FWD_HIDDEN, true><<<grid, fwd_threads(true), fwd_smem(true), s>>>(a);
+        else if (l < NL - 1)
+            k_fwd<FWD_HIDDEN, false><<<grid, fwd_threads(false), fwd_smem(false), s>>>(a);
         else if (train)
-            k_fwd<FWD_LAST_TRAIN><<<grid, THREADS, FWD_SMEM, s>>>(a);
+            k_fwd<FWD_LAST_TRAIN, false><<<grid, fwd_threads(false), fwd_smem(false), s>>>(a);
         else
-            k_fwd<FWD_LAST_PREDICT><<<grid, THREADS, FWD_SMEM, s>>>(a);
+            k_fwd<FWD_LAST_PREDICT, false><<<grid, fwd_threads(false), fwd_smem(false), s>>>(a);
         GL_LAUNCH_CHECK();
     }
 }
