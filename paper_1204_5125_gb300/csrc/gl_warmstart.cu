@@ -19,18 +19,19 @@
 //   * activations h^l are n x 64 BF16, node-major (128 B per node);
 //   * the dense layers are tcgen05 MMAs (kind::f16, BF16 operands, FP32
 //     accumulators in tensor memory), one 128-node tile per MMA group.  Operands
-//     are staged in shared memory as K-major tiles: the forward activations as rows of
-//     128 bytes with swizzled chunks (SWIZZLE_128B), the others of 8-row x 16-byte core
-//     matrices without swizzle: leading-dimension offset 128 B (next core matrix
-//     along K), stride-dimension offset 16 K bytes (next 8-row group);
+//     are staged in shared memory: activations and dz as rows of 128 bytes a node with
+//     swizzled chunks (SWIZZLE_128B), W as K-major tiles of 8-row x 16-byte core matrices
+//     without swizzle: leading-dimension offset 128 B (next core matrix along K),
+//     stride-dimension offset 16 K bytes (next 8-row group);
 //   * forward: one persistent kernel per layer builds [h, S h] for its tile
 //     (gathering the neighbours' BF16 rows), issues 8 MMAs (K = 16 each) into a
 //     128 x 64 FP32 accumulator, and applies relu (and the head on the last layer)
 //     in the epilogue;
 //   * backward: one persistent kernel per layer issues dA = dz W (M = 128 nodes,
 //     N = 128, K = 64) and accumulates dW^T += a^T dz (M = 128 inputs, N = 64,
-//     K = 128 nodes of the tile) in tensor memory across all of its tiles; the
-//     adjoint aggregation S^T and the relu mask follow in a gather kernel;
+//     K = 128 nodes of the tile) in tensor memory across all of its tiles, both from the
+//     same swizzled rows of [h, S h] and dz; the adjoint aggregation S^T and the relu mask
+//     follow in a gather kernel;
 //   * parameters are FP32 masters with Adam moments; BF16 images of each W in
 //     the two shared-memory operand layouts are rebuilt after every update.
 // Every reduction (loss, dW, dU, ||b||) sums per-block partials in a fixed order,
@@ -51,8 +52,6 @@ constexpr int NL = 4;                // layers
 constexpr int WSZ = CH * CIN;        // one W^l
 constexpr int NPARAM = NL * WSZ + 2 * CH;
 constexpr int TILE = 128;            // nodes per MMA tile (= M)
-constexpr int THREADS = 128;         // one thread per node row of the tile
-constexpr int BWD_SMEM = TILE * CH * 2 + CIN * CH * 2 + CIN * TILE * 2 + CH * TILE * 2;
 constexpr int DU_BLOCKS = 2 * NUM_SMS_HINT;
 constexpr long long WAIT_CYCLES = 4000000000LL;   // about 2 s at the maximum SM clock
 
@@ -74,9 +73,10 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t
 }
 
 // the same for rows of 64 BF16 (128 bytes) whose 16-byte chunks are XOR-swizzled by the
-// row within groups of eight rows (SWIZZLE_128B): 1024 bytes from group to group
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+// row within groups of eight rows (SWIZZLE_128B): 1024 bytes from group to group.  Rows
+// may be M or N (K-major) or K (MN-major; lbo: bytes to the next 64 columns of M or N)
+__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo = 16) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
@@ -155,10 +155,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                  "l"(src), "r"(bytes), "r"(smem_u32(mbar))
                  : "memory");
 }
-__device__ __forceinline__ void mbar_init(uint64_t *mbar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-}
 
 // ------------------------------------------------------------------ BF16 row helpers
 // 8 BF16 <-> 8 floats in one 16-byte word
@@ -179,52 +175,9 @@ __device__ __forceinline__ uint4 pack8(const float *f) {
     return u;
 }
 
-// (S h)_p for one node: sum over its K row of K_pq h_q per complex pair, scaled by
-// -1 / K_pp.  Rows of h are 64 BF16 (8 x 16 B).
-__device__ __forceinline__ void aggregate_row(const SellView<float2> &K, const float *__restrict__ kdiag,
-                                              const uint4 *__restrict__ H, int64_t p, float *acc) {
-#pragma unroll
-    for (int c = 0; c < CH; ++c) acc[c] = 0.f;
-    int64_t s = p >> 5;
-    int lane = (int)(p & 31);
-    int64_t beg = K.sptr[s];
-    int w = (int)((K.sptr[s + 1] - beg) >> 5);
-    for (int k = 0; k < w; ++k) {
-        int64_t q = beg + (int64_t)k * SELL_C + lane;
-        float2 kv = K.val[q];
-        if (kv.x == 0.f && kv.y == 0.f) continue;
-        const uint4 *row = H + (int64_t)K.col[q] * 8;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            float f[8];
-            unpack8(__ldg(row + j), f);
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                float re = f[2 * t], im = f[2 * t + 1];
-                acc[8 * j + 2 * t] += kv.x * re - kv.y * im;
-                acc[8 * j + 2 * t + 1] += kv.x * im + kv.y * re;
-            }
-        }
-    }
-    float sc = -1.f / kdiag[p];
-#pragma unroll
-    for (int c = 0; c < CH; ++c) acc[c] *= sc;
-}
-
-// accumulate K_pq h_q over one 16-byte chunk (four complex pairs) of h_q
-__device__ __forceinline__ void cacc4(float *acc, float2 v, uint4 r) {
-    float f[8];
-    unpack8(r, f);
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        acc[2 * t] += v.x * f[2 * t] - v.y * f[2 * t + 1];
-        acc[2 * t + 1] += v.x * f[2 * t + 1] + v.y * f[2 * t];
-    }
-}
-
-// The same sums two channel pairs at a time in packed FP32 arithmetic, rounding for rounding
-// what cacc4 compiles to: acc + fma(v.x, re, -(v.y im)) and acc + fma(v.x, im, v.y re).
-// Twelve packed instructions in place of 24; re/im of pairs (0, 1) and (2, 3).
+// accumulate K_pq h_q over one 16-byte chunk (four complex pairs) of h_q, two pairs at a
+// time in packed FP32 arithmetic: acc + fma(v.x, re, -(v.y im)), acc + fma(v.x, im, v.y re);
+// re/im of pairs (0, 1) and (2, 3).  Twelve instructions where scalar ones are 24.
 struct Acc4 {
     float2 re[2], im[2];
 };
@@ -363,12 +316,17 @@ __global__ void k_features(int64_t n, const double2 *__restrict__ b, const doubl
 // ------------------------------------------------------------------ forward layer
 enum { FWD_HIDDEN = 0, FWD_LAST_TRAIN = 1, FWD_LAST_PREDICT = 2 };
 
-struct FwdArgs {
+// the aggregated features of one layer
+struct TileArgs {
     int64_t n;
     int64_t ntiles;
     SellView<float2> K;
     const float *kdiag;
     const uint4 *Hin;        // n x 8 uint4 (compact: n x 2, the first and the last chunk)
+};
+
+struct FwdArgs {
+    TileArgs t;
     uint4 *Hout;             // n x 8 uint4 (hidden layers, and h^4 when training)
     const uint4 *Wimg;       // 64 x 128 BF16 operand image (1024 uint4)
     const float *U;          // 2 x 64 head (last layer)
@@ -384,8 +342,8 @@ struct FwdArgs {
 // the registers decide how many rows are in flight: one CTA per SM holds as many gathering
 // warps as its registers allow with two nodes a thread requested ahead, and nothing else
 // runs in those warps:
-//   * one warp brings the K entries, slice widths and -1 / K_pp of the tiles to come into
-//     shared memory (bulk copies; the offsets and diagonals they need are requested four
+//   * three warps bring the K entries, slice widths and -1 / K_pp of the tiles to come into
+//     shared memory (bulk copies; the offsets and diagonals they need are requested three
 //     tiles earlier, or their latency alone is 3 us a tile);
 //   * the gathering warps build operand tiles: their own rows by cp.async, S h from the
 //     neighbours' chunks, two channel pairs at a time in packed FP32.  Rows of 64 channels
@@ -394,23 +352,34 @@ struct FwdArgs {
 //   * four warps take the finished tiles: one thread issues the MMAs of the next one into the
 //     other of two accumulators, then all take the current accumulator through relu (and
 //     head) to global memory.
-// Fewer operand tiles leave more L1 to the gathers: two take 365 us where three take 377
-// (K entries of four tiles ahead instead of three: 392).  The first layer's rows hold two
-// chunks that are not zero; only these are stored and gathered (COMPACT), and there the
-// third operand tile pays: 163 us against 190.
+// Two operand tiles leave more L1 to the gathers than three (365 us against 377, before the
+// registers were split as below).  The first layer's rows hold two chunks that are not
+// zero; only these are stored and gathered (COMPACT), and there the third operand tile pays:
+// 160 us against 190.
 // Every wait is bounded; a warp whose wait runs out leaves, the others follow.
-// 128^3 nodes: 365 us a layer, 163 the first, 357 the last (588 each with three CTAs an SM
-// going through staging, gathers, MMA and epilogue in turn); 63^3 nodes: 47 us (70).
-constexpr int FWD_KSTAGES = 3;                         // tiles whose K entries are in shared memory
+// 128^3 nodes: 291 us a layer, 160 the first, 313 the last (588 each with three CTAs an SM
+// going through staging, gathers, MMA and epilogue in turn); 63^3 nodes: 37 us (70).
+constexpr int FWD_KSTAGES = 3;                         // tiles whose K entries are in shared memory (at most 4)
 constexpr int FWD_K = 6;                               // staged K entries a row (further ones are read where used)
 constexpr int FWD_TILE_BYTES = TILE * CIN * 2;
-// gathering warps; + four epilogue warps + one for the K entries
+// gathering warps; + four epilogue warps + four of which FWD_KSTAGES bring K entries
 __host__ __device__ constexpr int fwd_gw(bool compact) { return compact ? 8 : 16; }
 __host__ __device__ constexpr int fwd_stages(bool compact) { return compact ? 3 : 2; }
 __host__ __device__ constexpr int fwd_smem(bool compact) {  // operand tiles, W image, output rows, K entries
     return fwd_stages(compact) * FWD_TILE_BYTES + CH * CIN * 2 + TILE * CH * 2 + FWD_KSTAGES * FWD_K * TILE * 12;
 }
-__host__ __device__ constexpr int fwd_threads(bool compact) { return 32 * (fwd_gw(compact) + 5); }
+__host__ __device__ constexpr int fwd_threads(bool compact) { return 32 * (fwd_gw(compact) + 8); }
+// Of the 80 registers a thread of 24 warps can have, 16 warps' gathers want more and the
+// others need fewer: 16 x 96 + 4 x 64 + 4 x 32 = 24 x 80 (291 us a layer; 365 with 80 for all,
+// where the gathers' buffers spill)
+template <int N>
+__device__ __forceinline__ void regs_raise() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_lower() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
 
 // 16 bytes global -> shared behind the thread's back (zeros if !ok); not through L1
 __device__ __forceinline__ void copy16(void *dst, const void *src, bool ok) {
@@ -421,6 +390,165 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 template <int N>
 __device__ __forceinline__ void copy_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// shared memory of the tile-building warps
+struct TileBufs {
+    unsigned char *tiles;          // operand tiles: h, S h (and dz) of 128 nodes, 128 bytes a row, swizzled
+    float2 *val;                   // FWD_KSTAGES x 4 slices x FWD_K x 32 K entries
+    int32_t *col;
+    float (*sc)[TILE];             // -1 / K_pp
+    int (*wid)[TILE / SELL_C];     // entries a row of each slice
+    uint64_t *full, *empty, *kfull, *kempty;
+};
+
+// the warps that build operand tiles (true: a wait ran out)
+template <bool COMPACT, int GW, int STAGES, int BYTES, bool WITH_DZ>
+__device__ __forceinline__ bool build_tiles(const TileArgs &a, const TileBufs &b, const uint4 *__restrict__ dZ, int warp,
+                                            int lane) {
+    constexpr int NI = COMPACT ? 1 : 2;     // nodes of a tile for each thread
+    constexpr int RS = COMPACT ? 2 : 8;     // chunks of a stored row
+    const int jc = COMPACT ? (lane & 1) : (lane & 7), j = COMPACT ? 7 * jc : jc;
+    const int r0 = COMPACT ? warp * 16 + (lane >> 1) : warp * 4 + (lane >> 3);
+    const uint4 *__restrict__ Hj = a.Hin + jc;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    bool failed = false;
+    int st = 0, ks = 0;
+    uint32_t ph = 1, kph = 0;  // (the first round of the operand tiles is empty already)
+    // request a chunk of a node's own row (into the operand tile) and of its neighbours'
+    auto request = [&](uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
+        const int64_t p = t * TILE + r;
+        const bool ok = p < a.n;
+        copy16(b.tiles + stage * BYTES + r * 128 + ((j ^ (r & 7)) << 4), ok ? Hj + p * RS : Hj, ok);
+        if (WITH_DZ)
+            copy16(b.tiles + stage * BYTES + (2 * TILE + r) * 128 + ((j ^ (r & 7)) << 4), ok ? dZ + p * 8 + j : dZ, ok);
+        if (!ok) return;
+        const int w = b.wid[kst][r >> 5];
+        const int32_t *c = b.col + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
+#pragma unroll
+        for (int e = 0; e < FWD_K; ++e)
+            if (e < w) nb[e] = __ldg(Hj + (int64_t)c[e * SELL_C] * RS);
+    };
+    // the chunk of S h
+    auto finish = [&](const uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
+        const int64_t p = t * TILE + r;
+        uint4 out = zero;
+        if (p < a.n) {
+            Acc4 acc;
+            acc.re[0] = acc.re[1] = acc.im[0] = acc.im[1] = make_float2(0.f, 0.f);
+            const int w = b.wid[kst][r >> 5];
+            const float2 *v = b.val + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
+#pragma unroll
+            for (int e = 0; e < FWD_K; ++e)
+                if (e < w) cacc4_packed(acc, v[e * SELL_C], nb[e]);
+            // rows wider than FWD_K (not produced by the lattice meshes)
+            for (int e = FWD_K; e < w; ++e) {
+                const int64_t q = a.K.sptr[p >> 5] + (int64_t)e * SELL_C + (p & 31);
+                cacc4_packed(acc, a.K.val[q], __ldg(Hj + (int64_t)a.K.col[q] * RS));
+            }
+            const float sc = b.sc[kst][r];
+            const float f[8] = {acc.re[0].x * sc, acc.im[0].x * sc, acc.re[0].y * sc, acc.im[0].y * sc,
+                                acc.re[1].x * sc, acc.im[1].x * sc, acc.re[1].y * sc, acc.im[1].y * sc};
+            out = pack8(f);
+        }
+        *reinterpret_cast<uint4 *>(b.tiles + stage * BYTES + (TILE + r) * 128 + ((j ^ (r & 7)) << 4)) = out;
+    };
+    uint4 A[FWD_K], B[FWD_K];
+    bool more = blockIdx.x < a.ntiles;
+    if (more) {
+        failed = !__all_sync(0xffffffffu, mbar_wait(&b.kfull[0], 0));
+        if (!failed) request(A, blockIdx.x, 0, r0, 0);
+        if (NI == 1) copy_commit();
+    }
+    for (int64_t t = blockIdx.x; more && !failed; t += gridDim.x) {
+        more = t + gridDim.x < a.ntiles;
+        const int kn = ks + 1 == FWD_KSTAGES ? 0 : ks + 1, sn = st + 1 == STAGES ? 0 : st + 1;
+        const uint32_t kpn = kn ? kph : kph ^ 1, pn = sn ? ph : ph ^ 1;
+        if (NI == 2) {
+            request(B, t, ks, r0 + TILE / 2, st);
+            copy_commit();
+            finish(A, t, ks, r0, st);
+        }
+        if (more && !__all_sync(0xffffffffu, mbar_wait(&b.kfull[kn], kpn) && mbar_wait(&b.empty[sn], pn))) {
+            failed = true;
+            break;
+        }
+        if (NI == 2) {
+            if (more) request(A, t + gridDim.x, kn, r0, sn);
+            finish(B, t, ks, r0 + TILE / 2, st);
+            copy_wait<0>();
+        } else {
+            if (more) request(B, t + gridDim.x, kn, r0, sn);
+            copy_commit();
+            finish(A, t, ks, r0, st);
+            copy_wait<1>();
+#pragma unroll
+            for (int e = 0; e < FWD_K; ++e) A[e] = B[e];
+        }
+        __syncwarp();
+        if (lane == 0) {
+            mbar_arrive(&b.full[st]);
+            mbar_arrive(&b.kempty[ks]);
+        }
+        st = sn;
+        ph = pn;
+        ks = kn;
+        kph = kpn;
+    }
+    copy_wait<0>();
+    return failed;
+}
+
+// the warps that bring K entries for them, one for each stage of the ring; slice offsets and
+// diagonals are requested one round ahead
+__device__ __forceinline__ bool stage_entries(const TileArgs &a, const TileBufs &b, int ks, int lane) {
+    constexpr int NS = TILE / SELL_C;
+    const int64_t step = (int64_t)FWD_KSTAGES * gridDim.x;
+    int64_t s0;
+    int w;
+    float kd[NS];
+    auto fetch = [&](int64_t t) {
+        const int64_t sl = t * NS + lane;
+        s0 = 0;
+        w = 0;
+        if (lane < NS && sl * SELL_C < a.n) {
+            s0 = __ldg(a.K.sptr + sl);
+            w = (int)((__ldg(a.K.sptr + sl + 1) - s0) / SELL_C);
+        }
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            const int64_t p = t * TILE + SELL_C * q + lane;
+            kd[q] = p < a.n ? __ldg(a.kdiag + p) : 1.f;
+        }
+    };
+    uint32_t ph = 1;
+    int64_t t = blockIdx.x + (int64_t)ks * gridDim.x;
+    fetch(t);
+    for (; t < a.ntiles; t += step) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&b.kempty[ks], ph))) {
+            mbar_wait(&b.kfull[ks], ph);  // (the round before's)
+            return true;
+        }
+#pragma unroll
+        for (int q = 0; q < NS; ++q) b.sc[ks][SELL_C * q + lane] = -1.f / kd[q];
+        if (lane < NS) {
+            const uint32_t ne = (uint32_t)min(w, FWD_K) * SELL_C;
+            const int dst = (ks * NS + lane) * (FWD_K * SELL_C);
+            b.wid[ks][lane] = w;
+            mbar_arrive_tx(&b.kfull[ks], ne * 12);
+            if (ne) {
+                bulk_load(b.col + dst, a.K.col + s0, ne * 4, &b.kfull[ks]);
+                bulk_load(b.val + dst, a.K.val + s0, ne * 8, &b.kfull[ks]);
+            }
+        } else {
+            mbar_arrive(&b.kfull[ks]);
+        }
+        fetch(t + step);
+        ph ^= 1;
+        // no copy may be in flight when the block ends
+        if (t + step >= a.ntiles) mbar_wait(&b.kfull[ks], ph);
+    }
+    return false;
 }
 
 template <int MODE, bool COMPACT>
@@ -465,148 +593,16 @@ __global__ void __launch_bounds__(fwd_threads(COMPACT), 1) k_fwd(FwdArgs a) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tslot;
+    const TileBufs bufs{sA, sVal, sCol, sSc, sWid, full, empty, kfull, kempty};
     bool failed = false;
     if (warp < GW) {
-        // ---- operand tiles [h, S h] in BF16
-        constexpr int NI = COMPACT ? 1 : 2;     // nodes of a tile for each thread
-        constexpr int RS = COMPACT ? 2 : 8;     // chunks of a stored row
-        const int jc = COMPACT ? (lane & 1) : (lane & 7), j = COMPACT ? 7 * jc : jc;
-        const int r0 = COMPACT ? warp * 16 + (lane >> 1) : warp * 4 + (lane >> 3);
-        const uint4 *__restrict__ Hj = a.Hin + jc;
-        int st = 0, ks = 0;
-        uint32_t ph = 1, kph = 0;  // (the first round of the operand tiles is empty already)
-        // request a chunk of a node's own row (into the operand tile) and of its neighbours'
-        auto request = [&](uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
-            const int64_t p = t * TILE + r;
-            const bool ok = p < a.n;
-            copy16(sA + stage * FWD_TILE_BYTES + r * 128 + ((j ^ (r & 7)) << 4), ok ? Hj + p * RS : Hj, ok);
-            if (!ok) return;
-            const int w = sWid[kst][r >> 5];
-            const int32_t *c = sCol + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
-#pragma unroll
-            for (int e = 0; e < FWD_K; ++e)
-                if (e < w) nb[e] = __ldg(Hj + (int64_t)c[e * SELL_C] * RS);
-        };
-        // the chunk of S h
-        auto finish = [&](const uint4 (&nb)[FWD_K], int64_t t, int kst, int r, int stage) {
-            const int64_t p = t * TILE + r;
-            uint4 out = zero;
-            if (p < a.n) {
-                Acc4 acc;
-                acc.re[0] = acc.re[1] = acc.im[0] = acc.im[1] = make_float2(0.f, 0.f);
-                const int w = sWid[kst][r >> 5];
-                const float2 *v = sVal + (kst * (TILE / SELL_C) + (r >> 5)) * (FWD_K * SELL_C) + (r & 31);
-#pragma unroll
-                for (int e = 0; e < FWD_K; ++e)
-                    if (e < w) cacc4_packed(acc, v[e * SELL_C], nb[e]);
-                // rows wider than FWD_K (not produced by the lattice meshes)
-                for (int e = FWD_K; e < w; ++e) {
-                    const int64_t q = a.K.sptr[p >> 5] + (int64_t)e * SELL_C + (p & 31);
-                    cacc4_packed(acc, a.K.val[q], __ldg(Hj + (int64_t)a.K.col[q] * RS));
-                }
-                const float sc = sSc[kst][r];
-                const float f[8] = {acc.re[0].x * sc, acc.im[0].x * sc, acc.re[0].y * sc, acc.im[0].y * sc,
-                                    acc.re[1].x * sc, acc.im[1].x * sc, acc.re[1].y * sc, acc.im[1].y * sc};
-                out = pack8(f);
-            }
-            *reinterpret_cast<uint4 *>(sA + stage * FWD_TILE_BYTES + (TILE + r) * 128 + ((j ^ (r & 7)) << 4)) = out;
-        };
-        uint4 A[FWD_K], B[FWD_K];
-        bool more = blockIdx.x < a.ntiles;
-        if (more) {
-            failed = !__all_sync(0xffffffffu, mbar_wait(&kfull[0], 0));
-            if (!failed) request(A, blockIdx.x, 0, r0, 0);
-            if (NI == 1) copy_commit();
-        }
-        for (int64_t t = blockIdx.x; more && !failed; t += gridDim.x) {
-            more = t + gridDim.x < a.ntiles;
-            const int kn = ks + 1 == FWD_KSTAGES ? 0 : ks + 1, sn = st + 1 == STAGES ? 0 : st + 1;
-            const uint32_t kpn = kn ? kph : kph ^ 1, pn = sn ? ph : ph ^ 1;
-            if (NI == 2) {
-                request(B, t, ks, r0 + TILE / 2, st);
-                copy_commit();
-                finish(A, t, ks, r0, st);
-            }
-            if (more && !__all_sync(0xffffffffu, mbar_wait(&kfull[kn], kpn) && mbar_wait(&empty[sn], pn))) {
-                failed = true;
-                break;
-            }
-            if (NI == 2) {
-                if (more) request(A, t + gridDim.x, kn, r0, sn);
-                finish(B, t, ks, r0 + TILE / 2, st);
-                copy_wait<0>();
-            } else {
-                if (more) request(B, t + gridDim.x, kn, r0, sn);
-                copy_commit();
-                finish(A, t, ks, r0, st);
-                copy_wait<1>();
-#pragma unroll
-                for (int e = 0; e < FWD_K; ++e) A[e] = B[e];
-            }
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&full[st]);
-                mbar_arrive(&kempty[ks]);
-            }
-            st = sn;
-            ph = pn;
-            ks = kn;
-            kph = kpn;
-        }
-        copy_wait<0>();
-    } else if (warp == GW + 4) {
-        // ---- K entries of the tiles to come; slice offsets and diagonals are requested
-        // KPF tiles ahead of that
-        constexpr int KPF = 4, NS = TILE / SELL_C;
-        int64_t s0[KPF], s1[KPF];
-        float kd[KPF][NS];
-        auto fetch = [&](int u, int64_t t) {
-            const int64_t sl = t * NS + lane;
-            s0[u] = s1[u] = 0;
-            if (lane < NS && sl * SELL_C < a.n) {
-                s0[u] = __ldg(a.K.sptr + sl);
-                s1[u] = __ldg(a.K.sptr + sl + 1);
-            }
-#pragma unroll
-            for (int q = 0; q < NS; ++q) {
-                const int64_t p = t * TILE + SELL_C * q + lane;
-                kd[u][q] = p < a.n ? __ldg(a.kdiag + p) : 1.f;
-            }
-        };
-#pragma unroll
-        for (int u = 0; u < KPF; ++u) fetch(u, blockIdx.x + (int64_t)u * gridDim.x);
-        int i = 0, ks = 0;
-        uint32_t kph = 1;
-        for (int64_t t = blockIdx.x; t < a.ntiles && !failed;) {
-#pragma unroll
-            for (int u = 0; u < KPF; ++u) {
-                if (t >= a.ntiles || failed) break;
-                failed = !__all_sync(0xffffffffu, mbar_wait(&kempty[ks], kph));
-                if (failed) break;
-#pragma unroll
-                for (int q = 0; q < NS; ++q) sSc[ks][SELL_C * q + lane] = -1.f / kd[u][q];
-                if (lane < NS) {
-                    const int w = (int)((s1[u] - s0[u]) / SELL_C);
-                    const uint32_t ne = (uint32_t)min(w, FWD_K) * SELL_C;
-                    const int dst = (ks * NS + lane) * (FWD_K * SELL_C);
-                    sWid[ks][lane] = w;
-                    mbar_arrive_tx(&kfull[ks], ne * 12);
-                    if (ne) {
-                        bulk_load(sCol + dst, a.K.col + s0[u], ne * 4, &kfull[ks]);
-                        bulk_load(sVal + dst, a.K.val + s0[u], ne * 8, &kfull[ks]);
-                    }
-                } else {
-                    mbar_arrive(&kfull[ks]);
-                }
-                fetch(u, t + (int64_t)KPF * gridDim.x);
-                t += gridDim.x;
-                ++i;
-                if (++ks == FWD_KSTAGES) ks = 0, kph ^= 1;
-            }
-        }
-        // no copy may be in flight when the block ends
-        for (int q = max(0, i - FWD_KSTAGES); q < i; ++q) mbar_wait(&kfull[q % FWD_KSTAGES], (q / FWD_KSTAGES) & 1);
+        if (!COMPACT) regs_raise<96>();
+        failed = build_tiles<COMPACT, GW, STAGES, FWD_TILE_BYTES, false>(a.t, bufs, nullptr, warp, lane);
+    } else if (warp >= GW + 4) {
+        if (!COMPACT) regs_lower<32>();
+        if (warp < GW + 4 + FWD_KSTAGES) failed = stage_entries(a.t, bufs, warp - GW - 4, lane);
     } else {
+        if (!COMPACT) regs_lower<64>();
         // ---- MMAs (one thread) and epilogue: warp quarter's 32 rows of the 128 x 64
         // accumulator, one a thread
         const int quarter = warp - GW;
@@ -634,11 +630,11 @@ __global__ void __launch_bounds__(fwd_threads(COMPACT), 1) k_fwd(FwdArgs a) {
             return true;
         };
         const bool issuer = quarter == 0 && lane == 0;
-        if (issuer && blockIdx.x < a.ntiles) failed = !issue(0);
+        if (issuer && blockIdx.x < a.t.ntiles) failed = !issue(0);
         int it = 0;
-        for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++it) {
+        for (int64_t t = blockIdx.x; t < a.t.ntiles; t += gridDim.x, ++it) {
             const int buf = it & 1;
-            if (issuer && !failed && t + gridDim.x < a.ntiles) failed = !issue(it + 1);
+            if (issuer && !failed && t + gridDim.x < a.t.ntiles) failed = !issue(it + 1);
             __syncwarp();
             if (!__all_sync(0xffffffffu, !failed && mbar_wait(&tfull[buf], (it >> 1) & 1))) {
                 failed = true;
@@ -679,8 +675,8 @@ __global__ void __launch_bounds__(fwd_threads(COMPACT), 1) k_fwd(FwdArgs a) {
                     }
                 }
             }
-            if (MODE != FWD_HIDDEN && p < a.n) {
-                float inv = 1.f / a.kdiag[p];
+            if (MODE != FWD_HIDDEN && p < a.t.n) {
+                float inv = 1.f / a.t.kdiag[p];
                 if (MODE == FWD_LAST_TRAIN) {
                     a.xhat[p] = make_float2(y0 * inv, y1 * inv);
                 } else {
@@ -694,7 +690,7 @@ __global__ void __launch_bounds__(fwd_threads(COMPACT), 1) k_fwd(FwdArgs a) {
                 for (int i = 0; i < 8; ++i) {
                     const int idx = i * 32 + lane, rr = idx >> 3, c = idx & 7;
                     const int64_t node = t * TILE + quarter * 32 + rr;
-                    if (node < a.n) a.Hout[node * 8 + c] = stage[rr * 8 + (c ^ (rr & 7))];
+                    if (node < a.t.n) a.Hout[node * 8 + c] = stage[rr * 8 + (c ^ (rr & 7))];
                 }
                 __syncwarp();
             }
@@ -776,250 +772,297 @@ __global__ void k_gout(int64_t n, SellView<float2> K, const float *__restrict__ 
     dy[p] = make_float2(f * jx, f * jy);
 }
 
-// dU partials: block b, thread (o = tid / 64, c = tid % 64) sums dy_i[o] h4_i[c]
-__global__ void __launch_bounds__(128) k_du_part(int64_t n, const float2 *__restrict__ dy,
-                                                 const __nv_bfloat16 *__restrict__ H4, float *part) {
-    int o = threadIdx.x >> 6, c = threadIdx.x & 63;
-    float acc = 0.f;
-    for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
-        float2 g = dy[i];
-        acc = fmaf(o ? g.y : g.x, __bfloat162float(H4[i * CH + c]), acc);
+// dz^3 = (U^T dy) masked by h^4 > 0 (channel 63 -> 0), rounded to BF16, and the partials of
+// dU = sum_i dy_i h4_i^T: eight threads a node, one 16-byte chunk of h^4 each, so that a
+// warp reads whole lines.  63^3 nodes: 18 us (107 for dU alone when a block summed one node
+// after the other).
+__global__ void __launch_bounds__(256) k_head(int64_t n, const float2 *__restrict__ dy, const uint4 *__restrict__ H4,
+                                              const float *__restrict__ U, uint4 *__restrict__ dZ,
+                                              float *__restrict__ part) {
+    __shared__ float sh[8][2 * CH];
+    const int j = threadIdx.x & 7, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float u0[8], u1[8], d0[8], d1[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        u0[i] = U[8 * j + i];
+        u1[i] = U[CH + 8 * j + i];
+        d0[i] = d1[i] = 0.f;
     }
-    part[(int64_t)blockIdx.x * 128 + threadIdx.x] = acc;
+#pragma unroll 2
+    for (int64_t p = blockIdx.x * 32 + (threadIdx.x >> 3); p < n; p += (int64_t)gridDim.x * 32) {
+        const float2 g = dy[p];
+        float f[8], dz[8];
+        unpack8(__ldg(H4 + p * 8 + j), f);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            d0[i] = fmaf(g.x, f[i], d0[i]);
+            d1[i] = fmaf(g.y, f[i], d1[i]);
+            const float v = u0[i] * g.x + u1[i] * g.y;
+            dz[i] = f[i] > 0.f ? v : 0.f;
+        }
+        if (j == 7) dz[7] = 0.f;
+        dZ[p * 8 + j] = pack8(dz);
+    }
+    // the four nodes of a warp, then its block's warps, in a fixed order
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+#pragma unroll
+        for (int m = 8; m < 32; m <<= 1) {
+            d0[i] += __shfl_xor_sync(0xffffffffu, d0[i], m);
+            d1[i] += __shfl_xor_sync(0xffffffffu, d1[i], m);
+        }
+        if (lane < 8) {
+            sh[warp][8 * j + i] = d0[i];
+            sh[warp][CH + 8 * j + i] = d1[i];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * CH) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += sh[w][threadIdx.x];
+        part[(int64_t)blockIdx.x * 2 * CH + threadIdx.x] = t;
+    }
 }
-__global__ void k_du_final(const float *part, int np, float *gU) {
-    int t = threadIdx.x;
-    float a = 0.f;
-    for (int b = 0; b < np; ++b) a += part[(int64_t)b * 128 + t];
-    gU[t] += a;
+
+// g += the sum of np partials of a gradient.  A warp takes 32 neighbouring parameters, its
+// block's eight warps every eighth partial each (whole lines; one thread a parameter with
+// the partials strided took 40 us for a W, this one 5).  W: partials are dW^T (128 in x
+// 64 out), g is W's layout (64 out x 128 in).
+template <bool W>
+__global__ void __launch_bounds__(256) k_sum_parts(const float *__restrict__ part, int np, int width, float *g) {
+    __shared__ float sh[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;  // (width is a multiple of 32)
+    float t = 0.f;
+#pragma unroll 4
+    for (int b = warp; b < np; b += 8) t += __ldg(part + (int64_t)b * width + e);
+    sh[warp][lane] = t;
+    __syncthreads();
+    if (warp == 0) {
+        t = sh[0][lane];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) t += sh[w][lane];
+        g[W ? (e % CH) * CIN + e / CH : e] += t;
+    }
 }
 
 // ------------------------------------------------------------------ backward layer
 struct BwdArgs {
-    int64_t n;
-    int64_t ntiles;
-    SellView<float2> K;
-    const float *kdiag;
+    TileArgs t;              // h^l (the operand a^l is rebuilt)
     const float *volp;
-    const uint4 *Hin;        // h^l (operand a^l is rebuilt)
-    const uint4 *dZ;         // dz^l rows (BF16, masked) -- hidden layers
-    const float2 *dy;        // head: dy
-    const uint4 *H4;         // head: h^4 (mask)
-    const float *U;          // head: U (2 x 64)
+    const uint4 *dZ;         // dz^l rows (BF16, masked)
     const uint4 *Wbimg;      // 128 x 64 BF16 operand image of W^l (rows = inputs)
     float *dA;               // n x 128: [dA_self, dA_nbr / (K_ii |V_i|)]
     float *dWpart;           // grid x 128 x 64 (rows = inputs)
     int *err;
 };
 
-template <bool HEAD, bool NEED_DA>
-__global__ void __launch_bounds__(THREADS) k_bwd(BwdArgs a) {
+// One layer: dA = dz W and dW^T += a^T dz.  The same warps as in the forward layer build
+// [h, S h] and dz tiles, one row of 128 swizzled bytes a node; the MMA of dA reads dz with
+// the channels as K, that of dW reads both with the nodes as K (MN-major operands), so
+// nothing is transposed on the way.  Bound by the gathers, as the forward layer, and the
+// FP32 rows of dA (512 bytes a node), written through shared memory as whole lines.
+// 63^3 nodes: 59 us, 43 for the first layer, which needs no dA (163 to 203 and 158 with one
+// thread a node, whose rows and transposed two-byte stores met in the same banks).
+constexpr int BWD_TILE_BYTES = 3 * TILE * 128;
+constexpr int BWD_STAGES = 2;
+constexpr int BWD_GW = fwd_gw(false), BWD_THREADS = fwd_threads(false);
+constexpr int BWD_SMEM =
+    BWD_STAGES * BWD_TILE_BYTES + CIN * CH * 2 + TILE * 128 + FWD_KSTAGES * FWD_K * TILE * 12;
+
+template <bool NEED_DA>
+__global__ void __launch_bounds__(BWD_THREADS, 1) k_bwd(BwdArgs a) {
+    constexpr int GW = BWD_GW, STAGES = BWD_STAGES;
     extern __shared__ __align__(1024) unsigned char smem[];
-    __nv_bfloat16 *sDz = reinterpret_cast<__nv_bfloat16 *>(smem);                   // 128 nodes x 64 (K-major)
-    uint4 *sWb = reinterpret_cast<uint4 *>(smem + TILE * CH * 2);                     // 128 in x 64 out
-    __nv_bfloat16 *sAt = reinterpret_cast<__nv_bfloat16 *>(smem + TILE * CH * 2 + CIN * CH * 2);  // 128 in x 128 nodes
-    __nv_bfloat16 *sDzt = sAt + CIN * TILE;                                            // 64 out x 128 nodes
-    __shared__ __align__(8) uint64_t mbar;
+    unsigned char *sA = smem;                                                     // STAGES x [h, S h, dz] x 128 x 64
+    uint4 *sW = reinterpret_cast<uint4 *>(smem + STAGES * BWD_TILE_BYTES);        // 128 in x 64 out
+    float4 *sOut = reinterpret_cast<float4 *>(sW + CIN * CH / 8);                 // 128 rows of 32 FP32
+    float2 *sVal = reinterpret_cast<float2 *>(sOut + TILE * 8);
+    int32_t *sCol = reinterpret_cast<int32_t *>(sVal + FWD_KSTAGES * FWD_K * TILE);
+    __shared__ float sSc[FWD_KSTAGES][TILE];
+    __shared__ int sWid[FWD_KSTAGES][TILE / SELL_C];
+    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2], kfull[FWD_KSTAGES],
+        kempty[FWD_KSTAGES];
     __shared__ uint32_t tslot;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (NEED_DA)
-        for (int i = tid; i < CIN * CH / 8; i += THREADS) sWb[i] = a.Wbimg[i];
-    if (warp == 0) tmem_alloc(&tslot, 256);
-    if (tid == 0) mbar_init(&mbar);
+        for (int i = tid; i < CIN * CH / 8; i += BWD_THREADS) sW[i] = a.Wbimg[i];
+    if (warp == GW) tmem_alloc(&tslot, 512);
+    if (tid == 0) {
+        for (int i = 0; i < STAGES; ++i) {
+            mbar_init_n(&full[i], GW);
+            mbar_init_n(&empty[i], 1);
+        }
+        for (int i = 0; i < FWD_KSTAGES; ++i) {
+            mbar_init_n(&kfull[i], 32);
+            mbar_init_n(&kempty[i], GW);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init_n(&tfull[i], 1);
+            mbar_init_n(&tempty[i], 4);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    proxy_fence();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tslot;
-    const uint32_t tm_dA = tmem, tm_dW = tmem + 128;
-    const uint32_t id_dA = idesc_bf16(TILE, CIN);   // M = 128 nodes, N = 128 inputs
-    const uint32_t id_dW = idesc_bf16(CIN, CH);     // M = 128 inputs, N = 64 outputs
-    uint32_t phase = 0;
+    const uint32_t tmem = tslot;  // two accumulators of dA (128 columns each), then dW^T (64)
+    const uint32_t tm_dW = tmem + 2 * CIN;
+    const TileBufs bufs{sA, sVal, sCol, sSc, sWid, full, empty, kfull, kempty};
     bool failed = false;
-    int iter = 0;
-    __shared__ float sU[2 * CH];
-    if (HEAD) {
-        sU[tid] = a.U[tid];
-        __syncthreads();
-    }
-    for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++iter) {
-        const int64_t p = t * TILE + tid;
-        float dz[CH];
-        float av[CH];
-        uint4 *rowDz = reinterpret_cast<uint4 *>(sDz);
-        if (p < a.n) {
-            if (HEAD) {
-                float2 g = a.dy[p];
-                const uint4 *h4 = a.H4 + p * 8;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float f[8];
-                    unpack8(h4[j], f);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        int c = 8 * j + i;
-                        float v = sU[c] * g.x + sU[CH + c] * g.y;
-                        dz[c] = f[i] > 0.f ? v : 0.f;
-                    }
-                }
-                dz[CH - 1] = 0.f;
-                // round once to BF16 so both GEMMs see the same dz
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    uint4 u = pack8(dz + 8 * j);
-                    unpack8(u, dz + 8 * j);
-                    rowDz[cm_off(tid, 8 * j, CH) >> 3] = u;
-                }
-            } else {
-                const uint4 *dp = a.dZ + p * 8;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    uint4 u = dp[j];
-                    unpack8(u, dz + 8 * j);
-                    rowDz[cm_off(tid, 8 * j, CH) >> 3] = u;
-                }
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < CH; ++c) dz[c] = 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) rowDz[cm_off(tid, 8 * j, CH) >> 3] = make_uint4(0, 0, 0, 0);
-        }
-        // transposed operands of dW^T += a^T dz: column tid (this node)
-#pragma unroll
-        for (int c = 0; c < CH; ++c) sDzt[cm_off(c, tid, TILE)] = __float2bfloat16_rn(dz[c]);
-        if (p < a.n) {
-            const uint4 *hp = a.Hin + p * 8;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) unpack8(hp[j], av + 8 * j);
-        } else {
-#pragma unroll
-            for (int c = 0; c < CH; ++c) av[c] = 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < CH; ++c) sAt[cm_off(c, tid, TILE)] = __float2bfloat16_rn(av[c]);
-        if (p < a.n) {
-            aggregate_row(a.K, a.kdiag, a.Hin, p, av);
-        }
-#pragma unroll
-        for (int c = 0; c < CH; ++c) sAt[cm_off(CH + c, tid, TILE)] = __float2bfloat16_rn(av[c]);
-        proxy_fence();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) {
+    if (warp < GW) {
+        regs_raise<96>();
+        failed = build_tiles<false, GW, STAGES, BWD_TILE_BYTES, true>(a.t, bufs, a.dZ, warp, lane);
+    } else if (warp >= GW + 4) {
+        regs_lower<32>();
+        if (warp < GW + 4 + FWD_KSTAGES) failed = stage_entries(a.t, bufs, warp - GW - 4, lane);
+    } else {
+        regs_lower<64>();
+        const int quarter = warp - GW;
+        const uint32_t id_dA = idesc_bf16(TILE, CIN);                               // 128 nodes x 128 inputs
+        const uint32_t id_dW = idesc_bf16(CIN, CH) | (1u << 15) | (1u << 16);       // 128 inputs x 64 outputs, MN-major
+        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+        int st = 0;
+        uint32_t ph = 0;
+        auto issue = [&](int i) {
+            const int buf = i & 1;
+            if (!mbar_wait(&full[st], ph) || (NEED_DA && !mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1))) return false;
+            proxy_fence();
+            tc_fence_after();
+            const uint32_t a0 = smem_u32(sA + st * BWD_TILE_BYTES), dz0 = a0 + 2 * TILE * 128, b0 = smem_u32(sW);
             if (NEED_DA) {
-                uint32_t a0 = smem_u32(sDz), b0 = smem_u32(sWb);
 #pragma unroll
                 for (int ks = 0; ks < CH / 16; ++ks)
-                    mma_bf16(tm_dA, sdesc(a0 + ks * 256, 128, CH * 16), sdesc(b0 + ks * 256, 128, CH * 16), id_dA,
+                    mma_bf16(tmem + buf * CIN, sdesc_sw128(dz0 + ks * 32), sdesc(b0 + ks * 256, 128, CH * 16), id_dA,
                              ks > 0);
             }
-            uint32_t a1 = smem_u32(sAt), b1 = smem_u32(sDzt);
 #pragma unroll
             for (int ks = 0; ks < TILE / 16; ++ks)
-                mma_bf16(tm_dW, sdesc(a1 + ks * 256, 128, TILE * 16), sdesc(b1 + ks * 256, 128, TILE * 16), id_dW,
-                         (ks > 0 || iter > 0) ? 1u : 0u);
-            mma_commit(&mbar);
-        }
-        const bool done = mbar_wait(&mbar, phase);
-        if (__syncthreads_or(!done)) {
-            failed = true;
-            break;
-        }
-        phase ^= 1;
-        tc_fence_after();
-        if (NEED_DA) {
-            const uint32_t lane_base = tm_dA + ((uint32_t)(warp * 32) << 16);
-            float v[16];
-            float sn = 0.f;
-            if (p < a.n) sn = 1.f / (a.kdiag[p] * a.volp[p]);
+                mma_bf16(tm_dW, sdesc_sw128(a0 + ks * 16 * 128, TILE * 128), sdesc_sw128(dz0 + ks * 16 * 128, TILE * 128),
+                         id_dW, (ks > 0 || i > 0) ? 1u : 0u);
+            mma_commit(&empty[st]);
+            mma_commit(&tfull[buf]);
+            if (++st == STAGES) st = 0, ph ^= 1;
+            return true;
+        };
+        const bool issuer = quarter == 0 && lane == 0;
+        if (issuer && blockIdx.x < a.t.ntiles) failed = !issue(0);
+        int it = 0;
+        for (int64_t t = blockIdx.x; t < a.t.ntiles; t += gridDim.x, ++it) {
+            const int buf = it & 1;
+            if (issuer && !failed && t + gridDim.x < a.t.ntiles) failed = !issue(it + 1);
+            __syncwarp();
+            if (!__all_sync(0xffffffffu, !failed && mbar_wait(&tfull[buf], (it >> 1) & 1))) {
+                failed = true;
+                break;
+            }
+            tc_fence_after();
+            if (!NEED_DA) continue;
+            const int64_t p = t * TILE + quarter * 32 + lane;
+            const float sn = p < a.t.n ? 1.f / (a.t.kdiag[p] * a.volp[p]) : 0.f;
+            float4 *stage = sOut + quarter * 32 * 8;
 #pragma unroll
-            for (int c = 0; c < CIN; c += 16) {
-                tmem_ld16(lane_base + c, v);
-                if (p < a.n) {
-                    float4 *dst = reinterpret_cast<float4 *>(a.dA + p * CIN + c);
-                    float f = c < CH ? 1.f : sn;
+            for (int c = 0; c < CIN; c += 32) {
+                // 32 columns of the warp's rows through shared memory (chunks XOR-swizzled
+                // by row): stores of whole 128-byte lines
+                const float f = c < CH ? 1.f : sn;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    float v[16];
+                    tmem_ld16(lane_base + buf * CIN + c + 16 * u, v);
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        dst[i] = make_float4(v[4 * i] * f, v[4 * i + 1] * f, v[4 * i + 2] * f, v[4 * i + 3] * f);
+                        stage[lane * 8 + ((4 * u + i) ^ (lane & 7))] =
+                            make_float4(v[4 * i] * f, v[4 * i + 1] * f, v[4 * i + 2] * f, v[4 * i + 3] * f);
                 }
+                if (c == CIN - 32) {  // the accumulator has been read
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&tempty[buf]);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int rr = i * 4 + (lane >> 3), ch = lane & 7;
+                    const int64_t node = t * TILE + quarter * 32 + rr;
+                    if (node < a.t.n)
+                        *reinterpret_cast<float4 *>(a.dA + node * CIN + c + 4 * ch) = stage[rr * 8 + (ch ^ (rr & 7))];
+                }
+                __syncwarp();
             }
         }
-        tc_fence_before();
-        __syncthreads();
-    }
-    // dW^T partial of this CTA: lane = input feature (tid), 64 output columns
-    {
+        // dW^T partial of this CTA: lane = input feature, 64 output columns
+        const bool ok = it > 0 && !failed;
+        float *dst = a.dWpart + ((int64_t)blockIdx.x * CIN + quarter * 32 + lane) * CH;
         tc_fence_after();
-        float v[16];
-        const uint32_t lane_base = tm_dW + ((uint32_t)(warp * 32) << 16);
-        float *dst = a.dWpart + ((int64_t)blockIdx.x * CIN + tid) * CH;
 #pragma unroll
         for (int c = 0; c < CH; c += 16) {
-            tmem_ld16(lane_base + c, v);
+            float v[16];
+            tmem_ld16(tm_dW + ((uint32_t)(quarter * 32) << 16) + c, v);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) dst[c + i] = (iter > 0 && !failed) ? v[i] : 0.f;
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4 *>(dst + c + 4 * i) =
+                    ok ? make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         tc_fence_before();
     }
+    if (failed) atomicExch(a.err, 1);
     __syncthreads();
-    if (warp == 0) tmem_free(tmem, 256);
-    if (failed && tid == 0) atomicExch(a.err, 1);
+    if (warp == GW) tmem_free(tmem, 512);
 }
 
-// dz^{l-1}_k = (dA_self_k - |V_k| sum_i K_ki dA~_i) masked by h^l_k > 0 (channel 63 -> 0)
-__global__ void __launch_bounds__(128) k_dh(int64_t n, SellView<float2> K, const float *__restrict__ volp,
-                                            const float *__restrict__ dA, const uint4 *__restrict__ Hl,
-                                            uint4 *__restrict__ dZ) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// dz^{l-1}_k = (dA_self_k - |V_k| sum_i K_ki dA~_i) masked by h^l_k > 0 (channel 63 -> 0).
+// Bound by the latency of its gathers of 256-byte rows (0.44 GB from L2 at 63^3 nodes):
+// sixteen threads a node, one 16-byte chunk each, all of a batch's rows requested at once.
+// 82 us, 124 with one thread a node.  Fewer registers for more warps spill (104), several
+// slices a block one after the other share rows in L1 but wait longer (137).
+constexpr int DH_BATCH = 6;
+__global__ void __launch_bounds__(256, 4) k_dh(int64_t n, SellView<float2> K, const float *__restrict__ volp,
+                                            const float *__restrict__ dA, const uint2 *__restrict__ Hl,
+                                            uint2 *__restrict__ dZ) {
+    const int64_t p = blockIdx.x * (int64_t)16 + (threadIdx.x >> 4);
+    const int j = threadIdx.x & 15;
     if (p >= n) return;
-    float acc[CH];
+    const int64_t s = p >> 5, beg = K.sptr[s] + (p & 31);
+    const int w = (int)((K.sptr[s + 1] - K.sptr[s]) >> 5);
+    const float4 *rows = reinterpret_cast<const float4 *>(dA) + j;
+    const float4 self = __ldg(rows + p * (CIN / 4));
+    const uint2 h = __ldg(Hl + p * 16 + j);
+    const float vk = -volp[p];
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k0 = 0; k0 < w; k0 += DH_BATCH) {
+        float2 kv[DH_BATCH];
+        float4 u[DH_BATCH];
 #pragma unroll
-    for (int c = 0; c < CH; ++c) acc[c] = 0.f;
-    int64_t s = p >> 5;
-    int lane = (int)(p & 31);
-    int64_t beg = K.sptr[s];
-    int w = (int)((K.sptr[s + 1] - beg) >> 5);
-    for (int k = 0; k < w; ++k) {
-        int64_t q = beg + (int64_t)k * SELL_C + lane;
-        float2 kv = K.val[q];
-        if (kv.x == 0.f && kv.y == 0.f) continue;
-        const float4 *src = reinterpret_cast<const float4 *>(dA + (int64_t)K.col[q] * CIN + CH);
+        for (int k = 0; k < DH_BATCH; ++k)
+            if (k0 + k < w) {
+                const int64_t q = beg + (int64_t)(k0 + k) * SELL_C;
+                kv[k] = __ldg(K.val + q);
+                u[k] = __ldg(rows + (int64_t)__ldg(K.col + q) * (CIN / 4) + CH / 4);
+            }
 #pragma unroll
-        for (int j = 0; j < CH / 4; ++j) {
-            float4 u = __ldg(src + j);
-            acc[4 * j] += kv.x * u.x - kv.y * u.y;
-            acc[4 * j + 1] += kv.x * u.y + kv.y * u.x;
-            acc[4 * j + 2] += kv.x * u.z - kv.y * u.w;
-            acc[4 * j + 3] += kv.x * u.w + kv.y * u.z;
-        }
+        for (int k = 0; k < DH_BATCH; ++k)
+            if (k0 + k < w && (kv[k].x != 0.f || kv[k].y != 0.f)) {
+                acc[0] += kv[k].x * u[k].x - kv[k].y * u[k].y;
+                acc[1] += kv[k].x * u[k].y + kv[k].y * u[k].x;
+                acc[2] += kv[k].x * u[k].z - kv[k].y * u[k].w;
+                acc[3] += kv[k].x * u[k].w + kv[k].y * u[k].z;
+            }
     }
-    float vk = -volp[p];
-    const float4 *self = reinterpret_cast<const float4 *>(dA + p * CIN);
-    const uint4 *hl = Hl + p * 8;
+    const float sv[4] = {self.x, self.y, self.z, self.w};
+    const uint32_t hw[2] = {h.x, h.y};
+    float o[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        float hf[8], o[8];
-        unpack8(hl[j], hf);
-        float4 s0 = self[2 * j], s1 = self[2 * j + 1];
-        float sv[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            float g = sv[i] + vk * acc[8 * j + i];
-            o[i] = hf[i] > 0.f ? g : 0.f;
-        }
-        if (j == 7) o[7] = 0.f;
-        dZ[p * 8 + j] = pack8(o);
+    for (int i = 0; i < 4; ++i) {
+        const float hf = __uint_as_float((i & 1) ? (hw[i >> 1] & 0xffff0000u) : (hw[i >> 1] << 16));
+        const float g = sv[i] + vk * acc[i];
+        o[i] = hf > 0.f ? g : 0.f;
     }
-}
-
-// grad W^l (64 out x 128 in) += sum over CTAs of the partial dW^T (128 in x 64 out)
-__global__ void k_dw_final(const float *part, int np, float *gW) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;   // over 64 x 128 in output layout
-    if (idx >= WSZ) return;
-    int o = idx / CIN, i = idx % CIN;
-    float a = 0.f;
-    for (int b = 0; b < np; ++b) a += part[((int64_t)b * CIN + i) * CH + o];
-    gW[idx] += a;
+    if (j == 15) o[3] = 0.f;
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[1]), hi = __floats2bfloat162_rn(o[2], o[3]);
+    dZ[p * 16 + j] = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
 }
 
 // ------------------------------------------------------------------ zero-guess fallback
@@ -1122,7 +1165,7 @@ struct gl_warmstart_s {
     // partials and (alpha, 1 / ||a||_D)
     DBuf<double2> qa, rb, hp;
     DBuf<double> hpart, hsc;
-    int fwd_grid = 0, bwd_grid = 0;
+    int grid = 0;   // blocks of a layer's kernel
 };
 
 namespace {
@@ -1163,43 +1206,20 @@ void ws_reserve(gl_warmstart_s *w, int64_t n) {
 }
 
 void ws_setup_kernels(gl_warmstart_s *w) {
-    if (w->fwd_grid) return;
+    if (w->grid) return;
     GL_CUDA(cudaFuncSetAttribute(k_fwd<FWD_HIDDEN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem(true)));
     for (const void *fn : {(const void *)k_fwd<FWD_HIDDEN, false>, (const void *)k_fwd<FWD_LAST_TRAIN, false>,
                            (const void *)k_fwd<FWD_LAST_PREDICT, false>})
         GL_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, fwd_smem(false)));
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
-    // ask for the largest shared-memory carveout, or only one CTA fits an SM
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<true, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<false, true>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    GL_CUDA(cudaFuncSetAttribute(k_bwd<false, false>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    int dev = 0, nsm = 0, smem_sm = 0;
+    GL_CUDA(cudaFuncSetAttribute(k_bwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
+    GL_CUDA(cudaFuncSetAttribute(k_bwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BWD_SMEM));
+    int dev = 0, nsm = 0;
     GL_CUDA(cudaGetDevice(&dev));
     GL_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    GL_CUDA(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-    // CTAs per SM from the kernels' own register and shared-memory use (the
-    // occupancy query reports 0 for these kernels); tensor memory holds 512
-    // columns per SM: the forward kernel takes 64 and the backward 256.  The
-    // CTAs of one launch never wait on each other, so an estimate that is too
-    // high only queues CTAs.
-    auto per_sm = [&](const void *fn, int dyn, int cap) {
-        cudaFuncAttributes fa;
-        GL_CUDA(cudaFuncGetAttributes(&fa, fn));
-        int regs = ((fa.numRegs + 7) / 8) * 8 * THREADS;
-        int by_regs = regs > 0 ? 65536 / regs : cap;
-        int by_smem = smem_sm / (dyn + (int)fa.sharedSizeBytes + 1024);
-        return std::max(1, std::min(cap, std::min(by_regs, by_smem)));
-    };
-    int b = std::min(per_sm((const void *)k_bwd<true, true>, BWD_SMEM, 2),
-                     std::min(per_sm((const void *)k_bwd<false, true>, BWD_SMEM, 2),
-                              per_sm((const void *)k_bwd<false, false>, BWD_SMEM, 2)));
-    w->fwd_grid = nsm;  // one CTA per SM
-    w->bwd_grid = b * nsm;
+    w->grid = nsm;  // one CTA per SM
     w->part.alloc(RED_BLOCKS);
     w->bn.alloc(2);
-    w->dWpart.alloc((size_t)w->bwd_grid * CIN * CH);
+    w->dWpart.alloc((size_t)w->grid * CIN * CH);
     w->dUpart.alloc((size_t)DU_BLOCKS * 128);
     w->err.alloc(1);
     GL_CUDA(cudaMemset(w->err.get(), 0, sizeof(int)));
@@ -1239,7 +1259,7 @@ void ws_forward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const dou
     GL_LAUNCH_CHECK();
     note_launch(3);
     const int64_t ntiles = (n + TILE - 1) / TILE;
-    const int grid = (int)std::min<int64_t>(ntiles, w->fwd_grid);
+    const int grid = (int)std::min<int64_t>(ntiles, w->grid);
     // algorithmic bytes of one layer: each node's h row read once (neighbour rows
     // are re-reads of the same array), its K row (value + column) and K_ii, and
     // the written h row (the last layer of a prediction writes x0 instead)
@@ -1248,13 +1268,13 @@ void ws_forward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const dou
         const bool last_pred = (l == NL - 1) && !train;
         ProfScope ps("wsf", (double)n * (CH * 2 + (last_pred ? 16 : CH * 2)) + k_bytes, s);
         FwdArgs a{};
-        a.n = n;
-        a.ntiles = ntiles;
-        a.K = m->K32.view();
-        a.kdiag = m->kdiag32.get();
+        a.t.n = n;
+        a.t.ntiles = ntiles;
+        a.t.K = m->K32.view();
+        a.t.kdiag = m->kdiag32.get();
         // prediction ping-pongs between buffers 0 and 1
         int in = train ? l : (l & 1), out = train ? l + 1 : ((l + 1) & 1);
-        a.Hin = reinterpret_cast<const uint4 *>(Hbuf(w, in));
+        a.t.Hin = reinterpret_cast<const uint4 *>(Hbuf(w, in));
         a.Hout = reinterpret_cast<uint4 *>(Hbuf(w, out));
         a.Wimg = reinterpret_cast<const uint4 *>(w->Wf.get() + (size_t)l * WSZ);
         a.U = w->theta.get() + NL * WSZ;
@@ -1286,26 +1306,25 @@ void ws_backward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const do
     k_gout<<<grid_for(n, 256), 256, 0, s>>>(n, m->K32.view(), m->kdiag32.get(), m->volp32.get(), psi_p, w->r.get(),
                                             (float)scale, w->dy.get());
     float *gU = w->grad.get() + NL * WSZ;
-    k_du_part<<<DU_BLOCKS, 128, 0, s>>>(n, w->dy.get(), Hbuf(w, NL), w->dUpart.get());
-    k_du_final<<<1, 128, 0, s>>>(w->dUpart.get(), DU_BLOCKS, gU);
+    k_head<<<DU_BLOCKS, 256, 0, s>>>(n, w->dy.get(), reinterpret_cast<const uint4 *>(Hbuf(w, NL)),
+                                     w->theta.get() + NL * WSZ, reinterpret_cast<uint4 *>(w->dZ.get()),
+                                     w->dUpart.get());
+    k_sum_parts<false><<<2 * CH / 32, 256, 0, s>>>(w->dUpart.get(), DU_BLOCKS, 2 * CH, gU);
     GL_LAUNCH_CHECK();
     const int64_t ntiles = (n + TILE - 1) / TILE;
-    const int grid = (int)std::min<int64_t>(ntiles, w->bwd_grid);
+    const int grid = (int)std::min<int64_t>(ntiles, w->grid);
     const double k_bytes = (double)m->K32.nnz_stored * (sizeof(float2) + 4) + (double)n * 8;
     for (int l = NL - 1; l >= 0; --l) {
         // algorithmic bytes: h^l and dz rows read, K row, dA rows written
         note_launch(l > 0 ? 2 : 1);
         BwdArgs a{};
-        a.n = n;
-        a.ntiles = ntiles;
-        a.K = m->K32.view();
-        a.kdiag = m->kdiag32.get();
+        a.t.n = n;
+        a.t.ntiles = ntiles;
+        a.t.K = m->K32.view();
+        a.t.kdiag = m->kdiag32.get();
+        a.t.Hin = reinterpret_cast<const uint4 *>(Hbuf(w, l));
         a.volp = m->volp32.get();
-        a.Hin = reinterpret_cast<const uint4 *>(Hbuf(w, l));
         a.dZ = reinterpret_cast<const uint4 *>(w->dZ.get());
-        a.dy = w->dy.get();
-        a.H4 = reinterpret_cast<const uint4 *>(Hbuf(w, NL));
-        a.U = w->theta.get() + NL * WSZ;
         a.Wbimg = reinterpret_cast<const uint4 *>(w->Wb.get() + (size_t)l * WSZ);
         a.dA = w->dA.get();
         a.dWpart = w->dWpart.get();
@@ -1313,20 +1332,18 @@ void ws_backward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const do
         {
             // algorithmic bytes: h^l and dz rows read, K row, dA rows written
             ProfScope ps("wsb", (double)n * (CH * 2 + CH * 2 + (l > 0 ? CIN * 4 : 0)) + k_bytes, s);
-            if (l == NL - 1)
-                k_bwd<true, true><<<grid, THREADS, BWD_SMEM, s>>>(a);
-            else if (l > 0)
-                k_bwd<false, true><<<grid, THREADS, BWD_SMEM, s>>>(a);
+            if (l > 0)
+                k_bwd<true><<<grid, BWD_THREADS, BWD_SMEM, s>>>(a);
             else
-                k_bwd<false, false><<<grid, THREADS, BWD_SMEM, s>>>(a);
+                k_bwd<false><<<grid, BWD_THREADS, BWD_SMEM, s>>>(a);
         }
         GL_LAUNCH_CHECK();
-        k_dw_final<<<grid_for(WSZ, 256), 256, 0, s>>>(w->dWpart.get(), grid, w->grad.get() + (size_t)l * WSZ);
+        k_sum_parts<true><<<WSZ / 32, 256, 0, s>>>(w->dWpart.get(), grid, WSZ, w->grad.get() + (size_t)l * WSZ);
         GL_LAUNCH_CHECK();
         if (l > 0) {
-            k_dh<<<grid_for(n, 128), 128, 0, s>>>(n, m->K32.view(), m->volp32.get(), w->dA.get(),
-                                                  reinterpret_cast<const uint4 *>(Hbuf(w, l)),
-                                                  reinterpret_cast<uint4 *>(w->dZ.get()));
+            k_dh<<<grid_for(n, 16), 256, 0, s>>>(n, m->K32.view(), m->volp32.get(), w->dA.get(),
+                                                  reinterpret_cast<const uint2 *>(Hbuf(w, l)),
+                                                  reinterpret_cast<uint2 *>(w->dZ.get()));
             GL_LAUNCH_CHECK();
         }
     }
