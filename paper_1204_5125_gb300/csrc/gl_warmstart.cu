@@ -1341,7 +1341,7 @@ void ws_backward(gl_warmstart_s *w, gl_mesh_s *m, const double2 *psi_p, const do
         k_sum_parts<true><<<WSZ / 32, 256, 0, s>>>(w->dWpart.get(), grid, WSZ, w->grad.get() + (size_t)l * WSZ);
         GL_LAUNCH_CHECK();
         if (l > 0) {
-            k_dh<<<grid_for(n, 16), 256, 0, s>>>(n, m->K32.view(), m->volp32.get(), w->dA.get(),
+            k_dh<<<(unsigned)((n + 15) / 16), 256, 0, s>>>(n, m->K32.view(), m->volp32.get(), w->dA.get(),
                                                   reinterpret_cast<const uint2 *>(Hbuf(w, l)),
                                                   reinterpret_cast<uint2 *>(w->dZ.get()));
             GL_LAUNCH_CHECK();
