@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) k_bwd(BwdArgs a) {
         uint32_t ph = 0;
         auto issue = [&](int i) {
             const int buf = i & 1;
-            if (!mbar_wait(&full[st], ph) || (NEED_DA && !mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1))) return false;
+            if (!mbar_wait(&full[st], ph) || !mbar_wait(&tempty[buf], ((i >> 1) & 1) ^ 1)) return false;
             proxy_fence();
             tc_fence_after();
             const uint32_t a0 = smem_u32(sA + st * BWD_TILE_BYTES), dz0 = a0 + 2 * TILE * 128, b0 = smem_u32(sW);
@@ -959,7 +959,13 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) k_bwd(BwdArgs a) {
                 break;
             }
             tc_fence_after();
-            if (!NEED_DA) continue;
+            if (!NEED_DA) {
+                // nothing to read, but the issuer must not get two tiles ahead of this warp:
+                // tfull's parity would have turned twice and the wait above would miss both
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[buf]);
+                continue;
+            }
             const int64_t p = t * TILE + quarter * 32 + lane;
             const float sn = p < a.t.n ? 1.f / (a.t.kdiag[p] * a.volp[p]) : 0.f;
             float4 *stage = sOut + quarter * 32 * 8;
