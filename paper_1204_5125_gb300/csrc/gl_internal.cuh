@@ -2,9 +2,21 @@
 // points shared between the translation units of the library.
 #pragma once
 
+#include <atomic>
+
 #include "gl_common.cuh"
 
+namespace gl {
+// a number that no other handle of this process has had: a handle's address comes back
+// with the next one of its kind, so nothing that outlives a handle may be kept by it
+inline int64_t next_uid() {
+    static std::atomic<int64_t> next{1};
+    return next.fetch_add(1);
+}
+}  // namespace gl
+
 struct gl_mesh_s {
+    const int64_t uid = gl::next_uid();   // keys cached CUDA graphs
     int dim = 0, N = 0;
     int64_t n = 0;
     double h = 0, mu = 0, bhat[3] = {0, 0, 1};

@@ -13,8 +13,6 @@
 //     deterministic numeric pass), made exactly Hermitian as (A_c + A_c^H)/2
 //   * colours: red-black on the lattice level, Jones-Plassmann below
 //   * coarsest level: dense FP64 inverse by the blocked Hermitian sweep operator
-#include <atomic>
-
 #include <chrono>
 
 #include "gl_internal.cuh"
@@ -1191,8 +1189,7 @@ static void copy_csr(const CsrDev &a, CsrDev &b, cudaStream_t s) {
 // ------------------------------------------------------------------ driver
 void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_options &o, cudaStream_t s,
                    const gl_prec_s *like) {
-    static std::atomic<int64_t> next_uid{1};
-    p->uid = next_uid.fetch_add(1);
+    p->uid = next_uid();
     p->mesh = m;
     p->mesh_version = m->version;
     // GL_VERBOSE: wall time of the setup's phases (synchronising at each mark)

@@ -613,11 +613,11 @@ struct Graph {
 };
 
 struct GraphKey {
-    const void *m = nullptr, *psi = nullptr, *b = nullptr, *x = nullptr;
-    int64_t prec_uid = -1, generation = -1, mesh_version = -1;
+    const void *psi = nullptr, *b = nullptr, *x = nullptr;
+    int64_t mesh_uid = -1, prec_uid = -1, generation = -1, mesh_version = -1;
     int vc32 = 0, df = 0, loop = 0;
     bool operator==(const GraphKey &o) const {
-        return m == o.m && psi == o.psi && b == o.b && x == o.x && prec_uid == o.prec_uid &&
+        return psi == o.psi && b == o.b && x == o.x && mesh_uid == o.mesh_uid && prec_uid == o.prec_uid &&
                generation == o.generation && mesh_version == o.mesh_version && vc32 == o.vc32 && df == o.df &&
                loop == o.loop;
     }
@@ -920,7 +920,7 @@ static MinresResult minres(gl_mesh_s *m, gl_prec_s *p, const cplx_t<T> *psi, con
     // its own loop.
     const bool timing_class = profiler().active && !profiler().name.empty();
     const bool loop = device_loop && !timing_class && !(p && p->rinf);
-    GraphKey key{m, psi, b, x, p ? p->uid : -1, profiler().generation, m->version, vc32 ? 1 : 0, df ? 1 : 0,
+    GraphKey key{psi, b, x, m->uid, p ? p->uid : -1, profiler().generation, m->version, vc32 ? 1 : 0, df ? 1 : 0,
                  loop ? 1 : 0};
     if (!(key == W.key) || (loop ? !W.loop.exec : (!W.init.exec || !W.body.exec))) {
         W.key = key;
