@@ -117,12 +117,14 @@ __device__ void scal_init(MinresDev *S, double bb, double vv) {
     S->check_true = 0;
     S->lucky = 0;
     S->bnorm = sqrt(bb);
-    S->true_rel = (S->bnorm > 0) ? sqrt(vv) / S->bnorm : 0.0;
+    S->true_rel = S->bnorm == 0 ? 0.0 : sqrt(vv) / S->bnorm;
     // the tolerance is relative to b, the recurrence's estimate to r0 = b - J x0:
     // scaled by ||r0||_D / ||b||_D (exactly 1 from x0 = 0)
     S->rho0 = S->true_rel;
     S->est = 1.0;
-    if (!(S->bnorm > 0)) {
+    if (isnan(bb)) {  // (before b = 0: a comparison with NaN is false)
+        S->status = ST_NAN;
+    } else if (S->bnorm == 0) {
         S->status = ST_CONV;
         S->est = 0;
     } else if (use_true && S->true_rel <= tol) {
@@ -570,7 +572,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_true_resid(int64_t n, SellView<
     const double r2 = sum_parts(part, sh);
     if (threadIdx.x) return;
     if (final) {
-        if (S->bnorm > 0) S->true_rel = sqrt(r2) / S->bnorm;
+        if (S->bnorm != 0) S->true_rel = sqrt(r2) / S->bnorm;
         return;
     }
     scal_true(S, r2);
@@ -695,7 +697,7 @@ void precond_apply_any<float>(gl_prec_s *p, const float2 *v, float2 *z, const in
 // b = 0 has the solution x = 0 whatever the initial guess
 template <typename C>
 __global__ void k_zero_if_bzero(int64_t n, const MinresDev *S, C *x) {
-    if (S->bnorm > 0) return;
+    if (S->bnorm != 0) return;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) x[i] = mk(decltype(x[0].x)(0), decltype(x[0].x)(0));
 }
