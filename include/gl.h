@@ -239,7 +239,8 @@ GL_API gl_status gl_mesh_set_mu(gl_mesh mesh, double mu, void *stream);
 GL_API gl_status gl_mesh_info(gl_mesh mesh, int64_t *n, int64_t *nnz, double *volumes_dev);
 
 /* Discrete GL residual (Eq. discr ginla): r_i = (K psi)_i - psi_i (1 - |psi_i|^2),
- * K = D^-1 K-hat.  psi_dev, r_dev: n complex (FP64); may not alias. */
+ * K = D^-1 K-hat.  psi_dev, r_dev: n complex (FP64); not the same vector (where they
+ * overlap in part, the result is formed in the mesh's scratch first). */
 GL_API gl_status gl_residual(gl_mesh mesh, const void *psi_dev, void *r_dev, void *stream);
 
 /* d GL / d mu at fixed psi (the parameter derivative that pseudo-arclength
@@ -257,7 +258,8 @@ GL_API gl_status gl_energy(gl_mesh mesh, const void *psi_dev, double *energy_hos
 
 /* Discrete Jacobian (Sec. 3):
  *   y_i = (K phi)_i + (-1 + 2|psi_i|^2) phi_i + psi_i^2 conj(phi_i).
- * psi, phi, y: n complex FP64; y may not alias psi or phi.  GL_FP64: the stored
+ * psi, phi, y: n complex FP64; y is neither psi nor phi (where it overlaps one in
+ * part, the result is formed in the mesh's scratch first).  GL_FP64: the stored
  * K.  GL_APPLY_FP64_TABLES: the same operator formed matrix-free from the lattice
  * stencil's FP64 tables (meshes with an even number of nodes per side whose
  * stored K matches the tables to 16 ulp of its largest entry; GL_ERR_ARG on
@@ -278,9 +280,12 @@ GL_API gl_status gl_jacobian_apply(gl_mesh mesh, const void *psi_dev, const void
  * can fail or fragment it), and latency-critical loops (cudaMalloc/cudaFree may
  * synchronise the device).  The paper has no counterpart; this is an interface
  * convenience.
- * It allocates nothing and holds nothing: it runs the kernel of gl_jacobian_apply
- * on the caller's vectors.  Meshes with more than GL_NOALLOC_MAX_NODES = 262144
- * nodes are rejected with GL_ERR_CAPACITY.
+ * It allocates nothing: it runs the kernel of gl_jacobian_apply on the caller's
+ * vectors.  Where y overlaps psi or phi in part, the result is formed in a static
+ * device array of 4 MiB first, which all such calls on a device share: two of them
+ * must not overlap on the GPU, and the first should come before a stream capture.
+ * Meshes with more than GL_NOALLOC_MAX_NODES = 262144 nodes are rejected with
+ * GL_ERR_CAPACITY.
  * Arguments and layouts as gl_jacobian_apply. */
 GL_API gl_status gl_jacobian_apply_noalloc(gl_mesh mesh, const void *psi_dev, const void *phi_dev, void *y_dev,
                                            void *stream);

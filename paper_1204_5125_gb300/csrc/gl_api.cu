@@ -210,7 +210,14 @@ gl_status gl_residual(gl_mesh m, const void *psi, void *r, void *stream) {
     return guard([&] {
         GL_REQUIRE(m && psi && r, GL_ERR_ARG, "NULL argument");
         GL_REQUIRE(psi != r, GL_ERR_ARG, "psi and r must not alias");
-        residual_nodes(m, (const double2 *)psi, (double2 *)r, as_stream(stream));
+        cudaStream_t s = as_stream(stream);
+        if (overlap(psi, r, m->n)) {  // partly over one another
+            ensure_tmp(m);
+            residual_nodes(m, (const double2 *)psi, m->t0.get(), s);
+            GL_CUDA(cudaMemcpyAsync(r, m->t0.get(), m->t0.bytes(), cudaMemcpyDeviceToDevice, s));
+            return GL_OK;
+        }
+        residual_nodes(m, (const double2 *)psi, (double2 *)r, s);
         return GL_OK;
     });
 }
@@ -224,6 +231,12 @@ gl_status gl_jacobian_apply(gl_mesh m, const void *psi, const void *phi, void *y
                    GL_ERR_ARG, "unknown precision");
         cudaStream_t s = as_stream(stream);
         if (precision == GL_FP64) {
+            if (overlap(y, psi, m->n) || overlap(y, phi, m->n)) {
+                ensure_tmp(m);
+                jacobian_apply_nodes(m, (const double2 *)psi, (const double2 *)phi, m->t0.get(), s);
+                GL_CUDA(cudaMemcpyAsync(y, m->t0.get(), m->t0.bytes(), cudaMemcpyDeviceToDevice, s));
+                return GL_OK;
+            }
             jacobian_apply_nodes(m, (const double2 *)psi, (const double2 *)phi, (double2 *)y, s);
             return GL_OK;
         }

@@ -317,6 +317,12 @@ void jacobian_apply_pdf(gl_mesh_s *m, const double2 *psi, const double2 *phi, do
 // the FP64 Jacobian and residual on node-order vectors (no reordering)
 void jacobian_apply_nodes(const gl_mesh_s *m, const double2 *psi, const double2 *phi, double2 *y, cudaStream_t s);
 void residual_nodes(const gl_mesh_s *m, const double2 *psi, double2 *r, cudaStream_t s);
+// whether two vectors of n complex doubles share memory: a node's row reads other nodes'
+// values, so these two kernels cannot write over what they read
+inline bool overlap(const void *a, const void *b, int64_t n) {
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return (x < y ? y - x : x - y) < (uintptr_t)n * sizeof(double2);
+}
 // fills m->kcoln once K is built
 void mesh_node_columns(gl_mesh_s *m, cudaStream_t s);
 // node order: r <- -r, returns ||r||_R (part: RED_BLOCKS doubles, scal: 1 double)
