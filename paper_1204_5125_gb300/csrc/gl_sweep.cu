@@ -873,6 +873,9 @@ static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
                         1e3 * t);
             if (t < best) best = t, bestG = g, bestK = K;
         }
+        // a wait of a candidate ran out: the launches behind it returned at once, so the
+        // times say nothing; the choice is the one made without timing
+        if (sweeps_failed(p, s)) bestG = sweep_default_lanes(D.A.nnz, L.n), bestK = 1;
         sweep_shape<T>(L, sync, bestG, bestK, s);
         sweep_zero(D, s);
         GL_CUDA(cudaMemsetAsync(p->err.get(), 0, sizeof(int), s));
