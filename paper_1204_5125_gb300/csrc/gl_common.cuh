@@ -156,8 +156,9 @@ template <typename C>
 struct Sell {
     int64_t nrows = 0, nslices = 0, nnz_stored = 0, nnz_real = 0;
     DBuf<int64_t> sptr;
-    DBuf<int32_t> col;
+    DBuf<int32_t> col;  // (with node columns: nnz_stored of these behind the solve-order ones)
     DBuf<C> val;
+    const int32_t *node_col() const { return col.get() + nnz_stored; }
     SellView<C> view() const { return SellView<C>{nrows, nslices, sptr.get(), col.get(), val.get()}; }
     size_t bytes() const { return sptr.bytes() + col.bytes() + val.bytes(); }
 };

@@ -38,8 +38,7 @@ struct gl_mesh_s {
     int ncolors0 = 2;
     std::vector<int64_t> cstart0;
     gl::DBuf<int32_t> perm, iperm;
-    gl::Sell<double2> K;                  // off-diagonals of K = D^-1 K-hat (solve ordering)
-    gl::DBuf<int32_t> kcoln;              // the same entries' columns as node numbers
+    gl::Sell<double2> K;                  // off-diagonals of K = D^-1 K-hat (solve ordering), with node columns
     gl::DBuf<double> kdiag, volp;         // K_ii and |V_i| (solve ordering)
     bool has32 = false;
     gl::Sell<float2> K32;
@@ -220,9 +219,12 @@ void mesh_create_simplicial(gl_mesh_s *m, int dim, int64_t n, const double *xyz_
 // round-based smallest-last colouring of a graph (gl_setup.cu); returns the colour count
 int colour_graph_psl(const CsrDev &A, int32_t *color, cudaStream_t s);
 void mesh_ensure_fp32(gl_mesh_s *m, cudaStream_t s);
+// sliced ELL of A's rows perm[0..nrows) with columns mapped by icol; node_cols: the
+// columns as they were beside them (Sell::node_col)
 template <typename C>
 void build_sell(int64_t nrows, int64_t ncols, const int32_t *perm, const int32_t *icol, const CsrDev &A,
-                const double *row_scale, bool drop_diag, Sell<C> &out, double *diag_out, cudaStream_t s);
+                const double *row_scale, bool drop_diag, Sell<C> &out, double *diag_out, cudaStream_t s,
+                bool node_cols = false);
 void to_float(const double *in, float *out, int64_t n, cudaStream_t s);
 // grouped CSR of A's rows perm[0..nrows) with columns mapped by icol; columns
 // (after the map) below col_lo are left out
@@ -323,8 +325,6 @@ inline bool overlap(const void *a, const void *b, int64_t n) {
     const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
     return (x < y ? y - x : x - y) < (uintptr_t)n * sizeof(double2);
 }
-// fills m->kcoln once K is built
-void mesh_node_columns(gl_mesh_s *m, cudaStream_t s);
 // node order: r <- -r, returns ||r||_R (part: RED_BLOCKS doubles, scal: 1 double)
 double newton_rhs(const gl_mesh_s *m, double2 *r, double *part, double *scal, cudaStream_t s);
 void newton_update(int64_t n, const double2 *d, double2 *psi, cudaStream_t s);

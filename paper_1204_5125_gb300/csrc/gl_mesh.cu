@@ -416,33 +416,28 @@ __global__ void k_permute_real(int64_t n, const int32_t *perm, const double *in,
 }
 
 // ---------------------------------------------------------------- sliced ELL builder
-__global__ void k_sell_rowlen(int64_t nrows, const int32_t *perm, const int64_t *rp, const int32_t *ci, bool drop_diag,
-                              int32_t *len) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= nrows) return;
-    int64_t r = perm ? perm[p] : p;
-    int64_t l = rp[r + 1] - rp[r];
-    if (drop_diag)
-        for (int64_t q = rp[r]; q < rp[r + 1]; ++q)
-            if (ci[q] == r) --l;
-    len[p] = (int32_t)l;
-}
-
-__global__ void k_sell_width(int64_t nrows, int64_t nslices, const int32_t *len, int64_t *ssize) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= nslices) return;
-    int w = 0;
-    for (int l = 0; l < SELL_C; ++l) {
-        int64_t p = s * SELL_C + l;
-        if (p < nrows) w = max(w, len[p]);
+// a slice's longest row, one warp a slice
+__global__ void k_sell_width(int64_t nrows, int64_t nslices, const int32_t *perm, const int64_t *rp, const int32_t *ci,
+                             bool drop_diag, int64_t *ssize) {
+    static_assert(SELL_C == 32, "a lane takes a row of its slice");
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p / SELL_C >= nslices) return;
+    int len = 0;
+    if (p < nrows) {
+        const int64_t r = perm ? perm[p] : p;
+        len = (int)(rp[r + 1] - rp[r]);
+        if (drop_diag)
+            for (int64_t q = rp[r]; q < rp[r + 1]; ++q)
+                if (ci[q] == r) --len;
     }
-    ssize[s] = (int64_t)w * SELL_C;
+    const int w = __reduce_max_sync(0xffffffffu, len);
+    if (p % SELL_C == 0) ssize[p / SELL_C] = (int64_t)w * SELL_C;
 }
 
 template <typename C>
 __global__ void k_sell_fill(int64_t nrows, int64_t ncols, const int32_t *perm, const int32_t *icol, const int64_t *rp,
                             const int32_t *ci, const double2 *v, const double *row_scale, bool drop_diag,
-                            const int64_t *sptr, int32_t *scol, C *sval, double *diag_out) {
+                            const int64_t *sptr, int32_t *scol, C *sval, double *diag_out, int32_t *ncol) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= nrows) return;
     int64_t r = perm ? perm[p] : p;
@@ -461,6 +456,7 @@ __global__ void k_sell_fill(int64_t nrows, int64_t ncols, const int32_t *perm, c
             continue;
         }
         scol[base + (int64_t)k * SELL_C] = icol ? icol[c] : (int32_t)c;
+        if (ncol) ncol[base + (int64_t)k * SELL_C] = (int32_t)c;
         C val;
         val.x = a.x * sc;
         val.y = a.y * sc;
@@ -470,6 +466,7 @@ __global__ void k_sell_fill(int64_t nrows, int64_t ncols, const int32_t *perm, c
     int32_t pad = (int32_t)(p < ncols ? p : ncols - 1);
     for (; k < w; ++k) {
         scol[base + (int64_t)k * SELL_C] = pad;
+        if (ncol) ncol[base + (int64_t)k * SELL_C] = (int32_t)r;
         C z;
         z.x = 0;
         z.y = 0;
@@ -480,14 +477,12 @@ __global__ void k_sell_fill(int64_t nrows, int64_t ncols, const int32_t *perm, c
 
 template <typename C>
 void build_sell(int64_t nrows, int64_t ncols, const int32_t *perm, const int32_t *icol, const CsrDev &A,
-                const double *row_scale, bool drop_diag, Sell<C> &out, double *diag_out, cudaStream_t s) {
+                const double *row_scale, bool drop_diag, Sell<C> &out, double *diag_out, cudaStream_t s, bool node_cols) {
     out.nrows = nrows;
     out.nslices = (nrows + SELL_C - 1) / SELL_C;
-    DBuf<int32_t> len(nrows > 0 ? nrows : 1);
     out.sptr.alloc(out.nslices + 1);
-    k_sell_rowlen<<<grid_for(nrows, 256), 256, 0, s>>>(nrows, perm, A.rp.get(), A.ci.get(), drop_diag, len.get());
-    GL_LAUNCH_CHECK();
-    k_sell_width<<<grid_for(out.nslices, 256), 256, 0, s>>>(nrows, out.nslices, len.get(), out.sptr.get());
+    k_sell_width<<<grid_for(out.nslices * SELL_C, 256), 256, 0, s>>>(nrows, out.nslices, perm, A.rp.get(), A.ci.get(),
+                                                                    drop_diag, out.sptr.get());
     GL_LAUNCH_CHECK();
     scan_exclusive(out.sptr.get(), out.sptr.get(), out.nslices, true, s);
     int64_t total = 0;
@@ -495,19 +490,22 @@ void build_sell(int64_t nrows, int64_t ncols, const int32_t *perm, const int32_t
     GL_CUDA(cudaStreamSynchronize(s));
     out.nnz_stored = total;
     out.nnz_real = A.nnz - (drop_diag ? nrows : 0);
-    out.col.alloc(total > 0 ? total : 1);
+    // the node columns are part of this allocation and of the filling launch (a mesh of
+    // 512^2 nodes: 2.91 ms to create with one more of each and a row-length array, 2.70 so)
+    out.col.alloc(total > 0 ? (node_cols ? 2 : 1) * total : 1);
     out.val.alloc(total > 0 ? total : 1);
     k_sell_fill<C><<<grid_for(nrows, 256), 256, 0, s>>>(nrows, ncols, perm, icol, A.rp.get(), A.ci.get(), A.v.get(),
                                                         row_scale, drop_diag, out.sptr.get(), out.col.get(),
-                                                        out.val.get(), diag_out);
+                                                        out.val.get(), diag_out,
+                                                        node_cols ? out.col.get() + total : nullptr);
     GL_LAUNCH_CHECK();
     GL_CUDA(cudaStreamSynchronize(s));
 }
 
 template void build_sell<double2>(int64_t, int64_t, const int32_t *, const int32_t *, const CsrDev &, const double *,
-                                  bool, Sell<double2> &, double *, cudaStream_t);
+                                  bool, Sell<double2> &, double *, cudaStream_t, bool);
 template void build_sell<float2>(int64_t, int64_t, const int32_t *, const int32_t *, const CsrDev &, const double *,
-                                 bool, Sell<float2> &, double *, cudaStream_t);
+                                 bool, Sell<float2> &, double *, cudaStream_t, bool);
 
 // ---------------------------------------------------------------- grouped CSR builder
 __global__ void k_csrg_len(int64_t nrows, const int32_t *perm, const int32_t *icol, const int64_t *rp,
@@ -727,8 +725,7 @@ void mesh_create(gl_mesh_s *m, int dim, int N, double edge, double mu, const dou
 
     // K = D^-1 K-hat, off-diagonals as sliced ELL in the solve ordering
     m->kdiag.alloc(n);
-    build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s);
-    mesh_node_columns(m, s);
+    build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s, true);
     m->volp.alloc(n);
     k_permute_real<<<grid_for(n, 256), 256, 0, s>>>(n, m->perm.get(), m->vol.get(), m->volp.get());
     GL_LAUNCH_CHECK();
@@ -745,7 +742,7 @@ static void refill_sell(int64_t nrows, int64_t ncols, const int32_t *perm, const
                         const double *row_scale, bool drop_diag, Sell<C> &out, double *diag_out, cudaStream_t s) {
     k_sell_fill<C><<<grid_for(nrows, 256), 256, 0, s>>>(nrows, ncols, perm, icol, A.rp.get(), A.ci.get(), A.v.get(),
                                                         row_scale, drop_diag, out.sptr.get(), out.col.get(),
-                                                        out.val.get(), diag_out);
+                                                        out.val.get(), diag_out, nullptr);
     GL_LAUNCH_CHECK();
 }
 
@@ -1213,8 +1210,7 @@ void mesh_create_simplicial(gl_mesh_s *m, int dim, int64_t n, const double *xyz_
     m->nred = m->cstart0.size() > 1 ? m->cstart0[1] : n;
     // K = D^-1 K-hat, off-diagonals as sliced ELL in the solve ordering
     m->kdiag.alloc(n);
-    build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s);
-    mesh_node_columns(m, s);
+    build_sell<double2>(n, n, m->perm.get(), m->iperm.get(), K, m->vol.get(), true, m->K, m->kdiag.get(), s, true);
     m->volp.alloc(n);
     k_permute_real<<<grid_for(n, 256), 256, 0, s>>>(n, m->perm.get(), m->vol.get(), m->volp.get());
     GL_LAUNCH_CHECK();

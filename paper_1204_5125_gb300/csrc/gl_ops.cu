@@ -114,14 +114,6 @@ __global__ void __launch_bounds__(256) k_residual_nodes(int64_t n, SellView<doub
     const double d = kdiag[p] - 1.0 + a2;
     r[v] = mk(acc.x + d * ps.x, acc.y + d * ps.y);
 }
-// by rows: the last slice's lanes past the last row hold no entries
-__global__ void k_node_columns(int64_t n, SellView<double2> K, const int32_t *__restrict__ perm,
-                               int32_t *__restrict__ coln) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    for (int64_t e = K.sptr[p >> 5] + (p & 31); e < K.sptr[(p >> 5) + 1]; e += SELL_C) coln[e] = perm[K.col[e]];
-}
-
 // Newton right-hand side (Eq. Newton system): r <- -r in place, with per-block
 // partials of ||r||_R^2 = sum |V_i| |r_i|^2
 __global__ void k_negate_norm(int64_t n, const double *__restrict__ vol, double2 *__restrict__ r, double *part) {
@@ -178,18 +170,13 @@ void jacobian_apply_p32(const gl_mesh_s *m, const double2 *psi, const double2 *p
     GL_LAUNCH_CHECK();
 }
 void jacobian_apply_nodes(const gl_mesh_s *m, const double2 *psi, const double2 *phi, double2 *y, cudaStream_t s) {
-    k_jacobian_nodes<<<grid_for(m->n, 256), 256, 0, s>>>(m->n, m->K.view(), m->kcoln.get(), m->iperm.get(),
+    k_jacobian_nodes<<<grid_for(m->n, 256), 256, 0, s>>>(m->n, m->K.view(), m->K.node_col(), m->iperm.get(),
                                                          m->kdiag.get(), psi, phi, y);
     GL_LAUNCH_CHECK();
 }
 void residual_nodes(const gl_mesh_s *m, const double2 *psi, double2 *r, cudaStream_t s) {
-    k_residual_nodes<<<grid_for(m->n, 256), 256, 0, s>>>(m->n, m->K.view(), m->kcoln.get(), m->iperm.get(),
+    k_residual_nodes<<<grid_for(m->n, 256), 256, 0, s>>>(m->n, m->K.view(), m->K.node_col(), m->iperm.get(),
                                                          m->kdiag.get(), psi, r);
-    GL_LAUNCH_CHECK();
-}
-void mesh_node_columns(gl_mesh_s *m, cudaStream_t s) {
-    m->kcoln.alloc(m->K.col.n);
-    k_node_columns<<<grid_for(m->n, 256), 256, 0, s>>>(m->n, m->K.view(), m->perm.get(), m->kcoln.get());
     GL_LAUNCH_CHECK();
 }
 
