@@ -384,12 +384,22 @@ struct Sweep {
     // relax from unchanged neighbours; the residual has no work for the first colour's.
     template <SweepStage S>
     __device__ __forceinline__ bool run(int s0, int s1) const {
+        Block B;
+        first<S>(s0, s1, B);
+        return run<S>(s0, s1, B);
+    }
+    // the x-independent data of the first step of [s0, s1)
+    template <SweepStage S>
+    __device__ __forceinline__ void first(int s0, int s1, Block &B) const {
+        if (s0 < s1) load<S>(desc_of(S == ST_BWD ? s1 - 1 : s0), B);
+    }
+    // with that of the first step in B
+    template <SweepStage S>
+    __device__ __forceinline__ bool run(int s0, int s1, Block &B) const {
         constexpr int dir = S == ST_BWD ? -1 : 1;
         const int cnt = s1 - s0;
         if (cnt <= 0) return true;
         int step = dir > 0 ? s0 : s1 - 1;
-        Block B;
-        load<S>(desc_of(step), B);
         RowDesc dn;
         if (cnt > 1) dn = desc_of(step + dir);
         for (int k = 0; k < cnt; ++k, step += dir) {
@@ -403,17 +413,6 @@ struct Sweep {
             B = N;
         }
         return true;
-    }
-    // grid barrier: the steps [s0, s1) of one colour
-    template <SweepStage S>
-    __device__ __forceinline__ void run_colour(int s0, int s1) const {
-        for (int k = s0; k < s1; ++k) {
-            Block B;
-            Slot<R> raw[PF];
-            load<S>(desc_of(k), B);
-            request<S>(B.col, B.len, raw);
-            finish<S>(B, raw);
-        }
     }
 };
 
@@ -455,18 +454,26 @@ __global__ void __launch_bounds__(FLOW ? FLOW_THREADS : GRID_THREADS, FLOW ? swe
         const unsigned long long extra = threadIdx.x == 0 ? *a.extra : 0ull;
         unsigned k = 0;
         const int32_t *cf = a.cfirst + (size_t)w * (a.ncolors + 1);
-        if (!a.zero_start) S.template run_colour<ST_PRE>(s0, s1);
+        if (!a.zero_start) S.template run<ST_PRE>(s0, s1);
+        // the first rows of the next colour are loaded between arriving and waiting
+        typename Sweep<G, PF, C, R, FLOW>::Block B;
+        S.template first<ST_FWD>(cf[0], cf[1], B);
         for (int c = 0; c < a.ncolors; ++c) {
-            S.template run_colour<ST_FWD>(cf[c], cf[c + 1]);
+            S.template run<ST_FWD>(cf[c], cf[c + 1], B);
             grid_arrive(cnt, k, base);
+            if (c + 1 < a.ncolors)
+                S.template first<ST_FWD>(cf[c + 1], cf[c + 2], B);
+            else if (c > 0)
+                S.template first<ST_BWD>(cf[c - 1], cf[c], B);
             if (!grid_wait(cnt, k++, base, extra, a.err, a.stop)) return;
         }
         for (int c = a.ncolors - 2; c >= 0; --c) {
-            S.template run_colour<ST_BWD>(cf[c], cf[c + 1]);
+            S.template run<ST_BWD>(cf[c], cf[c + 1], B);
             grid_arrive(cnt, k, base);
+            if (c > 0) S.template first<ST_BWD>(cf[c - 1], cf[c], B);
             if (!grid_wait(cnt, k++, base, extra, a.err, a.stop)) return;
         }
-        if (resid) S.template run_colour<ST_POST>(s0, s1);
+        if (resid) S.template run<ST_POST>(s0, s1);
     }
 }
 
