@@ -358,8 +358,9 @@ GL_API gl_status gl_precond_level_info(gl_prec prec, int level, int64_t *n, int6
 /* How level l's Gauss-Seidel steps run in the given precision's V-cycle
  * (GL_FP64, or GL_MIXED / GL_MIXED_PRECOND for the FP32 V-cycle once built):
  * *lanes = lanes per row, *sync = 0 for a grid barrier between colours, 1 for
- * dataflow, *ctas = CTAs of the launch; 0 / -1 / 0 on a lattice's finest and on
- * the coarsest level, which have no such sweep.  Any output may be NULL. */
+ * dataflow, *ctas = CTAs of the launch; 0 / -1 / 0 on a finest level that is
+ * relaxed by a launch per colour (a lattice's, a large triangulation's) and on the
+ * coarsest level, which have no such sweep.  Any output may be NULL. */
 GL_API gl_status gl_precond_level_sweep(gl_prec prec, int level, int precision, int *lanes, int *sync, int *ctas);
 
 /* agg_host: n int32, the coarse node of each node of this level (not the coarsest). */

@@ -402,7 +402,7 @@ gl_status gl_precond_level_sweep(gl_prec p, int l, int precision, int *lanes, in
                    GL_ERR_ARG, "no sweep of that precision (FP32 copies not built)");
         const Level &L = p->L[l];
         const bool f32 = precision != GL_FP64;
-        const bool coarse = p->swept(l);
+        const bool coarse = p->swept(l, f32);
         if (lanes) *lanes = coarse ? (f32 ? L.sw32.G : L.sw64.G) : 0;
         int sy = -1, nb = 0;
         if (coarse) {

@@ -169,8 +169,10 @@ struct gl_prec_s {
                                       // gl_precond_debug(GL_DEBUG_STALL_SWEEPS) (reset with the error word)
     int nlev = 0;
     // level l's Gauss-Seidel steps are k_sweep launches (gl_sweep.cu): the levels between
-    // the finest and the coarsest, and a finest level with more than two colours
-    bool swept(int l) const { return l < nlev - 1 && (l > 0 || L[0].ncolors > 2); }
+    // the finest and the coarsest, and a finest level with more than two colours where
+    // these are the faster form (sweep_finest; [1]: in FP32)
+    bool finest_swept[2] = {false, false};
+    bool swept(int l, bool fp32) const { return l < nlev - 1 && (l > 0 || finest_swept[fp32]); }
     int cycles = 1;
     bool has32 = false;
     bool autotune = true;
@@ -335,7 +337,9 @@ void precond_apply_p(gl_prec_s *p, const double2 *v, double2 *z, const int *stop
 void precond_apply_p32(gl_prec_s *p, const float2 *v, float2 *z, const int *stop, cudaStream_t s);
 // autotuner: picks the lanes-per-row width of every grouped-CSR operator by timing
 void autotune_levels(gl_prec_s *p, bool fp32, cudaStream_t s);
-// gl_sweep.cu: the operator of a many-coloured level in the sweeps' form (and its
+// gl_sweep.cu: sets p->finest_swept
+void sweep_finest(gl_prec_s *p, int sync);
+// the operator of a many-coloured level in the sweeps' form (and its
 // diagonal), in the solve ordering given by perm / iperm, the rows divided by
 // row_scale (nullable)
 template <typename C>

@@ -1362,6 +1362,7 @@ void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_
     GL_CUDA(cudaMemsetAsync(p->err.get(), 0, sizeof(int), s));
     p->wait_extra.alloc(1);
     GL_CUDA(cudaMemsetAsync(p->wait_extra.get(), 0, sizeof(unsigned long long), s));
+    sweep_finest(p, o.sweep_sync);
     for (int k = 0; k < p->nlev; ++k) {
         Level &L = p->L[k];
         bool coarsest = (k == p->nlev - 1);
@@ -1370,7 +1371,7 @@ void precond_setup(gl_prec_s *p, gl_mesh_s *m, const double2 *psi_nat, const gl_
             k_pdiag<<<grid_for(n, 256), 256, 0, s>>>(n, m->kdiag.get(), p->psi_p.get(), L.diag.get());
             GL_LAUNCH_CHECK();
         }
-        if (p->swept(k)) {
+        if (p->swept(k, false)) {
             // (the finest level's operator is the row-scaled one, whose diagonal is above)
             build_split<double2>(L.n, L.perm, L.iperm, L.A_can, k == 0 ? m->vol.get() : nullptr, L.sw64.A,
                                  k == 0 ? nullptr : L.diag.get(), s);
@@ -1494,7 +1495,7 @@ void precond_ensure_fp32(gl_prec_s *p, cudaStream_t s) {
         if (k == 0) {
             L.A32 = &m->K32;
         }
-        if (p->swept(k))
+        if (p->swept(k, true))
             build_split<float2>(L.n, L.perm, L.iperm, L.A_can, k == 0 ? m->vol.get() : nullptr, L.sw32.A, nullptr, s);
         if (!coarsest) {
             Level &Lc = p->L[k + 1];

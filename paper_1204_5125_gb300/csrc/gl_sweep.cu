@@ -1,8 +1,8 @@
 // gl_sweep.cu -- the multicolour symmetric Gauss-Seidel steps of the V-cycle's
 // many-coloured levels (Sec. 4: one pre- and one post-step per level), each a
 // single launch, with the residual that follows the pre-step: the coarse levels,
-// and the finest level of a general simplicial mesh (on a lattice the finest level
-// is red-black: three large launches, gl_vcycle.cu).
+// and the finest level of a general simplicial mesh up to the sizes of sweep_finest (on a
+// lattice the finest level is red-black: three large launches, gl_vcycle.cu).
 //
 // A level's operator is stored by rows with the entries of lower colours (solve
 // positions below the row's own) first and those of higher colours behind them.
@@ -727,6 +727,29 @@ static void sweep_launch(gl_prec_s *p, Level &L, const typename SweepOps<T>::C *
     });
 }
 
+// Whether the finest level of a general mesh is swept by k_sweep (on a lattice it has two
+// colours and never is).  With a launch per colour the step and its residual read every
+// entry 4.5 times, k_sweep reads it 3 times, but writes, empties and polls slots and reads
+// lists of rows, 100 to 200 bytes a row more; past the caches that decides.  One
+// preconditioner application, a launch per colour against k_sweep, on triangulations (6
+// entries a row):
+//   nodes            360,000     640,000     1.0 M       1.44 M      2.25 M       16 M
+//   FP32 dataflow    339, 252    400, 345    448, 444    538, 568    657, 783     3406, 4962 us
+//   FP64 dataflow    500, 387    624, 521    762, 688    961, 893    1270, 1278   6999, 8108
+//   FP32 grid        418, 353    481, 445    520, 538    614, 674    727, 889     3515, 5113
+//   FP64 grid        637, 569    775, 723    904, 895    1119, 1127  1409, 1487   7255, 8320
+// and on a ball's tetrahedra (14 entries a row), 0.6 M and 3.5 M nodes: FP32 768, 480 and
+// 2026, 1703 us; FP64 1254, 755 and 4048, 2964; likewise with the grid barrier.  So rows
+// of ten entries and more are always swept, shorter ones up to 2^20 (FP32) and 2^21 rows
+// (FP64), three quarters of these with the grid barrier.
+void sweep_finest(gl_prec_s *p, int sync) {
+    const Level &L = p->L[0];
+    for (int fp32 = 0; fp32 < 2; ++fp32) {
+        const int64_t most = (sync == 1 ? 3 : 4) * (fp32 ? 1ll << 18 : 1ll << 19);
+        p->finest_swept[fp32] = L.ncolors > 2 && (L.n <= most || L.A_can.nnz >= 11 * L.n);
+    }
+}
+
 template <typename T>
 void sweep_step(gl_prec_s *p, int l, const typename CT<T>::type *b, typename CT<T>::type *x, bool zero_start,
                 typename CT<T>::type *r, const T *scale, const int *stop, cudaStream_t s) {
@@ -844,7 +867,7 @@ static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
         GL_CUDA(cudaEventCreate(&e1));
     }
     for (int l = 0; l < p->nlev - 1; ++l) {
-        if (!p->swept(l)) continue;
+        if (!p->swept(l, sizeof(T) == 4)) continue;
         Level &L = p->L[l];
         auto &D = O::data(L);
         sweep_alloc<T>(L, s);
@@ -902,7 +925,7 @@ void plan_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s) {
 template <typename T>
 static void adopt_sweeps_t(gl_prec_s *p, const int *lanes, const int *shifts, const int *sync, cudaStream_t s) {
     for (int l = 0; l < p->nlev - 1; ++l) {
-        if (!p->swept(l)) continue;
+        if (!p->swept(l, sizeof(T) == 4)) continue;
         Level &L = p->L[l];
         sweep_alloc<T>(L, s);
         sweep_shape<T>(L, sync[l], lanes[l], shifts[l], s);

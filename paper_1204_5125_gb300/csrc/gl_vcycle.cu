@@ -601,8 +601,8 @@ static bool lattice_for(const gl_prec_s *p, LatticeView &v) {
     return false;
 }
 
-// pre- or post-smoothing on the finest level: per-colour launches (two colours,
-// large sweeps, on a lattice)
+// pre- or post-smoothing on the finest level: per-colour launches (two colours on a
+// lattice, more on a general mesh beyond the sizes of sweep_finest)
 template <typename T>
 static void smooth_finest(gl_prec_s *p, const typename LevelOps<T>::C *b, typename LevelOps<T>::C *x, bool zero_start,
                           const int *stop, cudaStream_t s) {
@@ -629,7 +629,7 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         scale = l == 0 ? p->mesh->volp.get() : nullptr;
     else
         scale = l == 0 ? p->mesh->volp32.get() : nullptr;
-    if (p->swept(l)) {
+    if (p->swept(l, sizeof(T) == 4)) {
         sweep_step<T>(p, l, b, x, true, r, scale, stop, s);  // and the residual
     } else {
         smooth_finest<T>(p, b, x, true, stop, s);
@@ -673,7 +673,7 @@ static void vcycle(gl_prec_s *p, int l, const typename LevelOps<T>::C *b, typena
         ProfScope ps("prolong", 0, s);
         k_spmv<C><<<grid_for(L.n - lo, 256), 256, 0, s>>>(lo, L.n, O::P(L).view(), O::x(Lc), x, 1, stop);
     }
-    if (p->swept(l))
+    if (p->swept(l, sizeof(T) == 4))
         sweep_step<T>(p, l, b, x, false, nullptr, nullptr, stop, s);
     else
         smooth_finest<T>(p, b, x, false, stop, s);
