@@ -333,9 +333,13 @@ GL_API gl_status gl_precond_apply_precision(gl_prec prec, const void *x_dev, voi
  * run normally).  GL_DEBUG_NEGATE_COARSEST: multiplies the coarsest level's
  * dense inverse by -1, which makes R_k indefinite on a one-level hierarchy
  * (solves then end with GL_ERR_BREAKDOWN); permanent for this handle.
+ * GL_DEBUG_SWEEP_FORM + 64 K + G: the sweeps of every level in both precisions
+ * (FP32: once built) in the form that the setup's timing may choose, G = 2, 4, 8,
+ * 16 or 32 lanes per row and K = 1 or 2 shifts of warps; not for R_inf.
  * Synchronises the device. */
 #define GL_DEBUG_STALL_SWEEPS 1
 #define GL_DEBUG_NEGATE_COARSEST 2
+#define GL_DEBUG_SWEEP_FORM 1024
 GL_API gl_status gl_precond_debug(gl_prec prec, int action);
 GL_API gl_status gl_precond_destroy(gl_prec prec);
 

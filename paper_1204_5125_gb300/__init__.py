@@ -30,7 +30,7 @@ __all__ = [
     "gl_last_error", "EXPORTED", "GL_CYCLES_INF", "ContOptions", "ContPoint", "gl_mesh_create_edge",
     "gl_mesh_set_mu", "gl_residual_dmu", "gl_energy", "cont_options", "gl_continuation", "gl_precond_setup_like",
     "GL_COLOR_SL", "GL_COLOR_JP", "GL_COLOR_PSL", "gl_mesh_create_dipole", "gl_mesh_create_simplicial", "gl_precond_apply_precision", "gl_precond_debug",
-    "GL_DEBUG_STALL_SWEEPS", "GL_DEBUG_NEGATE_COARSEST", "gl_precond_level_sweep", "gl_measure_fma_peak",
+    "GL_DEBUG_STALL_SWEEPS", "GL_DEBUG_NEGATE_COARSEST", "GL_DEBUG_SWEEP_FORM", "gl_precond_level_sweep", "gl_measure_fma_peak",
     "gl_measure_sync_latency", "GL_APPLY_FP64_TABLES",
     "gl_profile_flops",
 ]
@@ -39,7 +39,8 @@ GL_FP64, GL_MIXED, GL_MIXED_PRECOND = 0, 1, 2
 GL_APPLY_FP64_TABLES = 3  # gl_jacobian_apply: the FP64 apply from the lattice stencil's FP64 tables
 GL_CYCLES_INF = -1  # options.cycles: R_inf, the V-cycle repeated until the 1e-12 residual test
 GL_COLOR_SL, GL_COLOR_JP, GL_COLOR_PSL = 0, 1, 2  # options.coloring of the coarse levels
-GL_DEBUG_STALL_SWEEPS, GL_DEBUG_NEGATE_COARSEST = 1, 2  # gl_precond_debug actions (fault injection for tests)
+# gl_precond_debug actions: fault injection for tests, and a chosen form of the sweeps
+GL_DEBUG_STALL_SWEEPS, GL_DEBUG_NEGATE_COARSEST, GL_DEBUG_SWEEP_FORM = 1, 2, 1024
 STATUS = {0: "GL_OK", 1: "GL_ERR_ARG", 2: "GL_ERR_CUDA", 3: "GL_ERR_OOM", 4: "GL_ERR_NOT_CONVERGED",
           5: "GL_ERR_BREAKDOWN", 6: "GL_ERR_NAN", 7: "GL_ERR_TIMEOUT", 8: "GL_ERR_CAPACITY"}
 

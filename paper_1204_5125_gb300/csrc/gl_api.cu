@@ -346,6 +346,13 @@ gl_status gl_precond_debug(gl_prec p, int action) {
             GL_CUDA(cudaMemcpy(p->wait_extra.get(), &far, sizeof far, cudaMemcpyHostToDevice));
         } else if (action == GL_DEBUG_NEGATE_COARSEST) {
             precond_negate_coarsest(p, nullptr);
+        } else if ((action & ~255) == GL_DEBUG_SWEEP_FORM) {
+            const int G = action & 63, K = action >> 6 & 3;
+            GL_REQUIRE(G >= 2 && G <= 32 && (G & (G - 1)) == 0 && K >= 1 && K <= 2, GL_ERR_ARG, "unknown sweep form");
+            GL_REQUIRE(!p->rinf, GL_ERR_ARG, "R_inf keeps its sweeps' form");
+            GL_CUDA(cudaDeviceSynchronize());
+            sweeps_form(p, G, K, nullptr);
+            GL_CUDA(cudaDeviceSynchronize());
         } else {
             GL_REQUIRE(false, GL_ERR_ARG, "unknown debug action");
         }

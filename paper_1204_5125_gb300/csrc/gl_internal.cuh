@@ -352,6 +352,8 @@ void sweep_step(gl_prec_s *p, int l, const typename CT<T>::type *b, typename CT<
                 typename CT<T>::type *r, const T *scale, const int *stop, cudaStream_t s);
 // picks, per level, the form of the sweep and its lanes per row (timed when autotuning)
 void plan_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s);
+// G lanes per row and K shifts in every sweep that is set up (for tests)
+void sweeps_form(gl_prec_s *p, int G, int K, cudaStream_t s);
 // the same choices as a template's (p->tuned)
 void adopt_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s);
 // after a wait of the coarse sweeps ran out: zeroes every level's synchronisation

@@ -944,6 +944,21 @@ void adopt_sweeps(gl_prec_s *p, bool fp32, cudaStream_t s) {
         adopt_sweeps_t<double>(p, lanes, shifts, sync, s);
 }
 
+template <typename T>
+static void sweeps_form_t(gl_prec_s *p, int G, int K, cudaStream_t s) {
+    for (int l = 0; l < p->nlev - 1; ++l) {
+        auto &D = SweepOps<T>::data(p->L[l]);
+        if (!D.state.get()) continue;
+        sweep_shape<T>(p->L[l], D.sync, G, K, s);
+        sweep_zero(D, s);
+    }
+}
+void sweeps_form(gl_prec_s *p, int G, int K, cudaStream_t s) {
+    sweeps_form_t<double>(p, G, K, s);
+    sweeps_form_t<float>(p, G, K, s);
+    p->uid = next_uid();  // captured solves hold the old lists
+}
+
 void sweeps_reset(gl_prec_s *p, cudaStream_t s) {
     for (int l = 0; l < p->nlev - 1; ++l) {
         sweep_zero(p->L[l].sw32, s);
