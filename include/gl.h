@@ -430,8 +430,10 @@ GL_API gl_status gl_batch_solve(int count, const gl_mesh *meshes, const void *co
 /* Measured arithmetic peak of the current GPU for the rooflines (not a paper
  * quantity): fused multiply-adds of independent chains on every SM, timed with
  * CUDA events; precision GL_FP64 for FP64, GL_MIXED for FP32.  *gflops_host =
- * GFLOP/s (2 per FMA), the best of repetitions grown to >= 20 ms.  Synchronises
- * `stream`. */
+ * GFLOP/s (2 per FMA), the best of repetitions grown to >= 20 ms: the larger of the
+ * rate on full SMs and of four times that of one warp on every SM (one of four
+ * sub-cores alone, which in FP64 is the bound that full SMs stay below).
+ * Synchronises `stream`. */
 GL_API gl_status gl_measure_fma_peak(int precision, double *gflops_host, void *stream);
 
 /* Measured latencies that bound one phase of the coarse-level Gauss-Seidel

@@ -72,7 +72,7 @@ __global__ void k_jacobian32(int64_t n, SellView<float2> K, const float *__restr
 // numbers.  Consecutive nodes alternate between the two colours of a lattice, so a
 // warp reads its matrix entries as two runs of 16 and its vectors as one of 32, and
 // nothing is gathered and scattered around the apply.  Bound by the FP64 pipe (35
-// operations a row in 3D, 124 us for 128^3 rows at 1.19 TFLOP/s; the bytes would take 55
+// operations a row in 3D, 117 us for 128^3 rows at 1.25 TFLOP/s; the bytes would take 55
 // us).  Whole calls, before (two gathers, the apply on reordered vectors, a scatter) and
 // now: Jacobian on 128^3 nodes 193 and
 // 129 us, on 64^2 22.8 and 15.0 us; residual on 1023^2 63 and 45 us.

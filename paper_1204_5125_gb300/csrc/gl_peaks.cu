@@ -14,6 +14,7 @@
 namespace gl {
 
 constexpr int PEAK_CHAINS = 8;  // independent accumulators per thread
+constexpr int SUBCORES = 4;     // schedulers of an SM, each with its own share of the units
 
 template <typename R>
 __global__ void __launch_bounds__(256) k_fma_peak(int64_t reps, R a, R b, R *sink) {
@@ -30,13 +31,9 @@ __global__ void __launch_bounds__(256) k_fma_peak(int64_t reps, R a, R b, R *sin
     if (t == (R)-12345.0) *sink = t;  // keeps the chains live
 }
 
+// GFLOP/s of `grid` blocks of `block` threads with `smem` bytes of shared memory each
 template <typename R>
-static double fma_peak_gflops(cudaStream_t s) {
-    int dev = 0, nsm = 0, per_sm = 0;
-    GL_CUDA(cudaGetDevice(&dev));
-    GL_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    GL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fma_peak<R>, 256, 0));
-    const int grid = nsm * std::max(per_sm, 1);
+static double fma_rate_gflops(int grid, int block, int smem, cudaStream_t s) {
     DBuf<R> sink(1);
     cudaEvent_t e0, e1;
     GL_CUDA(cudaEventCreate(&e0));
@@ -45,14 +42,14 @@ static double fma_peak_gflops(cudaStream_t s) {
     int64_t reps = 1 << 12;
     double best = 0;
     for (int trial = 0; trial < 12; ++trial) {
-        k_fma_peak<R><<<grid, 256, 0, s>>>(reps, (R)0.999999, (R)1e-7, sink.get());
+        k_fma_peak<R><<<grid, block, smem, s>>>(reps, (R)0.999999, (R)1e-7, sink.get());
         GL_CUDA(cudaEventRecord(e0, s));
-        k_fma_peak<R><<<grid, 256, 0, s>>>(reps, (R)0.999999, (R)1e-7, sink.get());
+        k_fma_peak<R><<<grid, block, smem, s>>>(reps, (R)0.999999, (R)1e-7, sink.get());
         GL_CUDA(cudaEventRecord(e1, s));
         GL_CUDA(cudaEventSynchronize(e1));
         float ms = 0;
         GL_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        const double flops = 2.0 * (double)grid * 256 * PEAK_CHAINS * (double)reps;
+        const double flops = 2.0 * (double)grid * block * PEAK_CHAINS * (double)reps;
         best = std::max(best, flops / (ms * 1e-3) / 1e9);
         if (ms >= 20.f) break;
         reps *= 2;
@@ -60,6 +57,25 @@ static double fma_peak_gflops(cudaStream_t s) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return best;
+}
+
+// The larger of the rate on full SMs and of four times that of one warp on every SM.  In
+// FP64 the second is the bound: a warp issues half a thread's operation a cycle on its
+// sub-core (1.49e11 a second over 152 SMs at 1.96 GHz), while full SMs reach 0.84 of four
+// times that in a loop of these FMAs, 0.92 when the multiplicands alternate, whatever the
+// warps, chains and unrolling: the sub-cores meet at shared units.  So 1.25 TFLOP/s, where
+// full SMs give 1.06, a rate that the FP64 Jacobian on 128^3 nodes exceeds (1.13).
+template <typename R>
+static double fma_peak_gflops(cudaStream_t s) {
+    int dev = 0, nsm = 0, per_sm = 0, smem_max = 0;
+    GL_CUDA(cudaGetDevice(&dev));
+    GL_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    GL_CUDA(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    GL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fma_peak<R>, 256, 0));
+    const double full = fma_rate_gflops<R>(nsm * std::max(per_sm, 1), 256, 0, s);
+    const int alone = smem_max / 2 + 1024;  // at most one block an SM
+    GL_CUDA(cudaFuncSetAttribute(k_fma_peak<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, alone));
+    return std::max(full, SUBCORES * fma_rate_gflops<R>(nsm, 32, alone, s));
 }
 
 // ---- latencies
@@ -91,8 +107,8 @@ __device__ __forceinline__ bool wait_geq(const unsigned long long *p, unsigned l
 
 // CTA 0 and CTA `partner` (one CTA per SM: the launch asks for more than half
 // an SM's shared memory; cooperative, so both are resident) pass a counter back
-// and forth `rounds` times with release stores and acquiring loads, as the
-// neighbour-flag sweep does; CTA 0 records the mean one-way hand-off in ns.
+// and forth `rounds` times with release stores and acquiring loads; CTA 0 records the
+// mean one-way hand-off in ns (the sweeps' rows hand values over with relaxed accesses).
 // flags[0], flags[1]: the two counters, starting at base.
 __global__ void k_pingpong(int partner, int rounds, unsigned long long base, unsigned long long *flags,
                            double *out, int *err) {

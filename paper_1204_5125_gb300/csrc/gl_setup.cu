@@ -921,14 +921,15 @@ __global__ void k_to_dense(int64_t n, const int64_t *rp, const int32_t *ci, cons
 // and is -A^-1 once every block has been swept.  M_KK is a Schur complement of A when
 // its turn comes, so its pivots are positive exactly if A is positive definite.
 //
-// The n^3 / 2 complex products are bound by this GPU's FP64 rate (1.06 TFLOP/s measured:
-// 76 ms at n = 2720), so shared memory and HBM have time to spare and small blocks cost
+// The n^3 / 2 complex products are bound by this GPU's FP64 rate (64 ms at n = 2720 at the
+// 1.25 TFLOP/s that four sub-cores issue; loops of FMAs alone reach 0.85 of that, as the
+// update does: 76 ms), so shared memory and HBM have time to spare and small blocks cost
 // nothing: with 16 rows a step still computes for 0.45 ms on 60 MB, while the chain in
 // front of it (the inverse of one 16 x 16 block, which every CTA of the panel kernel
 // forms for itself, and a 16-column panel) stays short.  The update's 32 x 32 tiles
 // have eight warps of 2 x 2 entries a thread, so a small matrix's few tiles still keep
 // every sub-core's FP64 unit busy.  Measured at n = 2720 (128^3 cube): 322 ms as
-// n rank-one Gauss-Jordan steps over all n^2 entries, 83 ms now (0.92 of the FP64 rate);
+// n rank-one Gauss-Jordan steps over all n^2 entries, 83 ms now;
 // n = 362 (1024^2 square): 4.0 and 1.2 ms.
 constexpr int INV_B = 16;     // rows of a pivot block
 constexpr int INV_T = 32;     // tile of the update
