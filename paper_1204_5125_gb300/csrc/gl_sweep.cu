@@ -223,7 +223,12 @@ enum SweepStage { ST_PRE, ST_FWD, ST_BWD, ST_POST };
 // its backward value have slots of their own), and the launch's set of slots was
 // emptied by the launch before it, so nothing is ever overwritten unread.  Plain x
 // is read in the pre-pass only, by rows of lower colours, and written by a row's
-// last relaxation, which waits for those rows' forward values.
+// last relaxation, which waits for those rows' forward values.  That read and that write
+// have no release and acquire between them: the read's value goes into the reader's
+// forward value, the writer polls that value, and what it writes is formed from it, so the
+// read could only see the write in a circle of dependences (a value out of thin air, which
+// the PTX memory model excludes).  It does not order the two otherwise: a pre-pass whose
+// result did not go into the polled value would need a copy of x.
 template <int G, int PF, typename C, typename R, bool FLOW>
 struct Sweep {
     static constexpr int RPW = 32 / G, H = G / 2;
