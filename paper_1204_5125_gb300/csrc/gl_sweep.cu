@@ -857,10 +857,16 @@ static int sweep_default_lanes(int64_t nnz, int64_t n) {
 // their first polls behind them when the phase before it stores; 48 to 43 us in FP64
 // and 33 to 29 us in FP32 for the pre- and post-step of the 64^2 square's level 1,
 // slower where the warps of both shifts no longer fit the SMs twice over).  With
-// autotuning G = 2, 4, 8 with one shift and, below a quarter of the GPU, two are
+// autotuning three numbers of lanes with one shift and, below a quarter of the GPU, two are
 // timed (a pre- and a post-step on zero vectors, best of two after a warm-up) and the
-// fastest kept; without it G follows from the mean row length, with one shift.  The
-// result depends on G only (the order of a row's sum).
+// fastest kept: G = 2, 4, 8, or 4, 8, 16 where rows have 48 entries and more (the third
+// level of a cube); without it G follows from the mean row length, with one shift.  The
+// result depends on G only (the order of a row's sum).  On 2, 4, 8 and 16 lanes, with the
+// better number of shifts:
+//   97^3, level 2 (1252 rows of 54): FP64 643, 348, 226, 185 us; FP32 222, 136, 132, 123
+//   128^3, level 2 (2720 rows): FP64 652, 364, 250, 201; FP32 237, 158, 160, 156
+//   97^3, level 1 (82,455 rows of 33 entries): FP64 271, 212, 196, 242; FP32 135, 121, 137, 183
+//   1024^2, level 1 (146,813 rows of 10): FP64 104, 124, 164, 294; FP32 60, 70, 94, 140
 template <typename T>
 static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
     using O = SweepOps<T>;
@@ -885,9 +891,10 @@ static void plan_sweeps_t(gl_prec_s *p, cudaStream_t s) {
         GL_CUDA(cudaMemsetAsync(b, 0, L.n * sizeof(C), s));
         GL_CUDA(cudaMemsetAsync(x, 0, L.n * sizeof(C), s));
         float best = 1e30f;
-        int bestG = 2, bestK = 1;
+        const int least = D.A.nnz >= 48 * L.n ? 4 : 2;
+        int bestG = least, bestK = 1;
         for (int cand = 0; cand < 6; ++cand) {
-            const int g = 2 << (cand % 3), K = 1 + cand / 3;
+            const int g = least << (cand % 3), K = 1 + cand / 3;
             if (K == 2 && (sync == 0 || sweep_ctas_wanted(L, g, 2, true) > 2 * NUM_SMS_HINT)) continue;
             sweep_shape<T>(L, sync, g, K, s);
             if (sync == 0) sweep_zero(D, s);  // another grid size on the barrier's counter
