@@ -37,4 +37,4 @@ def test_fp64_peak_is_not_exceeded():
         gl.gl_mesh_destroy(m)
     rate = 2 * 35 * 0.99 * n / (best * 1e-3) / 1e9
     print(f"{1e3 * best:.1f} us a call: {rate:.0f} of {peak:.0f} GFLOP/s")
-    assert 0.8 * peak < rate < peak
+    assert 0.6 * peak < rate < peak
